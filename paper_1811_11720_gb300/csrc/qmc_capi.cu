@@ -91,7 +91,6 @@ int qmc_points(const qmc_rule *rule, uint64_t i_begin, uint64_t count, double *o
     p.count = count;
     p.d = rule->dim;
     p.m = (int)rule->m;
-    p.L = 64;
     for (int j = 0; j < rule->dim; ++j) p.dc[j] = dim_const(rule->z[j] % rule->n, rule->n);
     p.shifts = rule->shifts;
     p.out = out;

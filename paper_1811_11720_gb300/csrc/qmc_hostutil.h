@@ -27,7 +27,7 @@ inline uint64_t gcd_u64(uint64_t a, uint64_t b) {
     return a;
 }
 
-// floor(z 2^128 / n) and z 2^128 mod n for z < n, by two 128/64 divisions.
+// The first 192 fraction bits of z / n for z < n, by three 128/64 divisions.
 inline DimConst dim_const(uint64_t z, uint64_t n) {
     u128_t a = (u128_t)z << 64;
     uint64_t q1 = (uint64_t)(a / n);
@@ -35,7 +35,8 @@ inline DimConst dim_const(uint64_t z, uint64_t n) {
     u128_t b = (u128_t)r1 << 64;
     uint64_t q0 = (uint64_t)(b / n);
     uint64_t r0 = (uint64_t)(b % n);
-    return DimConst{q1, q0, r0};
+    uint64_t rq = (uint64_t)(((u128_t)r0 << 64) / n);
+    return DimConst{q1, q0, rq};
 }
 
 inline double binom(int a, int b) {

@@ -20,12 +20,14 @@ cudaError_t launch_sums_poly(int family, int tkind, dim3 grid, dim3 block, cudaS
 struct PointsParams {
     uint64_t n, i_begin, count;
     int d, m;
-    uint32_t L;
+    // launch shape, set by launch_points: threads per block as rows x cols, steps per thread
+    int rows, cols;
+    uint32_t steps;
     DimConst dc[kMaxDim];
     const uint64_t *shifts;
     double *out;
 };
-cudaError_t launch_points(const PointsParams &p, cudaStream_t s);
+cudaError_t launch_points(PointsParams p, cudaStream_t s);
 
 // Reduce per-tile partials [tiles][m] (sum, comp) (and the im block) to double-double
 // sums [2m] (and [2m..4m) for im), fixed order.

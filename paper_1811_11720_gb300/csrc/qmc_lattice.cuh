@@ -16,9 +16,8 @@
 //     or rem != 0).  When V's high word is zero (v < 2^-64, which needs r/n + Delta within
 //     2^-64 of an integer) more quotient bits are produced from rem by long division.
 //
-// Everything here is exact integer arithmetic; the only floating-point objects are the
-// final bit pattern and, at the start of a stream, FP64 estimates of a quotient that is
-// then corrected exactly (divmod_128_64_fast).
+// Everything here is exact integer arithmetic; the only floating-point object is the final
+// bit pattern.
 #pragma once
 #include <cstdint>
 
@@ -26,8 +25,17 @@ namespace qmc {
 
 struct DimConst {
     uint64_t fz_hi, fz_lo;  // floor(z 2^128 / n)
-    uint64_t remz;          // z 2^128 mod n
+    uint64_t rq;            // the next 64 quotient bits, floor(remz 2^64 / n)
 };
+
+// What a step adds: F of one (or several) lattice steps and its exact remainder.
+struct LatticeStep {
+    uint64_t fz_hi, fz_lo, remz;
+};
+// remz = z 2^128 mod n: z 2^128 = F n + remz, so remz = -F n modulo 2^64, and remz < n < 2^63.
+__device__ __forceinline__ LatticeStep lattice_step_of(const DimConst &c, uint64_t n) {
+    return {c.fz_hi, c.fz_lo, 0 - c.fz_lo * n};
+}
 
 // Restoring division of (hi:lo) by n, requiring hi < n: quotient < 2^64.
 __host__ __device__ inline void divmod_128_64(uint64_t hi, uint64_t lo, uint64_t n, uint64_t *q,
@@ -48,60 +56,31 @@ __host__ __device__ inline void divmod_128_64(uint64_t hi, uint64_t lo, uint64_t
     *r = hi;
 }
 
-// The same quotient and remainder for n < 2^62 in a few dozen instructions: a quotient
-// estimate q0 from FP64 (within 2^13 + 2 of the exact one: the operands and 1/n carry
-// relative errors of a few 2^-53), the exact remainder r = p - q0 n in two's-complement
-// 128-bit arithmetic (|r| < 2^14 n), a second FP64 estimate of r / n (within 1), and at
-// most two exact corrections.  The result is exact; only the work differs from the loop.
-__device__ __forceinline__ void divmod_128_64_fast(uint64_t hi, uint64_t lo, uint64_t n,
-                                                   uint64_t *q, uint64_t *r) {
-    if (n >= (1ull << 62)) {
-        divmod_128_64(hi, lo, n, q, r);
-        return;
-    }
-    const double inv = 1.0 / (double)n;
-    const double pd = fma((double)hi, 0x1p64, (double)lo);
-    const double qd = fmin(fmax(pd * inv, 0.0), 0x1.fffffffffffffp63);
-    const uint64_t q0 = (uint64_t)qd;
-    const uint64_t ml = q0 * n, mh = __umul64hi(q0, n);
-    const uint64_t rl = lo - ml;
-    const uint64_t rh = hi - mh - (lo < ml ? 1ull : 0ull);   // r = (int64)rh 2^64 + rl
-    const double rd = fma((double)(long long)rh, 0x1p64, (double)rl);
-    const long long q1 = (long long)floor(rd * inv);
-    // r - q1 n lies in (-2n, 2n), inside the int64 range for n < 2^62: its low word is it
-    long long r2 = (long long)(rl - (uint64_t)q1 * n);
-    uint64_t qq = q0 + (uint64_t)q1;
-#pragma unroll 1
-    for (int it = 0; it < 3 && r2 < 0; ++it) {
-        r2 += (long long)n;
-        --qq;
-    }
-#pragma unroll 1
-    for (int it = 0; it < 3 && r2 >= (long long)n; ++it) {
-        r2 -= (long long)n;
-        ++qq;
-    }
-    *q = qq;
-    *r = (uint64_t)r2;
-}
-
-// Lattice state of one coordinate at index i: F(i) and rem(i) for r = i z mod n.
-// F(i) = (i Fz + floor(i remz / n)) mod 2^128, rem(i) = i remz mod n.
+// Lattice state of one coordinate at index i < 2^63: F(i) and rem(i) for r = i z mod n.
+// F(i) = (i Fz + floor(i remz / n)) mod 2^128 and rem(i) = i remz mod n = -F(i) n mod 2^64.
+// The quotient comes from the host's reciprocal word: with rq = floor(remz 2^64 / n),
+// i remz / n - i rq / 2^64 lies in [0, i / 2^64), below 1, so q = floor(i rq / 2^64) is the
+// exact quotient or one less, and the remainder it leaves lies in [0, 2n), which 64 bits
+// hold for n < 2^63: one conditional correction, no division.  (Every stream of a lattice
+// sum starts here; an FP64-assisted 128/64 division in its place cost ~30 FP64 warp
+// instructions of ~17 SM cycles each per warp.)
 __device__ __forceinline__ void lattice_state_at(uint64_t i, const DimConst &c, uint64_t n,
                                                  uint64_t &f_hi, uint64_t &f_lo,
                                                  uint64_t &rem) {
-    uint64_t p_lo = i * c.remz;
-    uint64_t p_hi = __umul64hi(i, c.remz);  // i < n and remz < n: p < n^2, p_hi < n
-    uint64_t q;
-    divmod_128_64_fast(p_hi, p_lo, n, &q, &rem);
-    uint64_t lo = i * c.fz_lo;
-    uint64_t hi = __umul64hi(i, c.fz_lo) + i * c.fz_hi;
-    f_lo = lo + q;
-    f_hi = hi + (f_lo < lo);
+    const uint64_t lo = i * c.fz_lo;
+    uint64_t add = __umul64hi(i, c.rq);
+    uint64_t r = 0 - (lo + add) * n;
+    if (r >= n) {
+        r -= n;
+        ++add;
+    }
+    rem = r;
+    f_lo = lo + add;
+    f_hi = __umul64hi(i, c.fz_lo) + i * c.fz_hi + (f_lo < lo);
 }
 
 // One lattice step i -> i+1.
-__device__ __forceinline__ void lattice_step(const DimConst &c, uint64_t n, uint64_t &f_hi,
+__device__ __forceinline__ void lattice_step(const LatticeStep &c, uint64_t n, uint64_t &f_hi,
                                              uint64_t &f_lo, uint64_t &rem) {
     uint64_t r2 = rem + c.remz;             // < 2n < 2^64 for n < 2^63
     uint64_t carry = (r2 >= n) ? 1u : 0u;

@@ -206,6 +206,7 @@ __device__ __forceinline__ void stream_sums_r(const P &p, const FamilyShared &fs
         // the warp is one group: lane j < d owns coordinate j
         const int lane = threadIdx.x & 31;
         uint64_t fh = 0, fl = 0, rm = 0;
+        const LatticeStep step = lattice_step_of(p.dc[lane < d ? lane : 0], n);
         if (lane < d) lattice_state_at(i0, p.dc[lane], n, fh, fl, rm);
 #pragma unroll 1
         for (uint64_t t = 0; t < cnt; ++t) {
@@ -224,7 +225,7 @@ __device__ __forceinline__ void stream_sums_r(const P &p, const FamilyShared &fs
                 [&](int j) { return wl->flo[b][j]; }, [&](int j) { return wl->rem[b][j]; }, g_re,
                 g_im, signfail);
             accumulate(t, g_re, g_im);
-            if (lane < d) lattice_step(p.dc[lane], n, fh, fl, rm);
+            if (lane < d) lattice_step(step, n, fh, fl, rm);
         }
     } else if (wl) {
         // groups of q < 32 lanes (q divides 32): the group's lane j < d owns coordinate j
@@ -233,6 +234,7 @@ __device__ __forceinline__ void stream_sums_r(const P &p, const FamilyShared &fs
         const int pos = lane - base;
         const unsigned mask = ((1u << q) - 1u) << base;
         uint64_t fh = 0, fl = 0, rm = 0;
+        const LatticeStep step = lattice_step_of(p.dc[pos < d ? pos : 0], n);
         if (pos < d) lattice_state_at(i0, p.dc[pos], n, fh, fl, rm);
 #pragma unroll 1
         for (uint64_t t = 0; t < cnt; ++t) {
@@ -251,7 +253,7 @@ __device__ __forceinline__ void stream_sums_r(const P &p, const FamilyShared &fs
                 [&](int j) { return wl->flo[b][base + j]; },
                 [&](int j) { return wl->rem[b][base + j]; }, g_re, g_im, signfail);
             accumulate(t, g_re, g_im);
-            if (pos < d) lattice_step(p.dc[pos], n, fh, fl, rm);
+            if (pos < d) lattice_step(step, n, fh, fl, rm);
         }
     } else {
         uint64_t fhi[kMaxDim], flo[kMaxDim], rem[kMaxDim];
@@ -265,7 +267,7 @@ __device__ __forceinline__ void stream_sums_r(const P &p, const FamilyShared &fs
                 [&](int j) { return flo[j]; }, [&](int j) { return rem[j]; }, g_re, g_im, signfail);
             accumulate(t, g_re, g_im);
 #pragma unroll 1
-            for (int j = 0; j < d; ++j) lattice_step(p.dc[j], n, fhi[j], flo[j], rem[j]);
+            for (int j = 0; j < d; ++j) lattice_step(lattice_step_of(p.dc[j], n), n, fhi[j], flo[j], rem[j]);
         }
     }
     acc_re += in_re;
