@@ -7,7 +7,6 @@
 #include <cstring>
 #include <vector>
 
-#include "qmc_batch.cuh"
 #include "qmc_gb300.h"
 #include "qmc_hostutil.h"
 #include "qmc_internal.h"
@@ -33,7 +32,7 @@ __device__ __forceinline__ dd2 dd2_add(dd2 a, dd2 b) {
 
 // Block (q, component, k): fold item q's tiles for shift k in fixed order.
 __global__ void __launch_bounds__(kBatchRedThreads)
-    batch_reduce_kernel(const BatchItem *items, int m, int cplx, const double *partials,
+    batch_reduce_kernel(const Integral *items, int m, int cplx, const double *partials,
                         double *sums) {
     __shared__ dd2 red[kBatchRedThreads];
     const int per_item = m * (cplx ? 2 : 1);
@@ -54,26 +53,27 @@ __global__ void __launch_bounds__(kBatchRedThreads)
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        double *o = sums + (size_t)q * 4 * m + 2 * (size_t)comp * m + 2 * k;
+        double *o = sums + (size_t)items[q].slot * 4 * m + 2 * (size_t)comp * m + 2 * k;
         o[0] = red[0].hi;
         o[1] = red[0].lo;
     }
 }
 
 // One thread per item: Qbar and sigma (Eq. (lattice), Eq. (lattice-error)).
-__global__ void batch_finalize_kernel(const BatchItem *__restrict__ items, int count, int m, int cplx,
+__global__ void batch_finalize_kernel(const Integral *__restrict__ items, int count, int m, int cplx,
                                       const double *__restrict__ sums, double *__restrict__ results) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= count) return;
     const double dn = (double)items[q].n;
-    double *res = results + 4 * (size_t)q;
+    const size_t slot = items[q].slot;
+    double *res = results + 4 * slot;
     for (int comp = 0; comp < 2; ++comp) {
         if (comp == 1 && !cplx) {
             res[2] = 0.0;
             res[3] = 0.0;
             break;
         }
-        const double *__restrict__ sc = sums + (size_t)q * 4 * m + 2 * (size_t)comp * m;
+        const double *__restrict__ sc = sums + slot * 4 * m + 2 * (size_t)comp * m;
         double mean = 0.0;
 #pragma unroll 8
         for (int k = 0; k < m; ++k) mean += (sc[2 * k] + sc[2 * k + 1]) / dn;
@@ -90,27 +90,20 @@ __global__ void batch_finalize_kernel(const BatchItem *__restrict__ items, int c
     }
 }
 
-template <int FAM>
-cudaError_t launch_batch_fam(const BatchItem *items, const uint64_t *tb, int count, uint64_t tiles,
-                             int m, int spb, double *partials, unsigned long long *counters,
-                             cudaStream_t s) {
-    const uint64_t grid = std::min<uint64_t>(tiles, 0x7FFFFFFFull);
-    batch_kernel<FAM><<<(unsigned)grid, spb * m, 0, s>>>(items, tb, count, tiles, m, spb, partials, counters);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_batch(int family, const BatchItem *items, const uint64_t *tb, int count,
-                         uint64_t tiles, int m, int spb, double *partials,
-                         unsigned long long *counters, cudaStream_t s) {
-    switch (family) {
-    case QMC_GENZ_OSCILLATORY: return launch_batch_fam<QMC_GENZ_OSCILLATORY>(items, tb, count, tiles, m, spb, partials, counters, s);
-    case QMC_GENZ_PRODUCT_PEAK: return launch_batch_fam<QMC_GENZ_PRODUCT_PEAK>(items, tb, count, tiles, m, spb, partials, counters, s);
-    case QMC_GENZ_CORNER_PEAK: return launch_batch_fam<QMC_GENZ_CORNER_PEAK>(items, tb, count, tiles, m, spb, partials, counters, s);
-    case QMC_GENZ_GAUSSIAN: return launch_batch_fam<QMC_GENZ_GAUSSIAN>(items, tb, count, tiles, m, spb, partials, counters, s);
-    case QMC_SECTOR: return launch_batch_fam<QMC_SECTOR>(items, tb, count, tiles, m, spb, partials, counters, s);
-    case QMC_FEYNMAN: return launch_batch_fam<QMC_FEYNMAN>(items, tb, count, tiles, m, spb, partials, counters, s);
-    default: return cudaErrorInvalidValue;
-    }
+cudaError_t launch_batch(int family, int tkind, int max_d, const Integral *items, const uint64_t *tb,
+                         int count, uint64_t first_tile, uint64_t end_tile, int m, int spb,
+                         double *partials, unsigned long long *counters, cudaStream_t s) {
+    LatticeLaunch lp{};
+    lp.items = items;
+    lp.tile_begin = tb;
+    lp.count = count;
+    lp.m = m;
+    lp.spb = spb;
+    lp.first_tile = first_tile;
+    lp.end_tile = end_tile;
+    lp.partials = partials;
+    lp.counters = counters;
+    return launch_sums_any(family, tkind, lp, max_d, s);
 }
 
 bool batch_family_supported(int fam) {
@@ -118,20 +111,20 @@ bool batch_family_supported(int fam) {
            fam == QMC_GENZ_GAUSSIAN || fam == QMC_SECTOR || fam == QMC_FEYNMAN;
 }
 
-cudaError_t launch_batch_reduce(const BatchItem *d_items, int count, int m, int cplx,
+cudaError_t launch_batch_reduce(const Integral *d_items, int count, int m, int cplx,
                                 const double *partials, double *sums, cudaStream_t s) {
     const uint64_t blocks = (uint64_t)count * m * (cplx ? 2 : 1);
     batch_reduce_kernel<<<(unsigned)blocks, kBatchRedThreads, 0, s>>>(d_items, m, cplx, partials, sums);
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_finalize(const BatchItem *d_items, int count, int m, int cplx,
+cudaError_t launch_batch_finalize(const Integral *d_items, int count, int m, int cplx,
                                   const double *sums, double *results, cudaStream_t s) {
     batch_finalize_kernel<<<(count + 127) / 128, 128, 0, s>>>(d_items, count, m, cplx, sums, results);
     return cudaGetLastError();
 }
 
-int fill_batch_item(BatchItem &it, const qmc_batch_item &b, int m, int spb, uint32_t Lcfg, int fam) {
+int fill_batch_item(Integral &it, const qmc_batch_item &b, int m, int spb, uint32_t Lcfg, int fam) {
     int st = check_integrand_shape(&b.f);
     if (st) return st;
     if ((st = check_rule(&b.rule))) return st;
@@ -144,32 +137,7 @@ int fill_batch_item(BatchItem &it, const qmc_batch_item &b, int m, int spb, uint
         Geometry g = geometry(range, m);
         L = (g.spb == spb) ? g.L : points_per_stream(range, (uint64_t)spb);
     }
-    const uint64_t ptile = (uint64_t)spb * L;
-    std::memset(&it, 0, sizeof(it));
-    it.n = b.rule.n;
-    it.i_begin = b.i_begin;
-    it.i_end = b.i_end;
-    it.tiles = (range + ptile - 1) / ptile;
-    it.L = L;
-    it.d = b.rule.dim;
-    for (int j = 0; j < it.d; ++j) it.dc[j] = dim_const(b.rule.z[j] % b.rule.n, b.rule.n);
-    it.shifts = b.rule.shifts;
-    it.t = make_transform(b.rule.transform);
-    it.cd = korobov_cd(b.rule.transform, it.t, it.d);
-    it.fit = b.rule.fit;
-    it.family = fam;
-    it.c = b.f.c;
-    it.w = b.f.w;
-    it.h = b.f.h;
-    it.nu = b.f.nu;
-    it.nf = b.f.nf;
-    it.ucoef = b.f.ucoef;
-    it.fcoef = b.f.fcoef;
-    it.uexp = b.f.uexp;
-    it.fexp = b.f.fexp;
-    it.pa = b.f.pa;
-    it.pb = b.f.pb;
-    it.lam = b.f.lambda;
+    fill_integral(it, &b.f, &b.rule, b.i_begin, b.i_end, spb, L);
     return QMC_OK;
 }
 
@@ -178,7 +146,11 @@ int fill_batch_item(BatchItem &it, const qmc_batch_item &b, int m, int spb, uint
 namespace {
 
 struct BatchPlan {
-    std::vector<BatchItem> items;
+    std::vector<Integral> items;        // grouped by transform kind, in input order within one
+    struct Group {
+        int kind, begin, end, max_d;
+    };
+    std::vector<Group> groups;          // one launch each
     std::vector<uint64_t> tile_begin;   // count + 1
     uint64_t total_tiles = 0;
     uint64_t partial_doubles = 0;
@@ -202,23 +174,34 @@ int plan_batch(const qmc_batch_item *in, int count, const qmc_batch_config *cfg,
     P.cplx = is_complex_family(fam);
     P.items.resize(count);
     P.tile_begin.resize(count + 1);
+    P.groups.clear();
+    for (int q = 0; q < count; ++q) {
+        int st = fill_batch_item(P.items[q], in[q], m, spb, Lcfg, fam);
+        if (st) return st;
+        P.items[q].slot = q;
+    }
+    // the kernel is compiled per transform kind: a batch of one kind (the usual one) is one
+    // launch in input order, a mixed one a launch per kind
+    std::stable_sort(P.items.begin(), P.items.end(),
+                     [](const Integral &a, const Integral &b) { return a.t.kind < b.t.kind; });
     uint64_t tiles = 0, poff = 0;
     for (int q = 0; q < count; ++q) {
-        BatchItem &it = P.items[q];
-        int st = fill_batch_item(it, in[q], m, spb, Lcfg, fam);
-        if (st) return st;
+        Integral &it = P.items[q];
         it.tile_begin = tiles;
         it.partial_off = poff;
         P.tile_begin[q] = tiles;
         tiles += it.tiles;
         poff += it.tiles * (uint64_t)m * 2 * (P.cplx ? 2 : 1);
+        if (P.groups.empty() || P.groups.back().kind != it.t.kind) P.groups.push_back({it.t.kind, q, q, 0});
+        P.groups.back().end = q + 1;
+        P.groups.back().max_d = std::max(P.groups.back().max_d, it.d);
     }
     P.tile_begin[count] = tiles;
     P.total_tiles = tiles;
     P.partial_doubles = poff;
     size_t o = 0;
     P.off_items = o;
-    o += align256(sizeof(BatchItem) * count);
+    o += align256(sizeof(Integral) * count);
     P.off_tb = o;
     o += align256(sizeof(uint64_t) * (count + 1));
     P.off_partials = o;
@@ -231,11 +214,14 @@ int plan_batch(const qmc_batch_item *in, int count, const qmc_batch_config *cfg,
 int launch_planned(const BatchPlan &P, int count, void *workspace, double *sums, double *results,
                    unsigned long long *counters, cudaStream_t s) {
     char *ws = (char *)workspace;
-    BatchItem *d_items = (BatchItem *)(ws + P.off_items);
+    Integral *d_items = (Integral *)(ws + P.off_items);
     uint64_t *d_tb = (uint64_t *)(ws + P.off_tb);
     double *d_part = (double *)(ws + P.off_partials);
-    if (launch_batch(P.family, d_items, d_tb, count, P.total_tiles, P.m, P.spb, d_part, counters, s) != cudaSuccess)
-        return QMC_ERR_CUDA;
+    for (const auto &g : P.groups)
+        if (launch_batch(P.family, g.kind, g.max_d, d_items + g.begin, d_tb + g.begin, g.end - g.begin,
+                         P.tile_begin[g.begin], P.tile_begin[g.end], P.m, P.spb, d_part, counters,
+                         s) != cudaSuccess)
+            return QMC_ERR_CUDA;
     if (launch_batch_reduce(d_items, count, P.m, P.cplx, d_part, sums, s) != cudaSuccess) return QMC_ERR_CUDA;
     if (results) {
         if (P.m < 2) return QMC_ERR_M;
@@ -248,7 +234,7 @@ int launch_planned(const BatchPlan &P, int count, void *workspace, double *sums,
 int run_batch(const BatchPlan &P, int count, void *workspace, double *sums, double *results,
               unsigned long long *counters, cudaStream_t s) {
     char *ws = (char *)workspace;
-    if (cudaMemcpyAsync(ws + P.off_items, P.items.data(), sizeof(BatchItem) * count, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(ws + P.off_items, P.items.data(), sizeof(Integral) * count, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(ws + P.off_tb, P.tile_begin.data(), sizeof(uint64_t) * (count + 1), cudaMemcpyHostToDevice, s) != cudaSuccess)
         return QMC_ERR_CUDA;
     return launch_planned(P, count, workspace, sums, results, counters, s);
@@ -274,7 +260,7 @@ extern "C" int qmc_batch_plan_create(const qmc_batch_item *items, int count,
     if (!st) {
         cudaStream_t s = (cudaStream_t)stream;
         char *ws = (char *)workspace;
-        if (cudaMemcpyAsync(ws + plan->P.off_items, plan->P.items.data(), sizeof(BatchItem) * count,
+        if (cudaMemcpyAsync(ws + plan->P.off_items, plan->P.items.data(), sizeof(Integral) * count,
                             cudaMemcpyHostToDevice, s) != cudaSuccess ||
             cudaMemcpyAsync(ws + plan->P.off_tb, plan->P.tile_begin.data(),
                             sizeof(uint64_t) * (count + 1), cudaMemcpyHostToDevice, s) != cudaSuccess ||

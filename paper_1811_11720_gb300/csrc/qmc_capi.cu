@@ -123,43 +123,31 @@ int qmc_sums(const qmc_integrand *f, const qmc_rule *rule, uint64_t i_begin, uin
     if ((st = device_ok())) return st;
     cudaStream_t s = (cudaStream_t)stream;
 
-    SumsParams p;
-    std::memset(&p, 0, sizeof(p));
-    p.n = rule->n;
-    p.i_begin = i_begin;
-    p.i_end = i_end;
-    p.d = rule->dim;
-    for (int j = 0; j < rule->dim; ++j) p.dc[j] = dim_const(rule->z[j] % rule->n, rule->n);
-    p.t = make_transform(rule->transform);
-    p.cd = korobov_cd(rule->transform, p.t, rule->dim);
-    p.fit = rule->fit;
-    fill_integrand(p, f);
-    p.counters = counters;
-
+    LatticeLaunch lp{};
     char *ws = (char *)workspace;
     const uint64_t m = rule->m;
     for (uint64_t k0 = 0; k0 < m; k0 += kMaxShiftGroup) {
         const int mg = (int)std::min<uint64_t>(kMaxShiftGroup, m - k0);
         Geometry g = geometry(i_end - i_begin, mg);
-        p.m = mg;
-        p.spb = g.spb;
-        p.L = g.L;
-        p.tiles = g.tiles;
-        p.shifts = rule->shifts + k0 * rule->dim;
-        p.partials = (double *)ws;
-        cudaError_t e = launch_sums_any(f->family, p.t.kind, dim3((unsigned)g.tiles),
-                                        dim3(g.threads), s, p);
+        if (k0 == 0 || (int)lp.m != mg) fill_integral(lp.one, f, rule, i_begin, i_end, g.spb, g.L);
+        lp.one.shifts = rule->shifts + k0 * rule->dim;
+        lp.m = mg;
+        lp.spb = g.spb;
+        lp.end_tile = g.tiles;
+        lp.partials = (double *)ws;
+        lp.counters = counters;
+        cudaError_t e = launch_sums_any(f->family, lp.one.t.kind, lp, rule->dim, s);
         if (e != cudaSuccess) return QMC_ERR_CUDA;
         // sums layout: re pairs for all m, then im pairs for all m; group k0 writes its slice
         double *grp = sums + 2 * k0;
         if (!cplx) {
-            e = launch_reduce_tiles(p.partials, g.tiles, mg, 0, grp, s);
+            e = launch_reduce_tiles(lp.partials, g.tiles, mg, 0, grp, s);
         } else {
             // the reduce kernel writes [re (2 mg)] [im (2 mg)] contiguously; reduce each
             // component separately so that im lands at sums + 2m + 2 k0
-            e = launch_reduce_tiles(p.partials, g.tiles, mg, 0, grp, s);
+            e = launch_reduce_tiles(lp.partials, g.tiles, mg, 0, grp, s);
             if (e == cudaSuccess)
-                e = launch_reduce_tiles(p.partials + 2 * g.tiles * (uint64_t)mg, g.tiles, mg, 0,
+                e = launch_reduce_tiles(lp.partials + 2 * g.tiles * (uint64_t)mg, g.tiles, mg, 0,
                                         sums + 2 * m + 2 * k0, s);
         }
         if (e != cudaSuccess) return QMC_ERR_CUDA;
@@ -195,26 +183,15 @@ int qmc_sums_tiles(const qmc_integrand *f, const qmc_rule *rule, uint64_t i_begi
 
     // the tiles of the whole range's decomposition: same L and streams per block, the
     // first point moved to tile_begin, the global end kept for the ragged last tile
-    SumsParams p;
-    std::memset(&p, 0, sizeof(p));
-    p.n = rule->n;
-    p.i_begin = i_begin + tile_begin * (uint64_t)g.spb * g.L;
-    p.i_end = i_end;
-    p.d = rule->dim;
-    for (int j = 0; j < rule->dim; ++j) p.dc[j] = dim_const(rule->z[j] % rule->n, rule->n);
-    p.t = make_transform(rule->transform);
-    p.cd = korobov_cd(rule->transform, p.t, rule->dim);
-    p.fit = rule->fit;
-    fill_integrand(p, f);
-    p.counters = counters;
-    p.m = mg;
-    p.spb = g.spb;
-    p.L = g.L;
-    p.tiles = tile_end - tile_begin;
-    p.shifts = rule->shifts;
-    p.partials = partials;
-    cudaError_t e = launch_sums_any(f->family, p.t.kind, dim3((unsigned)p.tiles), dim3(g.threads),
-                                    (cudaStream_t)stream, p);
+    LatticeLaunch lp{};
+    fill_integral(lp.one, f, rule, i_begin + tile_begin * (uint64_t)g.spb * g.L, i_end, g.spb, g.L);
+    lp.one.tiles = tile_end - tile_begin;
+    lp.m = mg;
+    lp.spb = g.spb;
+    lp.end_tile = lp.one.tiles;
+    lp.partials = partials;
+    lp.counters = counters;
+    cudaError_t e = launch_sums_any(f->family, lp.one.t.kind, lp, rule->dim, (cudaStream_t)stream);
     return e == cudaSuccess ? QMC_OK : QMC_ERR_CUDA;
 }
 
@@ -274,17 +251,16 @@ int qmc_evaluate(const qmc_integrand *f, uint64_t n, const uint64_t *z, int dim,
         if (z[j] % n == 0 || gcd_u64(z[j] % n, n) != 1) return QMC_ERR_GENVEC;
     if ((st = device_ok())) return st;
     if (count == 0) return QMC_OK;
-    SumsParams p;
+    Integral p;
     std::memset(&p, 0, sizeof(p));
     p.n = n;
     p.i_begin = i_begin;
     p.i_end = i_begin + count;
     p.d = dim;
-    p.m = 1;
     for (int j = 0; j < dim; ++j) p.dc[j] = dim_const(z[j] % n, n);
     p.shifts = shift;
     fill_integrand(p, f);
-    return cuda_status(launch_evaluate(p, out, (cudaStream_t)stream));
+    return cuda_status(launch_evaluate(f->family, p, out, (cudaStream_t)stream));
 }
 
 static uint32_t hist_blocks(uint64_t n) {
@@ -311,17 +287,16 @@ int qmc_histogram(const qmc_integrand *f, uint64_t n, const uint64_t *z, int dim
     uint32_t nb = hist_blocks(n);
     if (workspace_bytes < (size_t)nb * dim * bins * sizeof(double)) return QMC_ERR_WORKSPACE;
     if ((st = device_ok())) return st;
-    SumsParams p;
+    Integral p;
     std::memset(&p, 0, sizeof(p));
     p.n = n;
     p.i_begin = 0;
     p.i_end = n;
     p.d = dim;
-    p.m = 1;
     for (int j = 0; j < dim; ++j) p.dc[j] = dim_const(z[j] % n, n);
     p.shifts = shift;
     fill_integrand(p, f);
-    return cuda_status(launch_histogram(p, bins, hist, (double *)workspace, nb, (cudaStream_t)stream));
+    return cuda_status(launch_histogram(f->family, p, bins, hist, (double *)workspace, nb, (cudaStream_t)stream));
 }
 
 }  // extern "C"

@@ -205,8 +205,7 @@ inline Geometry geometry(uint64_t range, int mg) {
 
 inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-inline void fill_integrand(SumsParams &p, const qmc_integrand *f) {
-    p.family = f->family;
+inline void fill_integrand(Integral &p, const qmc_integrand *f) {
     p.c = f->c;
     p.w = f->w;
     p.h = f->h;
@@ -221,16 +220,37 @@ inline void fill_integrand(SumsParams &p, const qmc_integrand *f) {
     p.lam = f->lambda;
 }
 
-inline cudaError_t launch_sums_any(int family, int tkind, dim3 g, dim3 b, cudaStream_t s, const SumsParams &p) {
+inline cudaError_t launch_sums_any(int family, int tkind, const LatticeLaunch &lp, int max_d,
+                                   cudaStream_t s) {
     switch (family) {
     case QMC_GENZ_OSCILLATORY: case QMC_GENZ_PRODUCT_PEAK: case QMC_GENZ_CORNER_PEAK: case QMC_GENZ_GAUSSIAN:
-        return launch_sums_genz(family, tkind, g, b, s, p);
+        return launch_sums_genz(family, tkind, lp, max_d, s);
     case QMC_GENZ_C0: case QMC_GENZ_DISCONTINUOUS: case QMC_MONOMIAL: case QMC_TRIG:
-        return launch_sums_other(family, tkind, g, b, s, p);
+        return launch_sums_other(family, tkind, lp, max_d, s);
     case QMC_SECTOR: case QMC_FEYNMAN:
-        return launch_sums_poly(family, tkind, g, b, s, p);
+        return launch_sums_poly(family, tkind, lp, max_d, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// The device description of one integral over [i_begin, i_end) in tiles of spb L points
+// (arguments checked by the caller).
+inline void fill_integral(Integral &it, const qmc_integrand *f, const qmc_rule *rule,
+                          uint64_t i_begin, uint64_t i_end, int spb, uint32_t L) {
+    std::memset(&it, 0, sizeof(it));
+    it.n = rule->n;
+    it.i_begin = i_begin;
+    it.i_end = i_end;
+    const uint64_t ptile = (uint64_t)spb * L;
+    it.tiles = (i_end - i_begin + ptile - 1) / ptile;
+    it.L = L;
+    it.d = rule->dim;
+    for (int j = 0; j < it.d; ++j) it.dc[j] = dim_const(rule->z[j] % rule->n, rule->n);
+    it.shifts = rule->shifts;
+    it.t = make_transform(rule->transform);
+    it.cd = korobov_cd(rule->transform, it.t, it.d);
+    it.fit = rule->fit;
+    fill_integrand(it, f);
 }
 
 }  // namespace host

@@ -15,6 +15,7 @@
 // indexed by the reflection bit mask.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 
 #include "qmc_cos.cuh"
 #include "qmc_exp.cuh"
@@ -58,7 +59,8 @@ struct FixedForms {
     bool ok;
 };
 
-struct FamilyShared {
+// A family's constants in shared memory: of the separable families, or of the polynomial ones.
+struct SeparableShared {
     double c[kMaxDim], w[kMaxDim], aux[kMaxDim];
     double mcw[kMaxDim];    // -c w
     double c1w[kMaxDim];    // c (1 - w)
@@ -73,8 +75,14 @@ struct FamilyShared {
     };
     double exp2t[32];       // 2^(j/32) for exp_table
     FixedForms fx;
+};
+struct PolyFamilyShared {
     PolyShared poly;
 };
+template <int FAM>
+constexpr bool kPolyFamily = FAM == QMC_SECTOR || FAM == QMC_FEYNMAN;
+template <int FAM>
+using FamilyShared = std::conditional_t<kPolyFamily<FAM>, PolyFamilyShared, SeparableShared>;
 
 template <int FAM>
 constexpr bool kHasFixedForm = FAM == QMC_GENZ_OSCILLATORY || FAM == QMC_GENZ_PRODUCT_PEAK ||
@@ -158,7 +166,7 @@ __device__ __forceinline__ void stage_fixed_forms(const P &p, FixedForms &fx) {
 // Subset sums of c over the reflected dimensions, for the FP64 forms of families 1, 3
 // and 6 (reflected_c_sum); the fixed-point forms do not read them.
 template <int FAM, class P>
-__device__ __forceinline__ void stage_subset_sums(const P &p, FamilyShared &fs) {
+__device__ __forceinline__ void stage_subset_sums(const P &p, SeparableShared &fs) {
     if constexpr (FAM == QMC_GENZ_OSCILLATORY || FAM == QMC_GENZ_CORNER_PEAK ||
                   FAM == QMC_GENZ_DISCONTINUOUS) {
         for (int b = threadIdx.x; b < 256; b += blockDim.x) {
@@ -175,13 +183,13 @@ __device__ __forceinline__ void stage_subset_sums(const P &p, FamilyShared &fs) 
     }
 }
 
-// P: SumsParams or BatchItem (fields d, c, w, h, nu, nf, ucoef, fcoef, uexp, fexp, pa, pb, lam).
+// P: Integral (fields d, c, w, h, nu, nf, ucoef, fcoef, uexp, fexp, pa, pb, lam).
 // kSubsets = false leaves the subset-sum tables to the caller (stage_subset_sums), which
 // builds them only when an FP64 form may run.
 template <int FAM, bool kSubsets = true, class P>
-__device__ __forceinline__ void stage_family(const P &p, FamilyShared &fs) {
+__device__ __forceinline__ void stage_family(const P &p, FamilyShared<FAM> &fs) {
     const int tid = threadIdx.x;
-    if constexpr (FAM == QMC_SECTOR || FAM == QMC_FEYNMAN) {
+    if constexpr (kPolyFamily<FAM>) {
         stage_poly(p, fs.poly, FAM == QMC_SECTOR);
     } else {
         if (tid < p.d) {
@@ -213,7 +221,7 @@ template <int FAM>
 struct FamilyAcc;
 
 // sum of c_j over reflected dimensions
-__device__ __forceinline__ double reflected_c_sum(uint32_t mask, int d, const FamilyShared &fs) {
+__device__ __forceinline__ double reflected_c_sum(uint32_t mask, int d, const SeparableShared &fs) {
     double r = fs.sub_lo[mask & 255u];
     if (d > 8) r += fs.sub_hi[(mask >> 8) & 255u];
     return r;
@@ -226,12 +234,12 @@ struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
     static constexpr int kIntFinishMaxR = 4;   // integer finish up to this Korobov order
     double s;
     uint32_t mask;
-    __device__ __forceinline__ void init(const FamilyShared &fs) { s = fs.s0; mask = 0; }
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &fs) {
+    __device__ __forceinline__ void init(const SeparableShared &fs) { s = fs.s0; mask = 0; }
+    __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         s = fma(m.refl ? -fs.c[j] : fs.c[j], m.y, s);
         mask |= (uint32_t)m.refl << j;
     }
-    __device__ __forceinline__ void finish(int d, const FamilyShared &fs, double &re, double &im,
+    __device__ __forceinline__ void finish(int d, const SeparableShared &fs, double &re, double &im,
                                            unsigned long long &) {
         re = cos(mask ? s + reflected_c_sum(mask, d, fs) : s);
         im = 0.0;
@@ -241,7 +249,7 @@ struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
     uint64_t sl;
     __device__ __forceinline__ void init_fixed() { sl = 0; }
     template <bool kInt>
-    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const FamilyShared &fs) {
+    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         if constexpr (kInt) {
             // the integer turns per unit x only when some c_j >= 2 pi (a uniform branch;
             // the Genz ranges have ||c||_1 = 6)
@@ -252,7 +260,7 @@ struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
         }
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const FamilyShared &fs, double &re,
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
                                                  double &im, unsigned long long &) {
         if constexpr (kInt) re = cos_turns_fixed(sl + fs.fx.t0, fs.cos256);
         else re = cos(fs.s0 + scaled_fixed(sl, fs.fx.S));
@@ -266,13 +274,13 @@ struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
     static constexpr bool kComplex = false;
     static constexpr int kIntFinishMaxR = 6;   // integer finish up to this Korobov order
     double prod;
-    __device__ __forceinline__ void init(const FamilyShared &) { prod = 1.0; }
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &fs) {
+    __device__ __forceinline__ void init(const SeparableShared &) { prod = 1.0; }
+    __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         // x - w = y - w, or (1 - w) - y when reflected
         double t = m.refl ? fs.w1[j] - m.y : m.y - fs.w[j];
         prod *= fma(t, t, fs.aux[j]);
     }
-    __device__ __forceinline__ void finish(int, const FamilyShared &, double &re, double &im,
+    __device__ __forceinline__ void finish(int, const SeparableShared &, double &re, double &im,
                                            unsigned long long &) {
         re = 1.0 / prod;
         im = 0.0;
@@ -282,7 +290,7 @@ struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
     Fx pf;
     __device__ __forceinline__ void init_fixed() { pf = {0x8000000000000000ull, 1}; }
     template <bool kInt>
-    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const FamilyShared &fs) {
+    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
         const uint64_t a = x >= w ? x - w : w - x;                       // |x - w| 2^64
         const uint64_t q = mulhi_trunc(a, fs.fx.cq[j]);                 // c |x - w| 2^S
@@ -290,7 +298,7 @@ struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
         pf = fx_norm(fx_mul(pf, fx_norm({s, 128 - 2 * fs.fx.S})));
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const FamilyShared &fs, double &re,
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
                                                  double &im, unsigned long long &) {
         // prod c_j^2 times the reciprocal of the product (Newton on the integer pipe), or
         // one FP64 division
@@ -307,12 +315,12 @@ struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
     static constexpr int kIntFinishMaxR = 1;   // integer finish up to this Korobov order
     double s;
     uint32_t mask;
-    __device__ __forceinline__ void init(const FamilyShared &) { s = 1.0; mask = 0; }
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &fs) {
+    __device__ __forceinline__ void init(const SeparableShared &) { s = 1.0; mask = 0; }
+    __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         s = fma(m.refl ? -fs.c[j] : fs.c[j], m.y, s);
         mask |= (uint32_t)m.refl << j;
     }
-    __device__ __forceinline__ void finish(int d, const FamilyShared &fs, double &re, double &im,
+    __device__ __forceinline__ void finish(int d, const SeparableShared &fs, double &re, double &im,
                                            unsigned long long &) {
         const double t = mask ? s + reflected_c_sum(mask, d, fs) : s;
         re = 1.0 / ipow_u(t, d + 1);
@@ -321,11 +329,11 @@ struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
     uint64_t sl;
     __device__ __forceinline__ void init_fixed() { sl = 0; }
     template <bool kInt>
-    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const FamilyShared &fs) {
+    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         sl += mulhi_trunc(x, fs.fx.cl[j]);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int d, const FamilyShared &fs, double &re,
+    __device__ __forceinline__ void finish_fixed(int d, const SeparableShared &fs, double &re,
                                                  double &im, unsigned long long &) {
         if constexpr (kInt) {
             // 1 + s as Fx (s = sl 2^-S, sl < 2^63; S = 64 drops sl's lowest bit), its
@@ -347,13 +355,13 @@ struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
     static constexpr bool kComplex = false;
     static constexpr int kIntFinishMaxR = 3;   // integer finish up to this Korobov order
     double s;
-    __device__ __forceinline__ void init(const FamilyShared &) { s = 0.0; }
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &fs) {
+    __device__ __forceinline__ void init(const SeparableShared &) { s = 0.0; }
+    __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         // c (x - w) = c y - c w, or -c y + c (1 - w) when reflected: one fused multiply-add
         const double q = fma(m.refl ? -fs.c[j] : fs.c[j], m.y, m.refl ? fs.c1w[j] : fs.mcw[j]);
         s = fma(q, q, s);
     }
-    __device__ __forceinline__ void finish(int, const FamilyShared &, double &re, double &im,
+    __device__ __forceinline__ void finish(int, const SeparableShared &, double &re, double &im,
                                            unsigned long long &) {
         re = exp(-s);
         im = 0.0;
@@ -362,14 +370,14 @@ struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
     uint64_t sq;
     __device__ __forceinline__ void init_fixed() { sq = 0; }
     template <bool kInt>
-    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const FamilyShared &fs) {
+    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
         const uint64_t a = x >= w ? x - w : w - x;                       // |x - w| 2^64
         const uint64_t q = mulhi_trunc(a, fs.fx.cq[j]);                 // c |x - w| 2^S
         sq += sqhi_trunc(q);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const FamilyShared &fs, double &re,
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
                                                  double &im, unsigned long long &) {
         if constexpr (kInt) re = fx_to_double_sat(exp_fixed(sq, 2 * fs.fx.S - 64, true, fs.exp2q));
         else re = exp_table(-scaled_fixed(sq, 2 * fs.fx.S - 64), fs.exp2t);
@@ -383,12 +391,12 @@ struct FamilyAcc<QMC_GENZ_C0> {
     static constexpr bool kComplex = false;
     static constexpr int kIntFinishMaxR = 3;   // integer finish up to this Korobov order
     double s;
-    __device__ __forceinline__ void init(const FamilyShared &) { s = 0.0; }
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &fs) {
+    __device__ __forceinline__ void init(const SeparableShared &) { s = 0.0; }
+    __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         double t = m.refl ? fs.w1[j] - m.y : m.y - fs.w[j];
         s = fma(fs.c[j], fabs(t), s);
     }
-    __device__ __forceinline__ void finish(int, const FamilyShared &, double &re, double &im,
+    __device__ __forceinline__ void finish(int, const SeparableShared &, double &re, double &im,
                                            unsigned long long &) {
         re = exp(-s);
         im = 0.0;
@@ -396,13 +404,13 @@ struct FamilyAcc<QMC_GENZ_C0> {
     uint64_t sl;
     __device__ __forceinline__ void init_fixed() { sl = 0; }
     template <bool kInt>
-    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const FamilyShared &fs) {
+    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
         const uint64_t a = x >= w ? x - w : w - x;                       // |x - w| 2^64
         sl += mulhi_trunc(a, fs.fx.cl[j]);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const FamilyShared &fs, double &re,
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
                                                  double &im, unsigned long long &) {
         if constexpr (kInt) re = fx_to_double_sat(exp_fixed(sl, fs.fx.S, true, fs.exp2q));
         else re = exp_table(-scaled_fixed(sl, fs.fx.S), fs.exp2t);
@@ -418,15 +426,15 @@ struct FamilyAcc<QMC_GENZ_DISCONTINUOUS> {
     double s;
     uint32_t mask;
     bool zero;
-    __device__ __forceinline__ void init(const FamilyShared &) { s = 0.0; mask = 0; zero = false; }
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &fs) {
+    __device__ __forceinline__ void init(const SeparableShared &) { s = 0.0; mask = 0; zero = false; }
+    __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         // x > w is y > w, or (1 - y > w, i.e. y < 1 - w) when reflected; w may lie outside
         // [0, 1] here (the fixed-point form covers 0 <= w <= 1), so compare as doubles
         if (j < 2) zero |= m.refl ? (fs.w1[j] > m.y) : (m.y > fs.w[j]);
         s = fma(m.refl ? -fs.c[j] : fs.c[j], m.y, s);
         mask |= (uint32_t)m.refl << j;
     }
-    __device__ __forceinline__ void finish(int d, const FamilyShared &fs, double &re, double &im,
+    __device__ __forceinline__ void finish(int d, const SeparableShared &fs, double &re, double &im,
                                            unsigned long long &) {
         re = zero ? 0.0 : exp(mask ? s + reflected_c_sum(mask, d, fs) : s);
         im = 0.0;
@@ -434,12 +442,12 @@ struct FamilyAcc<QMC_GENZ_DISCONTINUOUS> {
     uint64_t sl;
     __device__ __forceinline__ void init_fixed() { sl = 0; zero = false; }
     template <bool kInt>
-    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const FamilyShared &fs) {
+    __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         if (j < 2) zero |= x > fs.fx.w64[j];
         sl += mulhi_trunc(x, fs.fx.cl[j]);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const FamilyShared &fs, double &re,
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
                                                  double &im, unsigned long long &) {
         if constexpr (kInt) re = zero ? 0.0 : fx_to_double_sat(exp_fixed(sl, fs.fx.S, false, fs.exp2q));
         else re = zero ? 0.0 : exp_table(scaled_fixed(sl, fs.fx.S), fs.exp2t);
@@ -452,9 +460,9 @@ template <>
 struct FamilyAcc<QMC_MONOMIAL> {
     static constexpr bool kComplex = false;
     double prod;
-    __device__ __forceinline__ void init(const FamilyShared &) { prod = 1.0; }
-    __device__ __forceinline__ void add(int, const Mapped &m, const FamilyShared &) { prod *= reflected(m); }
-    __device__ __forceinline__ void finish(int, const FamilyShared &, double &re, double &im,
+    __device__ __forceinline__ void init(const SeparableShared &) { prod = 1.0; }
+    __device__ __forceinline__ void add(int, const Mapped &m, const SeparableShared &) { prod *= reflected(m); }
+    __device__ __forceinline__ void finish(int, const SeparableShared &, double &re, double &im,
                                            unsigned long long &) {
         re = prod;
         im = 0.0;
@@ -466,12 +474,12 @@ template <>
 struct FamilyAcc<QMC_TRIG> {
     static constexpr bool kComplex = false;
     double prod;
-    __device__ __forceinline__ void init(const FamilyShared &) { prod = 1.0; }
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &fs) {
+    __device__ __forceinline__ void init(const SeparableShared &) { prod = 1.0; }
+    __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         double a = fma((double)fs.h[j], reflected(m), fs.w[j]);
         prod *= fma(fs.c[j], cospi(2.0 * a), 1.0);
     }
-    __device__ __forceinline__ void finish(int, const FamilyShared &, double &re, double &im,
+    __device__ __forceinline__ void finish(int, const SeparableShared &, double &re, double &im,
                                            unsigned long long &) {
         re = prod;
         im = 0.0;
@@ -483,9 +491,9 @@ template <>
 struct FamilyAcc<QMC_SECTOR> {
     static constexpr bool kComplex = false;
     double x[kMaxDim];
-    __device__ __forceinline__ void init(const FamilyShared &) {}
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &) { x[j] = reflected(m); }
-    __device__ __forceinline__ void finish(int d, const FamilyShared &fs, double &re, double &im,
+    __device__ __forceinline__ void init(const PolyFamilyShared &) {}
+    __device__ __forceinline__ void add(int j, const Mapped &m, const PolyFamilyShared &) { x[j] = reflected(m); }
+    __device__ __forceinline__ void finish(int d, const PolyFamilyShared &fs, double &re, double &im,
                                            unsigned long long &) {
         re = sector_value(x, d, fs.poly);
         im = 0.0;
@@ -497,9 +505,9 @@ template <>
 struct FamilyAcc<QMC_FEYNMAN> {
     static constexpr bool kComplex = true;
     double x[kMaxDim];
-    __device__ __forceinline__ void init(const FamilyShared &) {}
-    __device__ __forceinline__ void add(int j, const Mapped &m, const FamilyShared &) { x[j] = reflected(m); }
-    __device__ __forceinline__ void finish(int d, const FamilyShared &fs, double &re, double &im,
+    __device__ __forceinline__ void init(const PolyFamilyShared &) {}
+    __device__ __forceinline__ void add(int j, const Mapped &m, const PolyFamilyShared &) { x[j] = reflected(m); }
+    __device__ __forceinline__ void finish(int d, const PolyFamilyShared &fs, double &re, double &im,
                                            unsigned long long &signfail) {
         feynman_value(x, d, fs.poly, re, im, signfail);
     }

@@ -8,14 +8,12 @@
 
 namespace qmc {
 
-// Launches sums_kernel<FAM, TK> for the family group compiled in one translation unit.
+// Launches lattice_kernel<FAM, TK> for the family group compiled in one translation unit;
+// max_d: the largest dimension among the integrals (sizes the block's shift table).
 // Returns cudaErrorInvalidValue when (family, transform) is not in that group.
-cudaError_t launch_sums_genz(int family, int tkind, dim3 grid, dim3 block, cudaStream_t s,
-                             const SumsParams &p);
-cudaError_t launch_sums_other(int family, int tkind, dim3 grid, dim3 block, cudaStream_t s,
-                              const SumsParams &p);
-cudaError_t launch_sums_poly(int family, int tkind, dim3 grid, dim3 block, cudaStream_t s,
-                             const SumsParams &p);
+cudaError_t launch_sums_genz(int family, int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
+cudaError_t launch_sums_other(int family, int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
+cudaError_t launch_sums_poly(int family, int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
 
 struct PointsParams {
     uint64_t n, i_begin, count;
@@ -36,22 +34,25 @@ cudaError_t launch_reduce_tiles(const double *partials, uint64_t tiles, int m, i
 cudaError_t launch_finalize(const double *sums, int m, uint64_t n, int is_complex,
                             double *result, double *Q, cudaStream_t s);
 
-cudaError_t launch_evaluate(const SumsParams &p, double *out, cudaStream_t s);
-cudaError_t launch_histogram(const SumsParams &p, int bins, double *hist, double *work,
+cudaError_t launch_evaluate(int family, const Integral &p, double *out, cudaStream_t s);
+cudaError_t launch_histogram(int family, const Integral &p, int bins, double *hist, double *work,
                              uint32_t nblocks, cudaStream_t s);
 
 int sm_count();
 
 // Batch building blocks shared by qmc_batch_sums and the serving loop.  Item partial
-// offsets are relative to `partials`.
-int fill_batch_item(BatchItem &it, const qmc_batch_item &b, int m, int spb, uint32_t Lcfg, int fam);
+// offsets are relative to `partials`; sums, results and counters are indexed by the items'
+// slots.
+int fill_batch_item(Integral &it, const qmc_batch_item &b, int m, int spb, uint32_t Lcfg, int fam);
 bool batch_family_supported(int fam);
-cudaError_t launch_batch(int family, const BatchItem *items, const uint64_t *tile_begin, int count,
-                         uint64_t tiles, int m, int spb, double *partials,
+// One launch over items[0..count) of one transform kind, tiles [first_tile, end_tile).
+cudaError_t launch_batch(int family, int tkind, int max_d, const Integral *items,
+                         const uint64_t *tile_begin, int count, uint64_t first_tile,
+                         uint64_t end_tile, int m, int spb, double *partials,
                          unsigned long long *counters, cudaStream_t s);
-cudaError_t launch_batch_reduce(const BatchItem *d_items, int count, int m, int cplx,
+cudaError_t launch_batch_reduce(const Integral *d_items, int count, int m, int cplx,
                                 const double *partials, double *sums, cudaStream_t s);
-cudaError_t launch_batch_finalize(const BatchItem *d_items, int count, int m, int cplx,
+cudaError_t launch_batch_finalize(const Integral *d_items, int count, int m, int cplx,
                                   const double *sums, double *results, cudaStream_t s);
 
 }  // namespace qmc

@@ -19,39 +19,9 @@ namespace qmc {
 // columns are cut into equal chunks (blockIdx.y).  The instructions per double decide how
 // near the floor it comes: ~75 with the remainder stepped and all three words rounded, which
 // ran at 2.5 TB/s (1,072,187 points, d = 8, m = 4: 111 us; one thread per 64 points, its
-// writes scattered: 381 us), ~40 with the two short forms below: 61 us, 4.5 TB/s.
+// writes scattered: 381 us), ~40 with the short step and the short rounding of
+// qmc_lattice.cuh: 61 us, 4.5 TB/s.
 constexpr int kPointThreads = 256;
-
-// kShort, n < 2^32: the fraction is carried to 192 bits and stepped by one long addition
-// instead of an exact remainder.  The third word, i rq mod 2^64, is low by less than i + steps
-// < 2^33 units, so a carry out of it can be missed only where the true fraction of a unit of
-// 2^-128, rem / n, is below 2^33 / 2^64: with n < 2^32 only for rem = 0, that is at multiples
-// of n, where no thread steps to (points stop at i = n - 1).
-struct ShortState {
-    uint64_t f_hi, f_lo, f_2;
-    __device__ __forceinline__ void step(const DimConst &c) {
-        asm("add.cc.u64 %0, %0, %3; addc.cc.u64 %1, %1, %4; addc.u64 %2, %2, %5;"
-            : "+l"(f_2), "+l"(f_lo), "+l"(f_hi)
-            : "l"(c.rq), "l"(c.fz_lo), "l"(c.fz_hi));
-    }
-};
-
-__device__ __noinline__ double point_slow(uint64_t vhi, uint64_t vlo, uint64_t rem, uint64_t n) {
-    return fixed_to_double(vhi, vlo, rem, n);
-}
-
-// fixed_to_double for v >= 2^-10 with bits below the top word (vlo != 0, all but ~2^-10 of the
-// points): the top word holds the 53 bits and the round bit, and what lies below them is not
-// zero, so no bit of vlo is needed.
-__device__ __forceinline__ double point_round(uint64_t vhi, uint64_t vlo, uint64_t n) {
-    const uint32_t top = (uint32_t)(vhi >> 32);
-    if (top < 0x00400000u || !vlo) return point_slow(vhi, vlo, 0 - vlo * n, n);
-    const int lz = __clz(top);   // 0..9
-    const uint32_t hi = __funnelshift_l((uint32_t)vhi, top, lz) ^ 0x80000000u;   // leading one off
-    const uint32_t lo = ((uint32_t)vhi << lz) | 1u;                              // sticky
-    const uint64_t m = ((uint64_t)hi << 32 | lo) + (0x3FFu + ((lo >> 11) & 1u));
-    return __longlong_as_double((long long)((m >> 11) + ((uint64_t)(1022 - lz) << 52)));
-}
 
 template <bool kShort>
 __global__ void __launch_bounds__(kPointThreads) points_kernel(const __grid_constant__ PointsParams p) {
@@ -77,15 +47,15 @@ __global__ void __launch_bounds__(kPointThreads) points_kernel(const __grid_cons
         step.rq = step.rq ? rows * c.rq : 0;   // (a whole number of periods leaves none)
         ShortState s{fh, fl, i0 * c.rq};
         for (uint32_t q = 0; q < cnt; ++q) {
-            __stcs(o, point_round(s.f_hi + dsh, s.f_lo, n));
-            s.step(step);
+            __stcs(o, fixed_to_double(s.f_hi + dsh, s.f_lo, n));
+            s.step(step.fz_hi, step.fz_lo, step.rq);
             o += stride;
         }
     } else {
         LatticeStep step;
         lattice_state_at(rows, c, n, step.fz_hi, step.fz_lo, step.remz);
         for (uint32_t q = 0; q < cnt; ++q) {
-            __stcs(o, fixed_to_double(fh + dsh, fl, rem, n));
+            __stcs(o, fixed_to_double(fh + dsh, fl, n));
             lattice_step(step, n, fh, fl, rem);
             o += stride;
         }
@@ -110,7 +80,7 @@ cudaError_t launch_points(PointsParams p, cudaStream_t s) {
     }
     const dim3 grid((unsigned)blocks, chunks);
     const int threads = p.rows * p.cols;
-    if (p.n >> 32) points_kernel<false><<<grid, threads, 0, s>>>(p);
+    if (p.n >> kShortBits) points_kernel<false><<<grid, threads, 0, s>>>(p);
     else points_kernel<true><<<grid, threads, 0, s>>>(p);
     return cudaGetLastError();
 }
@@ -222,7 +192,7 @@ cudaError_t launch_finalize(const double *sums, int m, uint64_t n, int is_comple
 
 // ---- evaluate(): raw f on one shifted lattice, no transform ---------------------------
 template <int FAM>
-__device__ __forceinline__ void eval_point(const FamilyShared &fsh, const double *x, int d,
+__device__ __forceinline__ void eval_point(const FamilyShared<FAM> &fsh, const double *x, int d,
                                            double &re, double &im, unsigned long long &sf) {
     FamilyAcc<FAM> fa;
     fa.init(fsh);
@@ -236,8 +206,8 @@ constexpr int kEvalThreads = 128;
 constexpr uint32_t kEvalChunk = 32;
 
 template <int FAM>
-__global__ void __launch_bounds__(kEvalThreads) evaluate_kernel(const SumsParams p, double *out) {
-    __shared__ FamilyShared fsh;
+__global__ void __launch_bounds__(kEvalThreads) evaluate_kernel(const Integral p, double *out) {
+    __shared__ FamilyShared<FAM> fsh;
     stage_family<FAM>(p, fsh);
     __syncthreads();
     const int d = p.d;
@@ -258,7 +228,7 @@ __global__ void __launch_bounds__(kEvalThreads) evaluate_kernel(const SumsParams
             for (int j = 0; j < kMaxDim; ++j) {
                 x[j] = 0.0;
                 if (j < d) {
-                    x[j] = fixed_to_double(fhi[j] + dsh[j], flo[j], rem[j], p.n);
+                    x[j] = fixed_to_double(fhi[j] + dsh[j], flo[j], p.n);
                     lattice_step(lattice_step_of(p.dc[j], p.n), p.n, fhi[j], flo[j], rem[j]);
                 }
             }
@@ -281,10 +251,10 @@ __global__ void __launch_bounds__(kEvalThreads) evaluate_kernel(const SumsParams
 // (deterministic).  Block histograms go to work[block][d][bins] and are summed over
 // blocks in block order by hist_sum_kernel.
 template <int FAM>
-__global__ void __launch_bounds__(kEvalThreads) histogram_kernel(const SumsParams p, int bins,
+__global__ void __launch_bounds__(kEvalThreads) histogram_kernel(const Integral p, int bins,
                                                                  double *work) {
     extern __shared__ double hsm[];   // [d][bins]
-    __shared__ FamilyShared fsh;
+    __shared__ FamilyShared<FAM> fsh;
     __shared__ double val[kEvalThreads];
     __shared__ uint16_t bin[kEvalThreads][kMaxDim];
     stage_family<FAM>(p, fsh);
@@ -309,7 +279,7 @@ __global__ void __launch_bounds__(kEvalThreads) histogram_kernel(const SumsParam
                 if (j < d) {
                     uint64_t fh, fl, rm;
                     lattice_state_at(i, p.dc[j], n, fh, fl, rm);
-                    x[j] = fixed_to_double(fh + dsh[j], fl, rm, n);
+                    x[j] = fixed_to_double(fh + dsh[j], fl, n);
                     int b = (int)floor(x[j] * (double)bins);
                     bin[threadIdx.x][j] = (uint16_t)(b >= bins ? bins - 1 : b);
                 }
@@ -346,7 +316,7 @@ __global__ void hist_sum_kernel(const double *work, uint32_t nblocks, int cells,
 }
 
 template <int FAM>
-static cudaError_t eval_dispatch_one(const SumsParams &p, double *out, cudaStream_t s) {
+static cudaError_t eval_dispatch_one(const Integral &p, double *out, cudaStream_t s) {
     uint64_t count = p.i_end - p.i_begin;
     uint64_t chunks = (count + kEvalChunk - 1) / kEvalChunk;
     uint32_t blocks = (uint32_t)((chunks + kEvalThreads - 1) / kEvalThreads);
@@ -357,7 +327,7 @@ static cudaError_t eval_dispatch_one(const SumsParams &p, double *out, cudaStrea
 }
 
 template <int FAM>
-static cudaError_t hist_dispatch_one(const SumsParams &p, int bins, double *hist, double *work,
+static cudaError_t hist_dispatch_one(const Integral &p, int bins, double *hist, double *work,
                                      uint32_t nblocks, cudaStream_t s) {
     size_t smem = (size_t)p.d * bins * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(histogram_kernel<FAM>,
@@ -372,7 +342,7 @@ static cudaError_t hist_dispatch_one(const SumsParams &p, int bins, double *hist
 }
 
 #define QMC_FAMILY_SWITCH(FN, ...)                                                      \
-    switch (p.family) {                                                                 \
+    switch (family) {                                                                 \
     case QMC_GENZ_OSCILLATORY: return FN<QMC_GENZ_OSCILLATORY>(__VA_ARGS__);            \
     case QMC_GENZ_PRODUCT_PEAK: return FN<QMC_GENZ_PRODUCT_PEAK>(__VA_ARGS__);          \
     case QMC_GENZ_CORNER_PEAK: return FN<QMC_GENZ_CORNER_PEAK>(__VA_ARGS__);            \
@@ -386,11 +356,11 @@ static cudaError_t hist_dispatch_one(const SumsParams &p, int bins, double *hist
     default: return cudaErrorInvalidValue;                                              \
     }
 
-cudaError_t launch_evaluate(const SumsParams &p, double *out, cudaStream_t s) {
+cudaError_t launch_evaluate(int family, const Integral &p, double *out, cudaStream_t s) {
     QMC_FAMILY_SWITCH(eval_dispatch_one, p, out, s)
 }
 
-cudaError_t launch_histogram(const SumsParams &p, int bins, double *hist, double *work,
+cudaError_t launch_histogram(int family, const Integral &p, int bins, double *hist, double *work,
                              uint32_t nblocks, cudaStream_t s) {
     QMC_FAMILY_SWITCH(hist_dispatch_one, p, bins, hist, work, nblocks, s)
 }

@@ -93,6 +93,22 @@ __device__ __forceinline__ void lattice_step(const LatticeStep &c, uint64_t n, u
     f_hi = f_hi + c.fz_hi + c1 + c2;
 }
 
+// The same step for n < 2^32: the fraction is carried to 192 bits, started with the third
+// word i rq mod 2^64 and stepped by one long addition, without an exact remainder.  The third
+// word is low by less than i units, so a carry out of it can be missed only where the true
+// fraction of a unit of 2^-128, rem / n, is below i / 2^64 < 1 / n: only for rem = 0, at
+// multiples of n, and a stream of points 0 <= i < n steps to none (it may start at i = 0,
+// where all three words are exact).
+constexpr int kShortBits = 32;
+struct ShortState {
+    uint64_t f_hi, f_lo, f_2;
+    __device__ __forceinline__ void step(uint64_t z_hi, uint64_t z_lo, uint64_t z_2) {
+        asm("add.cc.u64 %0, %0, %3; addc.cc.u64 %1, %1, %4; addc.u64 %2, %2, %5;"
+            : "+l"(f_2), "+l"(f_lo), "+l"(f_hi)
+            : "l"(z_2), "l"(z_lo), "l"(z_hi));
+    }
+};
+
 // Round (vhi:vlo + rem/n) 2^-128 to the nearest double; general path for vhi == 0.
 static __device__ __noinline__ double fixed_to_double_small(uint64_t vlo, uint64_t rem, uint64_t n) {
     if (vlo == 0 && rem == 0) return 0.0;
@@ -122,9 +138,9 @@ static __device__ __noinline__ double fixed_to_double_small(uint64_t vlo, uint64
     return __longlong_as_double((long long)(((uint64_t)bexp << 52) + mant));
 }
 
-// u = RN((V + rem/n) 2^-128) for V = (vhi:vlo).  Fast path for vhi != 0.
-__device__ __forceinline__ double fixed_to_double(uint64_t vhi, uint64_t vlo, uint64_t rem,
-                                                  uint64_t n) {
+// u = RN((V + rem/n) 2^-128) for V = (vhi:vlo), any point.
+static __device__ __noinline__ double fixed_to_double_any(uint64_t vhi, uint64_t vlo, uint64_t n) {
+    const uint64_t rem = 0 - vlo * n;   // F n = -rem modulo 2^64; the shift leaves F's low word
     if (vhi == 0) return fixed_to_double_small(vlo, rem, n);
     int lz = __clzll(vhi);
     uint64_t whi = lz ? ((vhi << lz) | (vlo >> (64 - lz))) : vhi;
@@ -136,6 +152,19 @@ __device__ __forceinline__ double fixed_to_double(uint64_t vhi, uint64_t vlo, ui
     // value = mant 2^(-53-lz), biased exponent 1022 - lz; adding mant (implicit bit
     // included) to (exponent - 1) << 52 also handles the carry mant == 2^53.
     return __longlong_as_double((long long)(((uint64_t)(1021 - lz) << 52) + mant));
+}
+
+// The same.  A point v >= 2^-10 with bits below its top word (vlo != 0: all but ~2^-10 of
+// them) is rounded from that word alone: it holds the 53 bits and the round bit, and what lies
+// below is not zero.
+__device__ __forceinline__ double fixed_to_double(uint64_t vhi, uint64_t vlo, uint64_t n) {
+    const uint32_t top = (uint32_t)(vhi >> 32);
+    if (top < 0x00400000u || !vlo) return fixed_to_double_any(vhi, vlo, n);
+    const int lz = __clz(top);   // 0..9
+    const uint32_t hi = __funnelshift_l((uint32_t)vhi, top, lz) ^ 0x80000000u;   // leading one off
+    const uint32_t lo = ((uint32_t)vhi << lz) | 1u;                              // sticky
+    const uint64_t m = ((uint64_t)hi << 32 | lo) + (0x3FFu + ((lo >> 11) & 1u));
+    return __longlong_as_double((long long)((m >> 11) + ((uint64_t)(1022 - lz) << 52)));
 }
 
 }  // namespace qmc

@@ -29,50 +29,40 @@ struct TransformParams {
     double sidi_c[kMaxSidi + 1];  // Sidi: phi = cr * I_r, I_r via the sin-power reduction
 };
 
-struct SumsParams {
-    uint64_t n;
-    uint64_t i_begin, i_end;
-    uint64_t tiles;
-    uint32_t L;        // points per stream and tile
-    int d, m, spb;     // dimension, shifts, streams per block (blockDim = spb * m)
-    DimConst dc[kMaxDim];
-    const uint64_t *shifts;   // [m][d]
-    TransformParams t;
-    double cd;                // Korobov C^d, 1 for the other transforms
-    const double *fit;        // [d][6] or nullptr
-    // integrand (device pointers; the kernel stages them in shared memory)
-    int family;
-    const double *c, *w;
-    const int64_t *h;
-    int nu, nf;
-    const double *ucoef, *fcoef;
-    const int32_t *uexp, *fexp;
-    double pa, pb, lam;
-    // outputs
-    double *partials;                 // [tiles][m] (sum, comp) re, then [tiles][m] im
-    unsigned long long *counters;     // [2] or nullptr
-};
-
-// One integral of a batch (qmc_batch_sums), built on the host and kept in the workspace.
-// Field names match SumsParams so the staging and per-stream code serve both kernels.
-struct BatchItem {
+// One integral as the kernels see it: of a launch of its own (passed as a kernel parameter)
+// or of a batch (qmc_batch_*: built on the host and kept in the workspace).
+struct Integral {
     uint64_t n, i_begin, i_end;
-    uint64_t tile_begin, tiles;   // global index of the first tile, number of tiles
-    uint64_t partial_off;         // offset of this item's partials, in doubles
+    uint64_t tile_begin, tiles;   // index of the first tile in the launch, number of tiles
+    uint64_t partial_off;         // offset of this integral's partials, in doubles
     uint32_t L;                   // points per stream and tile
     int d;
-    double cd;                    // Korobov C^d
+    double cd;                    // Korobov C^d, 1 for the other transforms
     DimConst dc[kMaxDim];
     const uint64_t *shifts;       // [m][d]
     TransformParams t;
     const double *fit;            // [d][6] or nullptr
-    int family;
+    // integrand (device pointers; the kernel stages them in shared memory)
+    int slot;                     // position of its sums, results and counters in the batch
     const double *c, *w;
     const int64_t *h;
     int nu, nf;
     const double *ucoef, *fcoef;
     const int32_t *uexp, *fexp;
     double pa, pb, lam;
+};
+
+// A launch of the lattice-sum kernel: one integral (items null) or the integrals items[0..count)
+// whose tiles, laid end to end, are numbered by tile_begin[0..count]; all of one transform kind.
+struct LatticeLaunch {
+    Integral one;
+    const Integral *items;
+    const uint64_t *tile_begin;
+    int count;
+    int m, spb;                       // shifts, streams per block (blockDim = spb * m)
+    uint64_t first_tile, end_tile;    // the tiles of this launch
+    double *partials;                 // per integral: [tiles][m] (sum, comp) re, then im
+    unsigned long long *counters;     // [2] per integral, or nullptr
 };
 
 }  // namespace qmc

@@ -77,11 +77,11 @@ struct qmc_server {
     std::map<size_t, size_t> free_blocks;   // offset -> size
     // fixed regions
     size_t fixed_bytes = 0;
-    BatchItem *d_items = nullptr;
+    Integral *d_items = nullptr;
     uint64_t *d_tb = nullptr;
     double *d_sums = nullptr, *d_results = nullptr;
     unsigned long long *d_counters = nullptr;
-    BatchItem *h_items = nullptr;
+    Integral *h_items = nullptr;
     uint64_t *h_tb = nullptr;
     double *h_results = nullptr;
     unsigned long long *h_counters = nullptr;
@@ -247,7 +247,7 @@ extern "C" int qmc_server_create(const qmc_genvec_table *table, const qmc_server
     s->tz.assign(table->z, table->z + (size_t)table->count * table->s_max);
     s->stream = (cudaStream_t)stream;
     const size_t slots = cfg->max_slots;
-    s->fixed_bytes = al256(sizeof(BatchItem) * slots) + al256(sizeof(uint64_t) * (slots + 1)) +
+    s->fixed_bytes = al256(sizeof(Integral) * slots) + al256(sizeof(uint64_t) * (slots + 1)) +
                      al256(sizeof(double) * 4 * cfg->m * slots) + al256(sizeof(double) * 4 * slots) +
                      al256(sizeof(unsigned long long) * 2 * slots);
     if (cfg->memory_budget <= s->fixed_bytes) {
@@ -259,7 +259,7 @@ extern "C" int qmc_server_create(const qmc_genvec_table *table, const qmc_server
         delete s;
         return QMC_ERR_CUDA;
     }
-    if (cudaMallocHost(&s->h_items, sizeof(BatchItem) * slots) != cudaSuccess ||
+    if (cudaMallocHost(&s->h_items, sizeof(Integral) * slots) != cudaSuccess ||
         cudaMallocHost(&s->h_tb, sizeof(uint64_t) * (slots + 1)) != cudaSuccess ||
         cudaMallocHost(&s->h_results, sizeof(double) * 4 * slots) != cudaSuccess ||
         cudaMallocHost(&s->h_counters, sizeof(unsigned long long) * 2 * slots) != cudaSuccess) {
@@ -267,8 +267,8 @@ extern "C" int qmc_server_create(const qmc_genvec_table *table, const qmc_server
         return QMC_ERR_CUDA;
     }
     char *p = s->pool;
-    s->d_items = (BatchItem *)p;
-    p += al256(sizeof(BatchItem) * slots);
+    s->d_items = (Integral *)p;
+    p += al256(sizeof(Integral) * slots);
     s->d_tb = (uint64_t *)p;
     p += al256(sizeof(uint64_t) * (slots + 1));
     s->d_sums = (double *)p;
@@ -392,6 +392,7 @@ extern "C" int qmc_server_step(qmc_server *s, int *completed) {
     for (int fam : fams) {
         const size_t g0 = base;
         uint64_t tiles = 0;
+        int kind = 0, max_d = 1;
         for (uint64_t id : run) {
             Request &r = s->reqs[id];
             if (r.fh.family != fam) continue;
@@ -400,12 +401,15 @@ extern "C" int qmc_server_step(qmc_server *s, int *completed) {
             b.rule = rule_of(s, r);
             b.i_begin = 0;
             b.i_end = r.n;
-            BatchItem &it = s->h_items[base];
+            Integral &it = s->h_items[base];
             int st = fill_batch_item(it, b, m, spb, 0, fam);
             if (st) return st;
             if (it.tiles > r.tiles_cap) return QMC_ERR_WORKSPACE;   // never: see request_bytes
             it.tile_begin = tiles;
+            it.slot = (int)(base - g0);
             it.partial_off = (uint64_t)(r.d_partials - (double *)s->pool);
+            kind = it.t.kind;   // the server's transform: one kind for all
+            max_d = std::max(max_d, it.d);
             s->h_tb[base - g0] = tiles;
             tiles += it.tiles;
             order.push_back(id);
@@ -414,11 +418,12 @@ extern "C" int qmc_server_step(qmc_server *s, int *completed) {
         const int cnt = (int)(base - g0);
         s->h_tb[cnt] = tiles;
         const int cplx = is_complex_family(fam);
-        BatchItem *di = s->d_items + g0;
-        if (cudaMemcpyAsync(di, s->h_items + g0, sizeof(BatchItem) * cnt, cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
+        Integral *di = s->d_items + g0;
+        if (cudaMemcpyAsync(di, s->h_items + g0, sizeof(Integral) * cnt, cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
             cudaMemcpyAsync(s->d_tb, s->h_tb, sizeof(uint64_t) * (cnt + 1), cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
             return QMC_ERR_CUDA;
-        if (launch_batch(fam, di, s->d_tb, cnt, tiles, m, spb, (double *)s->pool, s->d_counters + 2 * g0, s->stream) != cudaSuccess ||
+        if (launch_batch(fam, kind, max_d, di, s->d_tb, cnt, 0, tiles, m, spb, (double *)s->pool,
+                         s->d_counters + 2 * g0, s->stream) != cudaSuccess ||
             launch_batch_reduce(di, cnt, m, cplx, (double *)s->pool, s->d_sums + g0 * 4 * m, s->stream) != cudaSuccess ||
             launch_batch_finalize(di, cnt, m, cplx, s->d_sums + g0 * 4 * m, s->d_results + 4 * g0, s->stream) != cudaSuccess)
             return QMC_ERR_CUDA;

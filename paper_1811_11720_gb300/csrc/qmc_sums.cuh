@@ -1,19 +1,20 @@
-// qmc_sums.cuh -- the persistent lattice-sum kernel (Eq. (lattice)).
+// qmc_sums.cuh -- the lattice-sum kernel (Eq. (lattice)): one integral, or many in one launch.
 //
-// Work decomposition.  The i-range [i_begin, i_end) is cut into tiles of spb * L points;
-// a block of spb * m threads owns one tile at a time (tiles are dealt round-robin to a
-// persistent grid).  Thread (s, k) evaluates shift k on the L consecutive points of
-// stream s, so the 32 lanes of a warp are 32 shifts of the same points when m is a
-// multiple of 32: the lattice state is shared across the warp (see stream_sums) and the
-// instruction stream is uniform.  The transform and, where the integrand allows, the
-// integrand's linear and quadratic forms run in integer fixed point (qmc_fixed.cuh,
-// qmc_integrands.cuh), and under the cheaper maps so does its final function (qmc_exp.cuh,
-// qmc_cos.cuh); FP64 is left to the final function under the higher Korobov orders and to
-// the sums.
+// Work decomposition.  An integral's i-range [i_begin, i_end) is cut into tiles of spb * L
+// points; a block of spb * m threads owns one tile.  In a batch the tiles of all integrals
+// form one sequence and a block looks up its integral, copies the descriptor to shared
+// memory and stages the coefficients; integrals differ in dimension, lattice, fit and
+// coefficients, and share the family and the transform kind (template parameters) and m (the
+// block shape).  Thread (s, k) evaluates shift k on the L consecutive points of stream s.
+// The transform and, where the integrand allows, the integrand's linear and quadratic forms
+// run in integer fixed point (qmc_fixed.cuh, qmc_integrands.cuh), and under the cheaper maps
+// so does its final function (qmc_exp.cuh, qmc_cos.cuh); FP64 is left to the final function
+// under the higher Korobov orders and to the sums.
 // Each thread accumulates its L samples in FP64; the tile's per-shift partial is
 // the Neumaier-compensated sum over its spb streams in fixed order, written to
 // partials[tile][k].  Tiles depend only on the i-range, so the result is bit-identical for
-// any grid size, and sharding on tile boundaries reproduces the same partials.
+// any grid size and in or out of a batch, and sharding on tile boundaries reproduces the
+// same partials.
 #pragma once
 #include <cstdint>
 
@@ -58,40 +59,95 @@ __device__ __forceinline__ void prepare_fit(const double *fit, int d, double *s_
     }
 }
 
-// Per-warp lattice state for the shared-state path: two buffers (the state at point t is
-// written to buffer t & 1) of one slot per lane, in shared memory.
-struct WarpLattice {
-    uint64_t fhi[2][32];
-    uint64_t flo[2][32];
-    uint64_t rem[2][32];
+// ---- lattice state shared by the warp --------------------------------------------------
+// The lanes of a warp are shifts of at most a few streams (one when m is a multiple of 32),
+// and the lattice point does not depend on the shift.  So the warp keeps one state per
+// (stream, coordinate) pair: lane e and, past 32 pairs, lane e - 32 own pair e in registers,
+// step it once per point and publish it to a double-buffered slot of shared memory; every
+// lane reads its stream's d coordinates from there, with one __syncwarp per point.  With the
+// state per thread instead (streams of m = 20 shifts did that: only m dividing 32 or a
+// multiple of 32 shared), each thread steps d coordinates and keeps 3 d words in local
+// memory.  More pairs than kPairs (m below ~6 with many dimensions) still do.
+constexpr int kPairs = 64;
+
+struct WarpStreams {
+    unsigned mask;    // the warp's threads
+    int first;        // first stream of the warp, within the block
+    int mine;         // this lane's stream, counted from `first`
+    int count;        // streams the warp's lanes belong to
 };
 
-// Lanes per stream group of a warp for the shared-state path: 32 when m is a multiple of
-// 32, m when m divides 32 and the stream's shifts can hold the d coordinates; 0 otherwise
-// (each thread keeps its own state).
-__device__ __forceinline__ int lattice_group_lanes(int m, int d) {
-    if (m % 32 == 0) return 32;
-    if (32 % m == 0 && d <= m) return m;
-    return 0;
+__device__ __forceinline__ WarpStreams warp_streams(int m) {
+    const int tid = threadIdx.x, base = tid & ~31;
+    const int last = min(base + 31, (int)blockDim.x - 1);
+    WarpStreams w;
+    w.mask = last - base == 31 ? 0xFFFFFFFFu : (1u << (last - base + 1)) - 1u;
+    w.first = base / m;
+    w.mine = tid / m - w.first;
+    w.count = last / m - w.first + 1;
+    return w;
 }
 
-// Shift accessors: dsh(j) is D_kj 2^11, the thread's 53-bit shift of coordinate j in units
-// of the lattice state's top word.
-struct ShiftsPre {      // values already multiplied by 2^11 (local or shared memory)
-    const uint64_t *s;
-    __device__ __forceinline__ uint64_t operator()(int j) const { return s[j]; }
-};
-struct ShiftsGlobal {   // the caller's row of D_kj in global memory, through the read-only path
-    const uint64_t *D;
-    __device__ __forceinline__ uint64_t operator()(int j) const { return __ldg(D + j) << 11; }
+// Words of the state that a transform reads: the maps that take the coordinate as x 2^64
+// read the top word, the others round both to u.
+template <int TK>
+constexpr bool kTopWordOnly = TK == kTKorobovInt;
+template <int TK>
+constexpr int kWords = kTopWordOnly<TK> ? 1 : 2;
+
+// The step constants of the d coordinates in shared memory (a warp's lanes read different j).
+// z2: the third fraction word for n < 2^32 (ShortState), else the exact remainder.
+struct BlockSteps {
+    uint64_t zh[kMaxDim], zl[kMaxDim], z2[kMaxDim];
+    __device__ __forceinline__ void set(int j, const DimConst &c, uint64_t n) {
+        const LatticeStep st = lattice_step_of(c, n);
+        zh[j] = st.fz_hi;
+        zl[j] = st.fz_lo;
+        z2[j] = n >> kShortBits ? st.remz : c.rq;
+    }
+    __device__ __forceinline__ void start(int j, uint64_t i, const DimConst &c, uint64_t n,
+                                          ShortState &s) const {
+        lattice_state_at(i, c, n, s.f_hi, s.f_lo, s.f_2);
+        if (!(n >> kShortBits)) s.f_2 = i * c.rq;
+    }
+    __device__ __forceinline__ void step(int j, uint64_t n, ShortState &s) const {
+        if (n >> kShortBits) lattice_step(LatticeStep{zh[j], zl[j], z2[j]}, n, s.f_hi, s.f_lo, s.f_2);
+        else s.step(zh[j], zl[j], z2[j]);
+    }
 };
 
-// One evaluation of g at the point whose coordinate j has lattice state (fhi(j), flo(j),
-// rem(j)); adds it to the two-level accumulator.
-template <int FAM, int TK, int R, class P, class Sh, class Hi, class Lo, class Rem>
-__device__ __forceinline__ void eval_point(const P &p, const FamilyShared &fsh, const double *s_fit,
-                                           bool use_fit, Sh dsh, double cd, Hi fhi,
-                                           Lo flo, Rem rem, double &g_re, double &g_im,
+// The published state of one warp: [buffer][word][pair].
+template <int TK>
+struct WarpLattice {
+    uint64_t w[2][kWords<TK>][kPairs];
+};
+
+// A point's coordinates as eval_point reads them: from the warp's buffer or a thread's own.
+struct SharedState {
+    const uint64_t *w;   // this lane's stream in the buffer
+    __device__ __forceinline__ uint64_t hi(int j) const { return w[j]; }
+    __device__ __forceinline__ uint64_t lo(int j) const { return w[kPairs + j]; }
+};
+struct OwnState {
+    const uint64_t *fhi, *flo;
+    __device__ __forceinline__ uint64_t hi(int j) const { return fhi[j]; }
+    __device__ __forceinline__ uint64_t lo(int j) const { return flo[j]; }
+};
+
+// The block's shifts in shared memory, D_kj 2^11 (the 53-bit shift in units of the lattice
+// state's top word) as [j][k]: the lanes of a warp read consecutive words.  (Read from the
+// caller's [k][j] rows through the read-only cache, a warp's load touched up to 20 lines.)
+struct Shifts {
+    const uint64_t *s;
+    int m;
+    __device__ __forceinline__ uint64_t operator()(int j) const { return s[j * m]; }
+};
+
+// One evaluation of g at a point with lattice state `st`.
+template <int FAM, int TK, int R, class St>
+__device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared<FAM> &fsh,
+                                           const double *s_fit, bool use_fit, Shifts dsh, double cd,
+                                           const St &st, double &g_re, double &g_im,
                                            unsigned long long &signfail) {
     Weight W{1.0, 1.0, 1.0, Fx{0x8000000000000000ull, 1}};
     FamilyAcc<FAM> fa;
@@ -107,7 +163,7 @@ __device__ __forceinline__ void eval_point(const P &p, const FamilyShared &fsh, 
             fa.init_fixed();
 #pragma unroll 1
             for (int j = 0; j < p.d; ++j)
-                fa.template add_fixed<kIntFinish>(j, transform_fixed<TK, R>(fhi(j) + dsh(j), W), fsh);
+                fa.template add_fixed<kIntFinish>(j, transform_fixed<TK, R>(st.hi(j) + dsh(j), W), fsh);
             const double wt = weight_finish<TK, R>(W, p.t, cd);
             fa.template finish_fixed<kIntFinish>(p.d, fsh, g_re, g_im, signfail);
             g_re *= wt;
@@ -120,7 +176,7 @@ __device__ __forceinline__ void eval_point(const P &p, const FamilyShared &fsh, 
         if (!use_fit && sector_fixed_ok(fsh.poly, p.d)) {
             uint64_t X[8];
 #pragma unroll 1
-            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(fhi(j) + dsh(j), W);
+            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), W);
             const double wt = weight_finish<TK, R>(W, p.t, cd);
             g_re = sector_value_x(X, p.d, fsh.poly) * wt;
             g_im = 0.0;
@@ -132,7 +188,7 @@ __device__ __forceinline__ void eval_point(const P &p, const FamilyShared &fsh, 
         if (!use_fit && feyn_fixed_ok(fsh.poly, p.d)) {
             uint64_t X[kFeynFixedMaxDim];
 #pragma unroll 1
-            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(fhi(j) + dsh(j), W);
+            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), W);
             const double wt = weight_finish<TK, R>(W, p.t, cd);
             feynman_value_x(X, p.d, fsh.poly, g_re, g_im, signfail);
             g_re *= wt;
@@ -144,14 +200,14 @@ __device__ __forceinline__ void eval_point(const P &p, const FamilyShared &fsh, 
 #pragma unroll 1
     for (int j = 0; j < p.d; ++j) {
         Mapped mx;
-        if constexpr (TK == kTKorobovInt && (FAM == QMC_SECTOR || FAM == QMC_FEYNMAN)) {
+        if constexpr (TK == kTKorobovInt && kPolyFamily<FAM>) {
             // the polynomial families use x itself: formed from x 2^64 by integer
             // operations instead of an FP64 conversion and reflection
-            mx = Mapped{fixed_u64_to_double(transform_fixed<TK, R>(fhi(j) + dsh(j), W), 64), false};
+            mx = Mapped{fixed_u64_to_double(transform_fixed<TK, R>(st.hi(j) + dsh(j), W), 64), false};
         } else if constexpr (TK == kTKorobovInt) {
-            mx = korobov_int_x<R>(fhi(j) + dsh(j), W);
+            mx = korobov_int_x<R>(st.hi(j) + dsh(j), W);
         } else {
-            const double u = fixed_to_double(fhi(j) + dsh(j), flo(j), rem(j), p.n);
+            const double u = fixed_to_double(st.hi(j) + dsh(j), st.lo(j), p.n);
             mx = apply_transform<TK>(u, p.t, W);
         }
         if (use_fit) mx = Mapped{apply_fit(reflected(mx), s_fit + kFitStride * j, W.w), false};
@@ -163,170 +219,142 @@ __device__ __forceinline__ void eval_point(const P &p, const FamilyShared &fsh, 
     if constexpr (FamilyAcc<FAM>::kComplex) g_im *= wt;
 }
 
-// One stream of one shift: sum of g over points [i0, i0 + cnt) of the lattice described by
-// P (fields n, d, dc[], t).  Two-level FP64 accumulation: blocks of kInner samples, then
-// the block sums (rounding error ~ (kInner + L/kInner) ulp instead of L ulp).
-//
-// Lattice state.  When the q = lattice_group_lanes(m, d) lanes of a warp group are q shifts
-// of the same stream (wl != nullptr; q = 32 for m a multiple of 32, q = m for m = 2..16
-// with d <= m), the state is shared: the group's lane j < d keeps coordinate j in
-// registers, computes its start point and steps it, and publishes it to the warp's shared
-// buffer once per point; every lane of the group reads the d coordinates from there
-// (broadcast loads), with one __syncwarp over the group per point.  That is one lattice
-// step per lane and point instead of d.  Otherwise each thread keeps all d coordinates in
-// local memory (L1) and steps them itself.
-template <int FAM, int TK, int R, class P, class Sh>
-__device__ __forceinline__ void stream_sums_r(const P &p, const FamilyShared &fsh, const double *s_fit,
-                                              bool use_fit, Sh dsh, double cd,
-                                              uint64_t i0, uint64_t cnt, WarpLattice *wl,
-                                              int q, double &acc_re, double &acc_im,
-                                              unsigned long long &nonfinite,
-                                              unsigned long long &signfail) {
+// A stream's running sums.  Two-level FP64 accumulation: blocks of kInner samples, then the
+// block sums (rounding error ~ (kInner + L/kInner) ulp instead of L ulp).
+struct StreamSum {
+    double in_re = 0.0, in_im = 0.0, re = 0.0, im = 0.0;
+    unsigned long long nonfinite = 0, signfail = 0;
+    template <bool CPLX>
+    __device__ __forceinline__ void add(double g_re, double g_im) {
+        if (not_finite(g_re) || (CPLX && not_finite(g_im))) ++nonfinite;
+        in_re += g_re;
+        if constexpr (CPLX) in_im += g_im;
+    }
+    template <bool CPLX>
+    __device__ __forceinline__ void flush() {
+        re += in_re;
+        in_re = 0.0;
+        if constexpr (CPLX) {
+            im += in_im;
+            in_im = 0.0;
+        }
+    }
+};
+
+// The sums of one tile: this thread's stream covers points [i0, i0 + cnt) of the lattice,
+// i0 = w0 + mine * L with w0 the first point of the warp's first stream.
+template <int FAM, int TK, int R>
+__device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilyShared<FAM> &fsh,
+                                              const double *s_fit, bool use_fit, Shifts dsh,
+                                              const BlockSteps &steps, const WarpStreams &ws,
+                                              WarpLattice<TK> &lat, uint64_t w0,
+                                              uint32_t cnt, StreamSum &acc) {
     constexpr bool kCplx = FamilyAcc<FAM>::kComplex;
     const int d = p.d;
     const uint64_t n = p.n;
-    double in_re = 0.0, in_im = 0.0;
-    acc_re = 0.0;
-    acc_im = 0.0;
-    if (!cnt) return;
-    auto accumulate = [&](uint64_t t, double g_re, double g_im) {
-        if (not_finite(g_re) || (kCplx && not_finite(g_im))) ++nonfinite;
-        in_re += g_re;
-        if constexpr (kCplx) in_im += g_im;
-        if ((t & (kInner - 1)) == kInner - 1) {
-            acc_re += in_re;
-            in_re = 0.0;
-            if constexpr (kCplx) {
-                acc_im += in_im;
-                in_im = 0.0;
-            }
-        }
-    };
-    if (wl && q == 32) {
-        // the warp is one group: lane j < d owns coordinate j
+    const double cd = p.cd;
+    const int stride = d | 1;   // pairs of a stream in the buffer: odd, no bank conflicts
+    const int pairs = ws.count * d;
+    const int lanes = __popc(ws.mask);   // 32 but in a ragged last warp
+    if (pairs <= 2 * lanes && ws.count * stride <= kPairs) {
+        // this lane's one or two pairs (stream, coordinate)
         const int lane = threadIdx.x & 31;
-        uint64_t fh = 0, fl = 0, rm = 0;
-        const LatticeStep step = lattice_step_of(p.dc[lane < d ? lane : 0], n);
-        if (lane < d) lattice_state_at(i0, p.dc[lane], n, fh, fl, rm);
+        struct Pair {
+            ShortState f{0, 0, 0};
+            int j = 0, at = 0;
+            bool own = false;
+        } a, b;
+        auto start = [&](Pair &s, int e) {
+            s.own = e < pairs;
+            if (!s.own) return;
+            const int st = e / d;
+            s.j = e - st * d;
+            s.at = st * stride + s.j;
+            steps.start(s.j, w0 + (uint64_t)st * p.L, p.dc[s.j], n, s.f);
+        };
+        start(a, lane);
+        start(b, lane + lanes);
+        const uint32_t most = __reduce_max_sync(ws.mask, cnt);
 #pragma unroll 1
-        for (uint64_t t = 0; t < cnt; ++t) {
-            const int b = (int)(t & 1);
-            if (lane < d) {
-                wl->fhi[b][lane] = fh;
-                if constexpr (TK != kTKorobovInt) {
-                    wl->flo[b][lane] = fl;
-                    wl->rem[b][lane] = rm;
-                }
+        for (uint32_t t = 0; t < most; ++t) {
+            auto &buf = lat.w[t & 1];
+            auto publish = [&](Pair &s) {
+                if (!s.own) return;
+                buf[0][s.at] = s.f.f_hi;
+                if constexpr (!kTopWordOnly<TK>) buf[1][s.at] = s.f.f_lo;
+                steps.step(s.j, n, s.f);
+            };
+            publish(a);
+            if (pairs > lanes) publish(b);
+            __syncwarp(ws.mask);
+            if (t < cnt) {
+                double g_re, g_im = 0.0;
+                eval_point<FAM, TK, R>(p, fsh, s_fit, use_fit, dsh, cd,
+                                       SharedState{&buf[0][ws.mine * stride]}, g_re, g_im, acc.signfail);
+                acc.template add<kCplx>(g_re, g_im);
             }
-            __syncwarp();
-            double g_re, g_im = 0.0;
-            eval_point<FAM, TK, R>(
-                p, fsh, s_fit, use_fit, dsh, cd, [&](int j) { return wl->fhi[b][j]; },
-                [&](int j) { return wl->flo[b][j]; }, [&](int j) { return wl->rem[b][j]; }, g_re,
-                g_im, signfail);
-            accumulate(t, g_re, g_im);
-            if (lane < d) lattice_step(step, n, fh, fl, rm);
-        }
-    } else if (wl) {
-        // groups of q < 32 lanes (q divides 32): the group's lane j < d owns coordinate j
-        const int lane = threadIdx.x & 31;
-        const int base = lane & ~(q - 1);
-        const int pos = lane - base;
-        const unsigned mask = ((1u << q) - 1u) << base;
-        uint64_t fh = 0, fl = 0, rm = 0;
-        const LatticeStep step = lattice_step_of(p.dc[pos < d ? pos : 0], n);
-        if (pos < d) lattice_state_at(i0, p.dc[pos], n, fh, fl, rm);
-#pragma unroll 1
-        for (uint64_t t = 0; t < cnt; ++t) {
-            const int b = (int)(t & 1);
-            if (pos < d) {
-                wl->fhi[b][lane] = fh;
-                if constexpr (TK != kTKorobovInt) {
-                    wl->flo[b][lane] = fl;
-                    wl->rem[b][lane] = rm;
-                }
-            }
-            __syncwarp(mask);
-            double g_re, g_im = 0.0;
-            eval_point<FAM, TK, R>(
-                p, fsh, s_fit, use_fit, dsh, cd, [&](int j) { return wl->fhi[b][base + j]; },
-                [&](int j) { return wl->flo[b][base + j]; },
-                [&](int j) { return wl->rem[b][base + j]; }, g_re, g_im, signfail);
-            accumulate(t, g_re, g_im);
-            if (pos < d) lattice_step(step, n, fh, fl, rm);
+            if ((t & (kInner - 1)) == kInner - 1) acc.template flush<kCplx>();
         }
     } else {
-        uint64_t fhi[kMaxDim], flo[kMaxDim], rem[kMaxDim];
+        uint64_t fhi[kMaxDim], flo[kMaxDim], f2[kMaxDim];
+        const uint64_t i0 = w0 + (uint64_t)ws.mine * p.L;
 #pragma unroll 1
-        for (int j = 0; j < d; ++j) lattice_state_at(i0, p.dc[j], n, fhi[j], flo[j], rem[j]);
+        for (int j = 0; j < d; ++j) {
+            ShortState s;
+            steps.start(j, i0, p.dc[j], n, s);
+            fhi[j] = s.f_hi;
+            flo[j] = s.f_lo;
+            f2[j] = s.f_2;
+        }
 #pragma unroll 1
-        for (uint64_t t = 0; t < cnt; ++t) {
+        for (uint32_t t = 0; t < cnt; ++t) {
             double g_re, g_im = 0.0;
-            eval_point<FAM, TK, R>(
-                p, fsh, s_fit, use_fit, dsh, cd, [&](int j) { return fhi[j]; },
-                [&](int j) { return flo[j]; }, [&](int j) { return rem[j]; }, g_re, g_im, signfail);
-            accumulate(t, g_re, g_im);
+            eval_point<FAM, TK, R>(p, fsh, s_fit, use_fit, dsh, cd, OwnState{fhi, flo}, g_re, g_im,
+                                   acc.signfail);
+            acc.template add<kCplx>(g_re, g_im);
+            if ((t & (kInner - 1)) == kInner - 1) acc.template flush<kCplx>();
 #pragma unroll 1
-            for (int j = 0; j < d; ++j) lattice_step(lattice_step_of(p.dc[j], n), n, fhi[j], flo[j], rem[j]);
+            for (int j = 0; j < d; ++j) {
+                ShortState s{fhi[j], flo[j], f2[j]};
+                steps.step(j, n, s);
+                fhi[j] = s.f_hi;
+                flo[j] = s.f_lo;
+                f2[j] = s.f_2;
+            }
         }
     }
-    acc_re += in_re;
-    if constexpr (kCplx) acc_im += in_im;
+    acc.template flush<kCplx>();
 }
 
-// The integer Korobov is compiled once per order r (uniform branch per stream).
-template <int FAM, int TK, class P, class Sh>
-__device__ __forceinline__ void stream_sums(const P &p, const FamilyShared &fsh, const double *s_fit,
-                                            bool use_fit, Sh dsh, double cd,
-                                            uint64_t i0, uint64_t cnt, WarpLattice *wl, int q,
-                                            double &acc_re, double &acc_im,
-                                            unsigned long long &nonfinite,
-                                            unsigned long long &signfail) {
+// The integer Korobov is compiled once per order r (uniform branch per tile).
+template <int FAM, int TK, class... A>
+__device__ __forceinline__ void stream_sums(const Integral &p, A &&...a) {
     if constexpr (TK == kTKorobovInt) {
         switch (p.t.r0) {
-        case 1:
-            stream_sums_r<FAM, TK, 1>(p, fsh, s_fit, use_fit, dsh, cd, i0, cnt, wl, q, acc_re, acc_im,
-                                      nonfinite, signfail);
-            return;
-        case 2:
-            stream_sums_r<FAM, TK, 2>(p, fsh, s_fit, use_fit, dsh, cd, i0, cnt, wl, q, acc_re, acc_im,
-                                      nonfinite, signfail);
-            return;
-        case 3:
-            stream_sums_r<FAM, TK, 3>(p, fsh, s_fit, use_fit, dsh, cd, i0, cnt, wl, q, acc_re, acc_im,
-                                      nonfinite, signfail);
-            return;
-        case 4:
-            stream_sums_r<FAM, TK, 4>(p, fsh, s_fit, use_fit, dsh, cd, i0, cnt, wl, q, acc_re, acc_im,
-                                      nonfinite, signfail);
-            return;
-        case 5:
-            stream_sums_r<FAM, TK, 5>(p, fsh, s_fit, use_fit, dsh, cd, i0, cnt, wl, q, acc_re, acc_im,
-                                      nonfinite, signfail);
-            return;
-        default:
-            stream_sums_r<FAM, TK, 6>(p, fsh, s_fit, use_fit, dsh, cd, i0, cnt, wl, q, acc_re, acc_im,
-                                      nonfinite, signfail);
-            return;
+        case 1: stream_sums_r<FAM, TK, 1>(p, a...); return;
+        case 2: stream_sums_r<FAM, TK, 2>(p, a...); return;
+        case 3: stream_sums_r<FAM, TK, 3>(p, a...); return;
+        case 4: stream_sums_r<FAM, TK, 4>(p, a...); return;
+        case 5: stream_sums_r<FAM, TK, 5>(p, a...); return;
+        default: stream_sums_r<FAM, TK, 6>(p, a...); return;
         }
     } else {
-        stream_sums_r<FAM, TK, 0>(p, fsh, s_fit, use_fit, dsh, cd, i0, cnt, wl, q, acc_re, acc_im,
-                                  nonfinite, signfail);
+        stream_sums_r<FAM, TK, 0>(p, a...);
     }
 }
 
 // Per-shift tile partial: fixed-order compensated sum over the block's spb streams of
-// shift k, written as (sum, compensation) to out_re[2k..] (and out_im).  Contains the
-// block barriers; every thread of the block must call it.
+// shift k, written as (sum, compensation) to out_re[2k..] (and out_im).  Contains a block
+// barrier; every thread of the block must call it.
 template <bool CPLX>
-__device__ __forceinline__ void tile_partial(double acc_re, double acc_im, double *s_red, int m,
-                                             int spb, int s_local, int k, bool active,
+__device__ __forceinline__ void tile_partial(const StreamSum &acc, double *s_red, int m, int spb,
                                              double *out_re, double *out_im) {
     const int tid = threadIdx.x;
-    s_red[tid] = acc_re;
-    if constexpr (CPLX) s_red[kSumsThreads + tid] = acc_im;
+    s_red[tid] = acc.re;
+    if constexpr (CPLX) s_red[kSumsThreads + tid] = acc.im;
     __syncthreads();
-    if (s_local == 0 && active) {
+    if (tid < m) {
+        const int k = tid;
         double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
         for (int s = 0; s < spb; ++s) {
             neumaier_add(sr, cr, s_red[s * m + k]);
@@ -339,87 +367,80 @@ __device__ __forceinline__ void tile_partial(double acc_re, double acc_im, doubl
             out_im[2 * k + 1] = ci;
         }
     }
-    __syncthreads();
 }
 
 // Blocks per SM the register allocation must allow: five for the separable families (48
-// registers; their throughput depends on hiding integer latency), no constraint for the
-// polynomial families (their per-thread working set needs the registers).
+// registers; their throughput depends on hiding integer latency), two for the sector family
+// (128 registers; left to itself the compiler takes more and one block runs alone: 9.0 ms
+// instead of 5.9 at d = 8, n = 1,072,187, m = 32), no constraint for the complex family (its
+// working set needs the registers).
 template <int FAM>
-constexpr bool kPolyFamily = FAM == QMC_SECTOR || FAM == QMC_FEYNMAN;
-template <int FAM>
-constexpr int kSumsMinBlocks = kPolyFamily<FAM> ? 1 : 5;
+constexpr int kSumsMinBlocks = FAM == QMC_FEYNMAN ? 1 : FAM == QMC_SECTOR ? 2 : 5;
 
+// Dynamic shared memory: the shifts, [kMaxDim or d][m].
 template <int FAM, int TK>
 __global__ void __launch_bounds__(kSumsThreads, kSumsMinBlocks<FAM>)
-    sums_kernel(const __grid_constant__ SumsParams p) {
-    __shared__ FamilyShared fsh;
+    lattice_kernel(const __grid_constant__ LatticeLaunch lp) {
+    extern __shared__ uint64_t s_dsh[];
+    __shared__ FamilyShared<FAM> fsh;
     __shared__ double s_fit[kMaxDim * kFitStride];
-    __shared__ double s_red[2 * kSumsThreads];
-    __shared__ WarpLattice s_lat[kSumsThreads / 32];
+    __shared__ double s_red[(FamilyAcc<FAM>::kComplex ? 2 : 1) * kSumsThreads];
+    __shared__ WarpLattice<TK> s_lat[kSumsThreads / 32];
+    __shared__ Integral s_item;
+    __shared__ BlockSteps s_step;
+    __shared__ int s_q;
     constexpr bool kCplx = FamilyAcc<FAM>::kComplex;
 
     const int tid = threadIdx.x;
-    stage_family<FAM, false>(p, fsh);
-    prepare_fit(p.fit, p.d, s_fit);
-    __syncthreads();
-    if constexpr (kHasFixedForm<FAM>) {
-        // the FP64 forms' subset-sum tables (256 FP64 sums per block), only when the
-        // fixed-point form does not take every evaluation (uniform over the block)
-        if (!(kFixedTransform<TK> && p.fit == nullptr && fsh.fx.ok)) {
-            stage_subset_sums<FAM>(p, fsh);
+    const int m = lp.m, spb = lp.spb;
+    const WarpStreams ws = warp_streams(m);
+    for (uint64_t tile = lp.first_tile + blockIdx.x; tile < lp.end_tile; tile += gridDim.x) {
+        __syncthreads();   // the previous tile's shared data is no longer read
+        const Integral *src = &lp.one;
+        if (lp.items) {
+            // the integral whose tiles hold this one: every thread looks at its share of the
+            // prefix sums, one round of loads instead of a chain of them
+            for (int q = tid; q < lp.count; q += blockDim.x)
+                if (lp.tile_begin[q] <= tile && tile < lp.tile_begin[q + 1]) s_q = q;
             __syncthreads();
+            src = lp.items + s_q;
         }
-    }
-
-    const int m = p.m, d = p.d;
-    const int k = tid % m;
-    const int s_local = tid / m;
-    const bool active = s_local < p.spb;
-    const double cd = p.cd;   // Korobov C^d (host-computed; 1 otherwise)
-
-    // The shifts D_kj, read once per dimension of every evaluation.  Under the cheap maps
-    // (baker, none) the separable families stage them, times 2^11 (the 53-bit shift in the
-    // high word's units), in shared memory, in the polynomial buffer they do not use, as
-    // [k][j] rows of odd length (the warp's lanes hit distinct banks).  Otherwise each
-    // thread reads its row of the caller's array through the read-only cache: the block's
-    // m rows (m d 8 bytes) are shared by all its warps and stay in L1, where a copy per
-    // thread in local memory (spb times as much) missed.
-    unsigned long long nonfinite = 0, signfail = 0;
-    const uint64_t ptile = (uint64_t)p.spb * p.L;
-    const int q = lattice_group_lanes(m, d);
-    auto run_tiles = [&](auto dsh) {
-        for (uint64_t tile = blockIdx.x; tile < p.tiles; tile += gridDim.x) {
-            const uint64_t i0 = p.i_begin + tile * ptile + (uint64_t)s_local * p.L;
-            uint64_t cnt = 0;
-            if (active && i0 < p.i_end) cnt = (p.i_end - i0 < p.L) ? (p.i_end - i0) : p.L;
-            double acc_re, acc_im;
-            stream_sums<FAM, TK>(p, fsh, s_fit, p.fit != nullptr, dsh, cd, i0, cnt,
-                                 q ? &s_lat[tid >> 5] : nullptr, q, acc_re, acc_im, nonfinite,
-                                 signfail);
-            double *out_re = p.partials + 2 * (tile * (uint64_t)m);
-            double *out_im = p.partials + 2 * (p.tiles * (uint64_t)m) + 2 * (tile * (uint64_t)m);
-            tile_partial<kCplx>(acc_re, acc_im, s_red, m, p.spb, s_local, k, active, out_re, out_im);
+        for (int w = tid; w < (int)(sizeof(Integral) / 8); w += blockDim.x)
+            reinterpret_cast<uint64_t *>(&s_item)[w] = reinterpret_cast<const uint64_t *>(src)[w];
+        __syncthreads();
+        const Integral &it = s_item;
+        const int d = it.d;
+        for (int i = tid; i < m * d; i += blockDim.x) {
+            const int k = i / d, j = i - k * d;
+            s_dsh[j * m + k] = it.shifts[i] << 11;
         }
-    };
-    bool staged = false;
-    if constexpr (!kPolyFamily<FAM> && (TK == QMC_T_BAKER || TK == QMC_T_NONE)) {
-        const int ds = d | 1;
-        if (m * ds <= 4 * kMaxTerms) {   // uniform over the block
-            uint64_t *s_dsh = fsh.poly.buf.u;
-            for (int i = tid; i < m * ds; i += blockDim.x) {
-                const int kk = i / ds, j = i - kk * ds;
-                s_dsh[i] = j < d ? (p.shifts[(size_t)kk * d + j] << 11) : 0ull;
+        if (tid < d) s_step.set(tid, it.dc[tid], it.n);
+        stage_family<FAM, false>(it, fsh);
+        prepare_fit(it.fit, d, s_fit);
+        __syncthreads();
+        if constexpr (kHasFixedForm<FAM>) {
+            // the FP64 forms' subset-sum tables (256 FP64 sums per block), only when the
+            // fixed-point form does not take every evaluation (uniform over the block)
+            if (!(kFixedTransform<TK> && it.fit == nullptr && fsh.fx.ok)) {
+                stage_subset_sums<FAM>(it, fsh);
+                __syncthreads();
             }
-            __syncthreads();
-            run_tiles(ShiftsPre{s_dsh + k * ds});
-            staged = true;
         }
-    }
-    if (!staged) run_tiles(ShiftsGlobal{p.shifts + (size_t)k * d});
-    if (p.counters && (nonfinite | signfail)) {
-        if (nonfinite) atomicAdd(p.counters, nonfinite);
-        if (signfail) atomicAdd(p.counters + 1, signfail);
+        const uint64_t local = tile - it.tile_begin;
+        const uint64_t w0 = it.i_begin + (local * (uint64_t)spb + ws.first) * it.L;
+        const uint64_t i0 = w0 + (uint64_t)ws.mine * it.L;
+        uint32_t cnt = 0;
+        if (i0 < it.i_end) cnt = it.i_end - i0 < it.L ? (uint32_t)(it.i_end - i0) : it.L;
+        StreamSum acc;
+        stream_sums<FAM, TK>(it, fsh, s_fit, it.fit != nullptr, Shifts{s_dsh + tid % m, m}, s_step, ws,
+                             s_lat[tid >> 5], w0, cnt, acc);
+        double *base = lp.partials + it.partial_off;
+        tile_partial<kCplx>(acc, s_red, m, spb, base + 2 * (local * (uint64_t)m),
+                            base + 2 * (it.tiles * (uint64_t)m) + 2 * (local * (uint64_t)m));
+        if (lp.counters) {
+            if (acc.nonfinite) atomicAdd(lp.counters + 2 * it.slot, acc.nonfinite);
+            if (acc.signfail) atomicAdd(lp.counters + 2 * it.slot + 1, acc.signfail);
+        }
     }
 }
 

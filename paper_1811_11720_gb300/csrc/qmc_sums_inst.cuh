@@ -1,4 +1,4 @@
-// qmc_sums_inst.cuh -- per-translation-unit instantiation of sums_kernel over the
+// qmc_sums_inst.cuh -- per-translation-unit instantiation of lattice_kernel over the
 // transforms (the four public kinds and the integer-pipe Korobov) for a list of families
 // (split across TUs so nvcc compiles them in parallel).
 #pragma once
@@ -8,20 +8,21 @@
 namespace qmc {
 
 template <int FAM, int TK>
-static cudaError_t launch_one(dim3 grid, dim3 block, cudaStream_t s, const SumsParams &p) {
-    sums_kernel<FAM, TK><<<grid, block, 0, s>>>(p);
+static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s) {
+    const uint64_t tiles = lp.end_tile - lp.first_tile;
+    const uint64_t grid = tiles < 0x7FFFFFFFull ? tiles : 0x7FFFFFFFull;
+    lattice_kernel<FAM, TK><<<(unsigned)grid, lp.spb * lp.m, sizeof(uint64_t) * max_d * lp.m, s>>>(lp);
     return cudaGetLastError();
 }
 
 template <int FAM>
-static cudaError_t launch_family(int tkind, dim3 grid, dim3 block, cudaStream_t s,
-                                 const SumsParams &p) {
+static cudaError_t launch_family(int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s) {
     switch (tkind) {
-    case QMC_T_NONE: return launch_one<FAM, QMC_T_NONE>(grid, block, s, p);
-    case QMC_T_BAKER: return launch_one<FAM, QMC_T_BAKER>(grid, block, s, p);
-    case QMC_T_KOROBOV: return launch_one<FAM, QMC_T_KOROBOV>(grid, block, s, p);
-    case QMC_T_SIDI: return launch_one<FAM, QMC_T_SIDI>(grid, block, s, p);
-    case kTKorobovInt: return launch_one<FAM, kTKorobovInt>(grid, block, s, p);
+    case QMC_T_NONE: return launch_one<FAM, QMC_T_NONE>(lp, max_d, s);
+    case QMC_T_BAKER: return launch_one<FAM, QMC_T_BAKER>(lp, max_d, s);
+    case QMC_T_KOROBOV: return launch_one<FAM, QMC_T_KOROBOV>(lp, max_d, s);
+    case QMC_T_SIDI: return launch_one<FAM, QMC_T_SIDI>(lp, max_d, s);
+    case kTKorobovInt: return launch_one<FAM, kTKorobovInt>(lp, max_d, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -2,11 +2,10 @@
 #include "qmc_sums_inst.cuh"
 
 namespace qmc {
-cudaError_t launch_sums_poly(int family, int tkind, dim3 grid, dim3 block, cudaStream_t s,
-                             const SumsParams &p) {
+cudaError_t launch_sums_poly(int family, int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s) {
     switch (family) {
-    case QMC_SECTOR: return launch_family<QMC_SECTOR>(tkind, grid, block, s, p);
-    case QMC_FEYNMAN: return launch_family<QMC_FEYNMAN>(tkind, grid, block, s, p);
+    case QMC_SECTOR: return launch_family<QMC_SECTOR>(tkind, lp, max_d, s);
+    case QMC_FEYNMAN: return launch_family<QMC_FEYNMAN>(tkind, lp, max_d, s);
     default: return cudaErrorInvalidValue;
     }
 }
