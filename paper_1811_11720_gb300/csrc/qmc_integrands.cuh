@@ -260,11 +260,9 @@ struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
         }
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
-                                                 double &im, unsigned long long &) {
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
         if constexpr (kInt) re = cos_turns_fixed(sl + fs.fx.t0, fs.cos256);
         else re = cos(fs.s0 + scaled_fixed(sl, fs.fx.S));
-        im = 0.0;
     }
 };
 
@@ -298,13 +296,11 @@ struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
         pf = fx_norm(fx_mul(pf, fx_norm({s, 128 - 2 * fs.fx.S})));
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
-                                                 double &im, unsigned long long &) {
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
         // prod c_j^2 times the reciprocal of the product (Newton on the integer pipe), or
         // one FP64 division
         if constexpr (kInt) re = fx_to_double(fx_mul(fs.fx.numx, fx_recip(pf)));
         else re = fs.fx.num / fx_to_double(pf);
-        im = 0.0;
     }
 };
 
@@ -333,8 +329,7 @@ struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
         sl += mulhi_trunc(x, fs.fx.cl[j]);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int d, const SeparableShared &fs, double &re,
-                                                 double &im, unsigned long long &) {
+    __device__ __forceinline__ void finish_fixed(int d, const SeparableShared &fs, double &re) {
         if constexpr (kInt) {
             // 1 + s as Fx (s = sl 2^-S, sl < 2^63; S = 64 drops sl's lowest bit), its
             // (d+1)-th power and the reciprocal, all on the integer pipe
@@ -345,7 +340,6 @@ struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
         } else {
             re = 1.0 / ipow_u(1.0 + scaled_fixed(sl, fs.fx.S), d + 1);
         }
-        im = 0.0;
     }
 };
 
@@ -377,11 +371,9 @@ struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
         sq += sqhi_trunc(q);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
-                                                 double &im, unsigned long long &) {
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
         if constexpr (kInt) re = fx_to_double_sat(exp_fixed(sq, 2 * fs.fx.S - 64, true, fs.exp2q));
         else re = exp_table(-scaled_fixed(sq, 2 * fs.fx.S - 64), fs.exp2t);
-        im = 0.0;
     }
 };
 
@@ -410,11 +402,9 @@ struct FamilyAcc<QMC_GENZ_C0> {
         sl += mulhi_trunc(a, fs.fx.cl[j]);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
-                                                 double &im, unsigned long long &) {
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
         if constexpr (kInt) re = fx_to_double_sat(exp_fixed(sl, fs.fx.S, true, fs.exp2q));
         else re = exp_table(-scaled_fixed(sl, fs.fx.S), fs.exp2t);
-        im = 0.0;
     }
 };
 
@@ -447,11 +437,9 @@ struct FamilyAcc<QMC_GENZ_DISCONTINUOUS> {
         sl += mulhi_trunc(x, fs.fx.cl[j]);
     }
     template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re,
-                                                 double &im, unsigned long long &) {
+    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
         if constexpr (kInt) re = zero ? 0.0 : fx_to_double_sat(exp_fixed(sl, fs.fx.S, false, fs.exp2q));
         else re = zero ? 0.0 : exp_table(scaled_fixed(sl, fs.fx.S), fs.exp2t);
-        im = 0.0;
     }
 };
 

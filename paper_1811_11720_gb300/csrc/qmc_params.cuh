@@ -16,6 +16,9 @@ constexpr int kSumsThreads = 256;   // threads per block of the lattice-sum kern
 // integer fixed point (qmc_fixed.cuh).  The public kind stays QMC_T_KOROBOV.
 constexpr int kTKorobovInt = 4;
 constexpr int kMaxKorobovInt = 6;
+// The asymmetric Korobov<r0,r1>, both orders in 1..kMaxKorobovInt, in integer fixed point
+// with the orders at run time.
+constexpr int kTKorobovGen = 5;
 
 // Korobov<r0,r1> (Eq. (korobov)) as used by the kernels: for u <= 1/2,
 //   phi(u) = u^(r0+1) sum_k A[k] u^k,  A[k] = C (-1)^k binom(r1,k) / (r0+k+1), k <= r1,
@@ -23,8 +26,17 @@ constexpr int kMaxKorobovInt = 6;
 // (B: r0 and r1 exchanged).  The weight is C u^r0 (1-u)^r1, C = (r0+r1+1) binom(r0+r1,r0).
 struct TransformParams {
     int kind, r0, r1, deg;        // deg = max(r0, r1): Horner length (zero-padded)
-    double A[kMaxKorobov + 1];
-    double B[kMaxKorobov + 1];
+    union {
+        struct {
+            double A[kMaxKorobov + 1];
+            double B[kMaxKorobov + 1];
+        };
+        struct {   // kTKorobovGen: binom(r0 + k, k) 2^kf and binom(r1 + k, k) 2^kf, k <= deg
+            uint64_t KA[kMaxKorobovInt + 1];
+            uint64_t KB[kMaxKorobovInt + 1];
+            int kf;
+        };
+    };
     double C;                     // Korobov constant, or Sidi (pi/2^r) Gamma(r+1)/Gamma((r+1)/2)^2
     double sidi_c[kMaxSidi + 1];  // Sidi: phi = cr * I_r, I_r via the sin-power reduction
 };

@@ -91,9 +91,7 @@ __device__ __forceinline__ WarpStreams warp_streams(int m) {
 // Words of the state that a transform reads: the maps that take the coordinate as x 2^64
 // read the top word, the others round both to u.
 template <int TK>
-constexpr bool kTopWordOnly = TK == kTKorobovInt;
-template <int TK>
-constexpr int kWords = kTopWordOnly<TK> ? 1 : 2;
+constexpr bool kTopWordOnly = kIntKorobov<TK>;
 
 // The step constants of the d coordinates in shared memory (a warp's lanes read different j).
 // z2: the third fraction word for n < 2^32 (ShortState), else the exact remainder.
@@ -116,10 +114,12 @@ struct BlockSteps {
     }
 };
 
-// The published state of one warp: [buffer][word][pair].
+// The published state of one warp: [buffer][][pair], the top words of two points or the words
+// of one.
 template <int TK>
 struct WarpLattice {
-    uint64_t w[2][kWords<TK>][kPairs];
+    static constexpr int kWords = kTopWordOnly<TK> ? 1 : 2;
+    uint64_t w[2][2][kPairs];
 };
 
 // A point's coordinates as eval_point reads them: from the warp's buffer or a thread's own.
@@ -143,40 +143,53 @@ struct Shifts {
     __device__ __forceinline__ uint64_t operator()(int j) const { return s[j * m]; }
 };
 
+// The separable families' evaluation of NP points entirely in fixed point, coordinate and
+// integrand form (no fit: the fit map needs x as a double).  Points share the loads of the
+// shift and of the dimension's constants and the loop around them, and their integer chains
+// interleave (FIGURE_NP).
+template <int FAM, int TK, int R, int NP, class St>
+__device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableShared &fsh, Shifts dsh,
+                                           double cd, const St (&st)[NP], double (&g)[NP]) {
+    // the final function (exp, power, cos) on the integer pipe where the map leaves it room;
+    // under the higher Korobov orders the integer multiply pipe is the bottleneck and the FP64
+    // form, on the otherwise idle FP64 pipe, is faster (the crossover order per family was
+    // measured)
+    constexpr bool kIntFinish = !kIntKorobov<TK> ||
+                                (TK == kTKorobovInt && R <= FamilyAcc<FAM>::kIntFinishMaxR);
+    Weight W[NP];
+    FamilyAcc<FAM> fa[NP];
+#pragma unroll
+    for (int u = 0; u < NP; ++u) fa[u].init_fixed();
+#pragma unroll 1
+    for (int j = 0; j < p.d; ++j) {
+        const uint64_t D = dsh(j);
+#pragma unroll
+        for (int u = 0; u < NP; ++u)
+            fa[u].template add_fixed<kIntFinish>(j, transform_fixed<TK, R>(st[u].hi(j) + D, p.t, W[u]), fsh);
+    }
+#pragma unroll
+    for (int u = 0; u < NP; ++u) {
+        const double wt = weight_finish<TK, R>(W[u], p.t, cd);
+        fa[u].template finish_fixed<kIntFinish>(p.d, fsh, g[u]);
+        g[u] *= wt;
+    }
+}
+
 // One evaluation of g at a point with lattice state `st`.
 template <int FAM, int TK, int R, class St>
 __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared<FAM> &fsh,
                                            const double *s_fit, bool use_fit, Shifts dsh, double cd,
                                            const St &st, double &g_re, double &g_im,
                                            unsigned long long &signfail) {
-    Weight W{1.0, 1.0, 1.0, Fx{0x8000000000000000ull, 1}};
+    Weight W;
     FamilyAcc<FAM> fa;
-    if constexpr (kFixedTransform<TK> && kHasFixedForm<FAM>) {
-        // coordinate and integrand form entirely in fixed point (no fit: the fit map
-        // needs x as a double)
-        if (!use_fit && fsh.fx.ok) {
-            // the final function (exp, power, cos) on the integer pipe where the map leaves
-            // it room; under the higher Korobov orders the integer multiply pipe is the
-            // bottleneck and the FP64 form, on the otherwise idle FP64 pipe, is faster (the
-            // crossover order per family was measured)
-            constexpr bool kIntFinish = TK != kTKorobovInt || R <= FamilyAcc<FAM>::kIntFinishMaxR;
-            fa.init_fixed();
-#pragma unroll 1
-            for (int j = 0; j < p.d; ++j)
-                fa.template add_fixed<kIntFinish>(j, transform_fixed<TK, R>(st.hi(j) + dsh(j), W), fsh);
-            const double wt = weight_finish<TK, R>(W, p.t, cd);
-            fa.template finish_fixed<kIntFinish>(p.d, fsh, g_re, g_im, signfail);
-            g_re *= wt;
-            return;
-        }
-    }
     if constexpr (kFixedTransform<TK> && FAM == QMC_SECTOR) {
         // the real family with F in fixed point takes the coordinates as x 2^64 from the
         // integer-pipe transform (no fit map)
         if (!use_fit && sector_fixed_ok(fsh.poly, p.d)) {
             uint64_t X[8];
 #pragma unroll 1
-            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), W);
+            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), p.t, W);
             const double wt = weight_finish<TK, R>(W, p.t, cd);
             g_re = sector_value_x(X, p.d, fsh.poly) * wt;
             g_im = 0.0;
@@ -188,7 +201,7 @@ __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared
         if (!use_fit && feyn_fixed_ok(fsh.poly, p.d)) {
             uint64_t X[kFeynFixedMaxDim];
 #pragma unroll 1
-            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), W);
+            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), p.t, W);
             const double wt = weight_finish<TK, R>(W, p.t, cd);
             feynman_value_x(X, p.d, fsh.poly, g_re, g_im, signfail);
             g_re *= wt;
@@ -200,12 +213,12 @@ __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared
 #pragma unroll 1
     for (int j = 0; j < p.d; ++j) {
         Mapped mx;
-        if constexpr (TK == kTKorobovInt && kPolyFamily<FAM>) {
+        if constexpr (kIntKorobov<TK> && kPolyFamily<FAM>) {
             // the polynomial families use x itself: formed from x 2^64 by integer
             // operations instead of an FP64 conversion and reflection
-            mx = Mapped{fixed_u64_to_double(transform_fixed<TK, R>(st.hi(j) + dsh(j), W), 64), false};
-        } else if constexpr (TK == kTKorobovInt) {
-            mx = korobov_int_x<R>(st.hi(j) + dsh(j), W);
+            mx = Mapped{fixed_u64_to_double(transform_fixed<TK, R>(st.hi(j) + dsh(j), p.t, W), 64), false};
+        } else if constexpr (kIntKorobov<TK>) {
+            mx = korobov_int_x<TK, R>(st.hi(j) + dsh(j), p.t, W);
         } else {
             const double u = fixed_to_double(st.hi(j) + dsh(j), st.lo(j), p.n);
             mx = apply_transform<TK>(u, p.t, W);
@@ -242,17 +255,14 @@ struct StreamSum {
 };
 
 // The sums of one tile: this thread's stream covers points [i0, i0 + cnt) of the lattice,
-// i0 = w0 + mine * L with w0 the first point of the warp's first stream.
-template <int FAM, int TK, int R>
-__device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilyShared<FAM> &fsh,
-                                              const double *s_fit, bool use_fit, Shifts dsh,
-                                              const BlockSteps &steps, const WarpStreams &ws,
-                                              WarpLattice<TK> &lat, uint64_t w0,
-                                              uint32_t cnt, StreamSum &acc) {
-    constexpr bool kCplx = FamilyAcc<FAM>::kComplex;
+// i0 = w0 + mine * L with w0 the first point of the warp's first stream.  eval(states, g_re,
+// g_im, signfail) takes NP points at a time (one with a thread's own state).
+template <bool CPLX, int NP, class Lat, class Eval>
+__device__ __forceinline__ void run_stream(const Integral &p, const BlockSteps &steps,
+                                           const WarpStreams &ws, Lat &lat, uint64_t w0, uint32_t cnt,
+                                           StreamSum &acc, Eval &&eval) {
     const int d = p.d;
     const uint64_t n = p.n;
-    const double cd = p.cd;
     const int stride = d | 1;   // pairs of a stream in the buffer: odd, no bank conflicts
     const int pairs = ws.count * d;
     const int lanes = __popc(ws.mask);   // 32 but in a ragged last warp
@@ -276,24 +286,32 @@ __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilySha
         start(b, lane + lanes);
         const uint32_t most = __reduce_max_sync(ws.mask, cnt);
 #pragma unroll 1
-        for (uint32_t t = 0; t < most; ++t) {
-            auto &buf = lat.w[t & 1];
+        for (uint32_t t = 0; t < most; t += NP) {
+            auto &buf = lat.w[(t / NP) & 1];
             auto publish = [&](Pair &s) {
                 if (!s.own) return;
-                buf[0][s.at] = s.f.f_hi;
-                if constexpr (!kTopWordOnly<TK>) buf[1][s.at] = s.f.f_lo;
-                steps.step(s.j, n, s.f);
+#pragma unroll
+                for (int u = 0; u < NP; ++u) {
+                    buf[u][s.at] = s.f.f_hi;
+                    if constexpr (NP == 1 && Lat::kWords == 2) buf[1][s.at] = s.f.f_lo;
+                    steps.step(s.j, n, s.f);
+                }
             };
             publish(a);
             if (pairs > lanes) publish(b);
             __syncwarp(ws.mask);
             if (t < cnt) {
-                double g_re, g_im = 0.0;
-                eval_point<FAM, TK, R>(p, fsh, s_fit, use_fit, dsh, cd,
-                                       SharedState{&buf[0][ws.mine * stride]}, g_re, g_im, acc.signfail);
-                acc.template add<kCplx>(g_re, g_im);
+                double g_re[NP], g_im[NP];
+                SharedState st[NP];
+#pragma unroll
+                for (int u = 0; u < NP; ++u) st[u].w = &buf[u][ws.mine * stride];
+                eval(st, g_re, g_im, acc.signfail);
+                acc.template add<CPLX>(g_re[0], g_im[0]);
+#pragma unroll
+                for (int u = 1; u < NP; ++u)
+                    if (t + u < cnt) acc.template add<CPLX>(g_re[u], g_im[u]);
             }
-            if ((t & (kInner - 1)) == kInner - 1) acc.template flush<kCplx>();
+            if (((t + NP - 1) & (kInner - 1)) == kInner - 1) acc.template flush<CPLX>();
         }
     } else {
         uint64_t fhi[kMaxDim], flo[kMaxDim], f2[kMaxDim];
@@ -308,11 +326,11 @@ __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilySha
         }
 #pragma unroll 1
         for (uint32_t t = 0; t < cnt; ++t) {
-            double g_re, g_im = 0.0;
-            eval_point<FAM, TK, R>(p, fsh, s_fit, use_fit, dsh, cd, OwnState{fhi, flo}, g_re, g_im,
-                                   acc.signfail);
-            acc.template add<kCplx>(g_re, g_im);
-            if ((t & (kInner - 1)) == kInner - 1) acc.template flush<kCplx>();
+            double g_re[1], g_im[1];
+            const OwnState st[1] = {{fhi, flo}};
+            eval(st, g_re, g_im, acc.signfail);
+            acc.template add<CPLX>(g_re[0], g_im[0]);
+            if ((t & (kInner - 1)) == kInner - 1) acc.template flush<CPLX>();
 #pragma unroll 1
             for (int j = 0; j < d; ++j) {
                 ShortState s{fhi[j], flo[j], f2[j]};
@@ -323,7 +341,32 @@ __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilySha
             }
         }
     }
-    acc.template flush<kCplx>();
+    acc.template flush<CPLX>();
+}
+
+template <int FAM, int TK, int R>
+__device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilyShared<FAM> &fsh,
+                                              const double *s_fit, bool use_fit, Shifts dsh,
+                                              const BlockSteps &steps, const WarpStreams &ws,
+                                              WarpLattice<TK> &lat, uint64_t w0, uint32_t cnt,
+                                              StreamSum &acc) {
+    constexpr bool kCplx = FamilyAcc<FAM>::kComplex;
+    const double cd = p.cd;
+    if constexpr (kFixedTransform<TK> && kHasFixedForm<FAM>) {
+        if (!use_fit && fsh.fx.ok) {   // uniform over the block
+            run_stream<false, 1>(p, steps, ws, lat, w0, cnt, acc,
+                                 [&](auto &st, auto &g_re, auto &, unsigned long long &) {
+                                     eval_fixed<FAM, TK, R>(p, fsh, dsh, cd, st, g_re);
+                                 });
+            return;
+        }
+    }
+    run_stream<kCplx, 1>(p, steps, ws, lat, w0, cnt, acc,
+                         [&](auto &st, auto &g_re, auto &g_im, unsigned long long &signfail) {
+                             g_im[0] = 0.0;
+                             eval_point<FAM, TK, R>(p, fsh, s_fit, use_fit, dsh, cd, st[0], g_re[0],
+                                                    g_im[0], signfail);
+                         });
 }
 
 // The integer Korobov is compiled once per order r (uniform branch per tile).

@@ -1,5 +1,5 @@
 // qmc_sums_inst.cuh -- per-translation-unit instantiation of lattice_kernel over the
-// transforms (the four public kinds and the integer-pipe Korobov) for a list of families
+// transforms (the four public kinds and the two integer-pipe Korobov kinds) for a list of families
 // (split across TUs so nvcc compiles them in parallel).
 #pragma once
 #include "qmc_internal.h"
@@ -23,6 +23,7 @@ static cudaError_t launch_family(int tkind, const LatticeLaunch &lp, int max_d, 
     case QMC_T_KOROBOV: return launch_one<FAM, QMC_T_KOROBOV>(lp, max_d, s);
     case QMC_T_SIDI: return launch_one<FAM, QMC_T_SIDI>(lp, max_d, s);
     case kTKorobovInt: return launch_one<FAM, kTKorobovInt>(lp, max_d, s);
+    case kTKorobovGen: return launch_one<FAM, kTKorobovGen>(lp, max_d, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -28,10 +28,11 @@ namespace qmc {
 //    t_j = v_j (1 - v_j) (one fused multiply-add) and raised to r once per evaluation.
 //  * Korobov<r0,r1>: prod u_j and prod (1 - u_j), raised to r0 and r1 once.
 //  * w: other factors (fit Jacobian, Sidi weights).
-//  * wp: integer-pipe Korobov<r,r>, prod_j t_j as a normalized Fx.
+//  * wp: integer-pipe Korobov<r,r>, prod_j t_j as a normalized Fx; of the asymmetric map, wp
+//    and wq hold prod u_j and prod (1 - u_j).
 struct Weight {
-    double wu, w1, w;
-    Fx wp;
+    double wu = 1.0, w1 = 1.0, w = 1.0;
+    Fx wp{0x8000000000000000ull, 1}, wq{0x8000000000000000ull, 1};
 };
 
 struct Mapped {
@@ -66,7 +67,7 @@ __device__ __forceinline__ Mapped apply_transform(double u, const TransformParam
         }
         return {y, !lo};
     } else {
-        static_assert(TK == QMC_T_SIDI, "kTKorobovInt is evaluated by korobov_int_x");
+        static_assert(TK == QMC_T_SIDI, "the integer Korobov maps are evaluated by korobov_int_x");
         // phi = cr I_r(u), I_r = base I_(r mod 2) - (cos(pi u)/pi) sum_q a_q sin^(r-1-2q)
         double s, c;
         sincospi(u, &s, &c);
@@ -88,27 +89,33 @@ __device__ __forceinline__ Mapped apply_transform(double u, const TransformParam
     }
 }
 
-// The integer-pipe Korobov<R,R> (kTKorobovInt) takes the lattice state's top word
-// X = x 2^64 instead of the rounded u: v = min(x, 1 - x) in 0.64 fixed point.
-template <int R>
-__device__ __forceinline__ Mapped korobov_int_x(uint64_t X, Weight &W) {
+// The integer-pipe Korobov maps take the lattice state's top word X = x 2^64 instead of the
+// rounded u: v = min(x, 1 - x) in 0.64 fixed point.
+template <int TK, int R>
+__device__ __forceinline__ Mapped korobov_int_x(uint64_t X, const TransformParams &t, Weight &W) {
     const bool lo = !(X >> 63);
-    return {fixed_to_double64(korobov_phi_fixed<R>(lo ? X : ~X, W.wp)), !lo};
+    if constexpr (TK == kTKorobovGen) return {fixed_to_double64(korobov_gen_phi(X, t, W.wp, W.wq)), !lo};
+    else return {fixed_to_double64(korobov_phi_fixed<R>(lo ? X : ~X, W.wp)), !lo};
 }
 
 // Transforms that are exact or fixed-point on the integer pipe can hand the integrand the
 // coordinate itself in 0.64 fixed point, x 2^64 (truncated), when the integrand takes it
 // (FamilyAcc::add_fixed): none (x is the shifted lattice fraction), baker (2 min(x, 1 - x))
-// and the integer Korobov (phi, or 1 - phi when reflected).
+// and the integer Korobov maps (phi, or 1 - phi when reflected).
 template <int TK>
-constexpr bool kFixedTransform = TK == QMC_T_NONE || TK == QMC_T_BAKER || TK == kTKorobovInt;
+constexpr bool kIntKorobov = TK == kTKorobovInt || TK == kTKorobovGen;
+template <int TK>
+constexpr bool kFixedTransform = TK == QMC_T_NONE || TK == QMC_T_BAKER || kIntKorobov<TK>;
 
 template <int TK, int R>
-__device__ __forceinline__ uint64_t transform_fixed(uint64_t X, Weight &W) {
+__device__ __forceinline__ uint64_t transform_fixed(uint64_t X, const TransformParams &t, Weight &W) {
     if constexpr (TK == QMC_T_NONE) {
         return X;
     } else if constexpr (TK == QMC_T_BAKER) {
         return ((X >> 63) ? ~X : X) << 1;   // min(X, 2^64 - 1 - X) < 2^63
+    } else if constexpr (TK == kTKorobovGen) {
+        const uint64_t F = korobov_gen_phi(X, t, W.wp, W.wq);
+        return X >> 63 ? ~F : F;
     } else {
         static_assert(TK == kTKorobovInt, "no fixed-point form");
         const bool lo = !(X >> 63);
@@ -126,6 +133,8 @@ __device__ __forceinline__ double weight_finish(const Weight &W, const Transform
         return cd * ipow_u(W.wu, t.r0) * ipow_u(W.w1, t.r1) * W.w;
     } else if constexpr (TK == kTKorobovInt) {
         return korobov_weight_fixed<R>(W.wp, fx_of_double(cd)) * W.w;
+    } else if constexpr (TK == kTKorobovGen) {
+        return korobov_gen_weight(W.wp, W.wq, t, fx_of_double(cd)) * W.w;
     } else {
         return W.w;
     }
