@@ -146,7 +146,9 @@ struct Shifts {
 // The separable families' evaluation of NP points entirely in fixed point, coordinate and
 // integrand form (no fit: the fit map needs x as a double).  Points share the loads of the
 // shift and of the dimension's constants and the loop around them, and their integer chains
-// interleave (FIGURE_NP).
+// interleave : osc d = 6 baker at n = 1,072,187, m = 32
+// 520 -> 445 us, Gaussian d = 10 Korobov-3 at n = 10,560,653 16.29 -> 15.32 ms (two points;
+// 48 registers and five blocks beat 64 and four).
 template <int FAM, int TK, int R, int NP, class St>
 __device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableShared &fsh, Shifts dsh,
                                            double cd, const St (&st)[NP], double (&g)[NP]) {
@@ -354,7 +356,7 @@ __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilySha
     const double cd = p.cd;
     if constexpr (kFixedTransform<TK> && kHasFixedForm<FAM>) {
         if (!use_fit && fsh.fx.ok) {   // uniform over the block
-            run_stream<false, 1>(p, steps, ws, lat, w0, cnt, acc,
+            run_stream<false, 2>(p, steps, ws, lat, w0, cnt, acc,
                                  [&](auto &st, auto &g_re, auto &, unsigned long long &) {
                                      eval_fixed<FAM, TK, R>(p, fsh, dsh, cd, st, g_re);
                                  });
