@@ -263,8 +263,9 @@ int qmc_evaluate(const qmc_integrand *f, uint64_t n, const uint64_t *z, int dim,
     return cuda_status(launch_evaluate(f->family, p, out, (cudaStream_t)stream));
 }
 
-static uint32_t hist_blocks(uint64_t n) {
-    uint64_t b = (n + 4095) / 4096;
+// Blocks of the histogram pass: ~512 points each.
+static uint32_t hist_blocks(uint64_t n, uint64_t points = 512) {
+    uint64_t b = (n + points - 1) / points;
     return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(b, 1024));
 }
 
@@ -284,8 +285,10 @@ int qmc_histogram(const qmc_integrand *f, uint64_t n, const uint64_t *z, int dim
     if (bins < 1 || (size_t)dim * bins > 20480) return QMC_ERR_RANGE;
     for (int j = 0; j < dim; ++j)
         if (z[j] % n == 0 || gcd_u64(z[j] % n, n) != 1) return QMC_ERR_GENVEC;
-    uint32_t nb = hist_blocks(n);
-    if (workspace_bytes < (size_t)nb * dim * bins * sizeof(double)) return QMC_ERR_WORKSPACE;
+    // a smaller workspace, down to one block per 4096 points, takes fewer and longer blocks
+    const size_t per_block = (size_t)dim * bins * sizeof(double);
+    if (workspace_bytes < hist_blocks(n, 4096) * per_block) return QMC_ERR_WORKSPACE;
+    const uint32_t nb = (uint32_t)std::min<uint64_t>(hist_blocks(n), workspace_bytes / per_block);
     if ((st = device_ok())) return st;
     Integral p;
     std::memset(&p, 0, sizeof(p));
