@@ -36,8 +36,11 @@ constexpr int kDenseCap = 1024;   // >= C(16 + 3, 3) = 969 coefficients of a den
 //    multivariate Horner scheme, duplicates of the input list merged in input order.
 // Dense costs C(d+D, D) + ... fused multiply-adds independent of the number of input
 // monomials; it is chosen when that is cheaper than the sparse loop.
+constexpr int kSumLanes = 16;   // partial sums of a coefficient list (a fixed order for any block)
+
 struct PolyShared {
     int nu, nf, d;
+    double part[2][kSumLanes];
     int dense_u, dense_f;   // 0: sparse; 2 or 3: dense degree
     double pa, pb, lam;
     union {                          // U owns [0, 1024), F owns [1024, 2048), either form:
@@ -56,6 +59,8 @@ struct PolyShared {
     // whose error bound passes (stage_poly): the dense coefficients in place as
     // round(c 2^sfix) (unsigned), evaluated by dense_eval_fixed
     int fixed_f, sfix;
+    // the dense U in the same form, where F is (stage_poly), at u[kMaxTerms + e]
+    int fixed_u, sfix_u;
     // a = 1 and b = n + 1/2 (0 <= n <= 15): n, so that U^a F^-b = U / (F^n sqrt F) needs no
     // per-evaluation tests of the exponents; -1 otherwise
     int pow_half;
@@ -205,6 +210,22 @@ __device__ __forceinline__ bool feyn_tensor_cheaper(const PolyShared &ps, const 
     return dense < sparse;
 }
 
+// Partial sum l of a list of non-negative coefficients; -infinity when one is negative (NaN).
+__device__ __forceinline__ double sum_nonneg(const double *c, int n, int l) {
+    double s = 0.0;
+    for (int e = l; e < n; e += kSumLanes) s += c[e] >= 0.0 ? c[e] : -INFINITY;
+    return s;
+}
+
+// What the products of dense_eval_fixed truncate on average, in units of 2^-s, as added to the
+// constant term: a high product is 1.25 units low on average (mulhi_trunc: half a unit for
+// each cross product's dropped low half and a quarter for the low product), the loss of an
+// inner one is scaled by the coordinates (1/2 on average) that multiply it further out.
+__device__ __forceinline__ uint64_t dense_truncation(int d, int D) {
+    const double n1 = d, n2 = d * (d + 1) / 2, n3 = d * (d + 1) * (d + 2) / 6;
+    return (uint64_t)(1.25 * (n1 + 0.5 * n2 + (D == 3 ? 0.25 * n3 : 0.0)));
+}
+
 // allow_dense: the real sector family evaluates through the dense Horner form when
 // cheaper; the complex deformed family uses the symmetric-tensor form when cheaper.
 template <class P>
@@ -222,6 +243,7 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
         ps.maxdeg_f = 0;
         ps.feyn_fixed = 0;
         ps.fixed_f = 0;
+        ps.fixed_u = 0;
         const double tb = 2.0 * p.pb;
         ps.pow_half = (p.pa == 1.0 && tb >= 1.0 && tb <= 31.0 && tb == floor(tb) &&
                        ((int)tb & 1)) ? (int)tb / 2 : -1;
@@ -338,26 +360,46 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
         // cube; s = 62 - ilogb(B) keeps every partial sum below 2^63 with 2^-s <= 2^-62 B,
         // and N products at under 4.5 units of 2^-s each (dense_eval_fixed) give a
         // relative error below 4.5 N (B / c0) 2^-62, required <= 2^-42.
+        // Then U too, when a = 1 with b = n + 1/2 and its dense coefficients are non-negative.
+        // Its error is absolute, below 4.5 N 2^-62 of its coefficients' sum (measured: a
+        // tenth of that), where FP64's is relative; U enters the integrand as a factor, so
+        // what counts is that error against the mean of U where F^-b is large, and F's own
+        // bound (B / c0 times as much) is the larger one wherever that is.
+        __syncthreads();
+        const double *cf = ps.buf.v + 2 * kMaxTerms;
+        for (int l = tid; l < kSumLanes; l += blockDim.x) {
+            ps.part[0][l] = sum_nonneg(cf, n3, l);
+            ps.part[1][l] = use_u ? sum_nonneg(ps.buf.v, dense_size(V, use_u), l) : -INFINITY;
+        }
         __syncthreads();
         if (tid == 0) {
-            const double *c = ps.buf.v + 2 * kMaxTerms;
-            double B = 0.0;
-            int ok = 1;
-            for (int e = 0; e < n3; ++e) {
-                ok = ok && c[e] >= 0.0;
-                B += c[e];
+            double B = 0.0, Bu = 0.0;
+            for (int l = 0; l < kSumLanes; ++l) {
+                B += ps.part[0][l];
+                Bu += ps.part[1][l];
             }
-            const double c0 = c[n3 - 1];   // x_d^D: the constant term
+            const double c0 = cf[n3 - 1];   // x_d^D: the constant term
             const int N = n3 + (use_f == 3 ? dense_size(V, 2) : 0) + V;
-            ok = ok && c0 > 0.0 && B < 1e300 && 4.5 * N * B <= 0x1p20 * c0;
+            const int ok = B >= 0.0 && c0 > 0.0 && B < 1e300 && 4.5 * N * B <= 0x1p20 * c0;
+            const int ok_u = ok && ps.pow_half >= 0 && Bu > 0x1p-900 && Bu < 1e300 &&
+                             dense_size(V, use_u) <= kMaxTerms;
             ps.fixed_f = ok;
             ps.sfix = ok ? 62 - ilogb(B) : 0;
+            ps.fixed_u = ok_u;
+            ps.sfix_u = ok_u ? 62 - ilogb(Bu) : 0;
         }
         __syncthreads();
         if (ps.fixed_f)
             for (int e = tid; e < n3; e += blockDim.x)
                 ps.buf.u[2 * kMaxTerms + e] =
-                    (uint64_t)llrint(ldexp(ps.buf.v[2 * kMaxTerms + e], ps.sfix));
+                    (uint64_t)llrint(ldexp(ps.buf.v[2 * kMaxTerms + e], ps.sfix)) +
+                    (e == n3 - 1 ? dense_truncation(d, use_f) : 0);
+        if (ps.fixed_u) {
+            const int n2 = dense_size(V, use_u);
+            for (int e = tid; e < n2; e += blockDim.x)
+                ps.buf.u[kMaxTerms + e] = (uint64_t)llrint(ldexp(ps.buf.v[e], ps.sfix_u)) +
+                                          (e == n2 - 1 ? dense_truncation(d, use_u) : 0);
+        }
     } else {
         for (int q = tid; q < p.nf; q += blockDim.x) {
             ps.buf.v[2 * kMaxTerms + q] = p.fcoef[q];
@@ -552,43 +594,32 @@ __device__ __forceinline__ double sector_power(double U, double F, const PolySha
 }
 
 // The real family with F in fixed point, both forms dense and d compiled in (d = 3..8):
-// the coordinates and the unrolled loops stay in registers.  x (doubles, for U) and X
-// (x 2^64, for F) hold the same point.
+// the coordinates, X = x 2^64, and the unrolled loops stay in registers; U in fixed point
+// with F, else in FP64 at x formed from X by integer operations (truncated).
+// With U in FP64 (its 45 + 9 fused multiply-adds at d = 8 and the power) the FP64 pipe was
+// 70 % busy and the multiply pipe 51 %: n = 1,072,187, m = 32 took 5.88 ms, with U here 4.50.
 template <int D>
-__device__ __forceinline__ double sector_fixed_core(const double *x, const uint64_t *X,
-                                                    const PolyShared &ps) {
+static __device__ __noinline__ double sector_value_fixed_x(const uint64_t *Xin, const PolyShared &ps) {
+    uint64_t X[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) X[k] = Xin[k];
     constexpr int V = D + 1;
-    const double U = ps.dense_u == 3 ? dense_eval_t<V, 3>(x, ps.buf.v) : dense_eval_t<V, 2>(x, ps.buf.v);
+    double U;
+    if (ps.fixed_u) {
+        const uint64_t *Cu = ps.buf.u + kMaxTerms;
+        const uint64_t Uq = ps.dense_u == 3 ? dense_eval_fixed<V>(X, V, 3, Cu) : dense_eval_fixed<V>(X, V, 2, Cu);
+        U = fixed_u64_to_double(Uq, ps.sfix_u);
+    } else {
+        double x[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) x[k] = fixed_u64_to_double(X[k], 64);
+        U = ps.dense_u == 3 ? dense_eval_t<V, 3>(x, ps.buf.v) : dense_eval_t<V, 2>(x, ps.buf.v);
+    }
     const uint64_t *C = ps.buf.u + 2 * kMaxTerms;
     const uint64_t Fq = ps.dense_f == 3 ? dense_eval_fixed<V>(X, V, 3, C) : dense_eval_fixed<V>(X, V, 2, C);
     return sector_power(U, fixed_u64_to_double(Fq, ps.sfix), ps);   // F >= c0 > 0
 }
-template <int D>
-static __device__ __noinline__ double sector_value_fixed(const double *xin, const PolyShared &ps) {
-    double x[D];
-    uint64_t X[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-        x[k] = xin[k];
-        X[k] = unit_to_fixed64(x[k]);
-    }
-    return sector_fixed_core<D>(x, X, ps);
-}
-// The same from the coordinates in 0.64 fixed point (the integer-pipe transforms), x
-// from X by integer operations (truncated).
-template <int D>
-static __device__ __noinline__ double sector_value_fixed_x(const uint64_t *Xin, const PolyShared &ps) {
-    double x[D];
-    uint64_t X[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-        X[k] = Xin[k];
-        x[k] = fixed_u64_to_double(X[k], 64);
-    }
-    return sector_fixed_core<D>(x, X, ps);
-}
-
-// Whether sector_value_fixed(_x) serves this integrand (uniform over the block).
+// Whether sector_value_fixed_x serves this integrand (uniform over the block).
 __device__ __forceinline__ bool sector_fixed_ok(const PolyShared &ps, int d) {
     return ps.fixed_f && ps.dense_u && d >= 3 && d <= 8;
 }
@@ -605,26 +636,24 @@ __device__ __forceinline__ double sector_value_x(const uint64_t *X, int d, const
 }
 
 __device__ __forceinline__ double sector_value(const double *xin, int d, const PolyShared &ps) {
+    // a fit map that is not monotone leaves the cube: U in fixed point does not follow it there
+    bool inside = true;
+#pragma unroll 1
+    for (int k = 0; k < d; ++k)
+        inside &= (unsigned long long)__double_as_longlong(xin[k]) <= 0x3FF0000000000000ull;
     if (sector_fixed_ok(ps, d)) {
-        switch (d) {
-        case 3: return sector_value_fixed<3>(xin, ps);
-        case 4: return sector_value_fixed<4>(xin, ps);
-        case 5: return sector_value_fixed<5>(xin, ps);
-        case 6: return sector_value_fixed<6>(xin, ps);
-        case 7: return sector_value_fixed<7>(xin, ps);
-        case 8: return sector_value_fixed<8>(xin, ps);
-        default: break;
-        }
+        uint64_t X[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) X[k] = k < d ? unit_to_fixed64(xin[k]) : 0;
+        if (inside) return sector_value_x(X, d, ps);
     }
     double x[kMaxDim + 1];
 #pragma unroll 1
     for (int k = 0; k < d; ++k) x[k] = xin[k];
     x[d] = 1.0;
-    const double U = ps.dense_u ? dense_eval(x, d + 1, ps.dense_u, ps.buf.v)
-                                : poly_real(x, ps.nu, ps.buf.v, ps.buf.u + kMaxTerms);
-    double F;
+    double U, F;
+    uint64_t X[kMaxDim];
     if (ps.fixed_f) {
-        uint64_t X[kMaxDim];
 #pragma unroll 1
         for (int k = 0; k < d; ++k) X[k] = unit_to_fixed64(x[k]);
         F = fixed_u64_to_double(dense_eval_fixed<0>(X, d + 1, ps.dense_f, ps.buf.u + 2 * kMaxTerms),
@@ -633,6 +662,11 @@ __device__ __forceinline__ double sector_value(const double *xin, int d, const P
         F = ps.dense_f ? dense_eval(x, d + 1, ps.dense_f, ps.buf.v + 2 * kMaxTerms)
                        : poly_real(x, ps.nf, ps.buf.v + 2 * kMaxTerms, ps.buf.u + 3 * kMaxTerms);
     }
+    if (ps.fixed_u && inside)
+        U = fixed_u64_to_double(dense_eval_fixed<0>(X, d + 1, ps.dense_u, ps.buf.u + kMaxTerms), ps.sfix_u);
+    else
+        U = ps.dense_u ? dense_eval(x, d + 1, ps.dense_u, ps.buf.v)
+                       : poly_real(x, ps.nu, ps.buf.v, ps.buf.u + kMaxTerms);
     return sector_power(U, F, ps);
 }
 

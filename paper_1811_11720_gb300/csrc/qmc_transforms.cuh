@@ -147,10 +147,19 @@ __device__ __forceinline__ double weight_finish(const Weight &W, const Transform
 //   [9] 2 a5, [10] 3 a6 (the derivative's coefficients).
 constexpr int kFitStride = 11;
 
+// 1/a within one unit of 2^-53 for a normal a with a normal reciprocal: the hardware's ~20-bit
+// estimate and one cubic step, three FP64 instructions instead of a full division.
+__device__ __forceinline__ double recip_cubic(double a) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+    const double e = fma(-a, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 __device__ __forceinline__ double apply_fit(double x, const double *fp, double &jac) {
     const double d0 = fp[0] - x;
     const double d1 = fp[1] - x;
-    const double inv = 1.0 / (d0 * d1);
+    const double inv = recip_cubic(d0 * d1);
     const double r0 = d1 * inv;   // 1 / (a0 - x)
     const double r1 = d0 * inv;   // 1 / (a1 - x)
     const double poly = fma(fma(fp[6], x, fp[5]), x, fp[4]);
