@@ -26,9 +26,13 @@
 #include <cuda_runtime.h>
 #include <cufft.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <memory>
+#include <mutex>
+#include <new>
 #include <vector>
 
 #include "qmc_gb300.h"
@@ -43,26 +47,36 @@ constexpr int kCbcThreads = 256;
 
 __host__ __device__ inline double omega_k(double x) { return kTwoPi2 * (x * x - x + 1.0 / 6.0); }
 
-// a b mod n for a, b < n < 2^53: the quotient estimated in FP64 is within 2 of the exact
-// one, and the remainder is corrected exactly in 64-bit two's complement.
-__device__ __forceinline__ uint64_t mulmod_dev(uint64_t a, uint64_t b, uint64_t n) {
+// Arithmetic modulo n with what it needs precomputed: n < 2^32 takes the quotient from the
+// 64-bit reciprocal floor(2^64 / n) (at most 2 low), larger n < 2^53 an FP64 estimate (within 2
+// of the exact one); the remainder is then corrected exactly.
+struct Modulus {
+    uint64_t n, inv;   // inv = floor(2^64 / n) for n < 2^32, else 0
+};
+
+__device__ __forceinline__ uint64_t mulmod_dev(uint64_t a, uint64_t b, const Modulus &m) {
     const uint64_t lo = a * b;
-    const double qd = floor((double)a * (double)b / (double)n);
+    if (m.inv) {
+        uint64_t r = lo - __umul64hi(lo, m.inv) * m.n;
+        if (r >= 2 * m.n) r -= 2 * m.n;
+        return r >= m.n ? r - m.n : r;
+    }
+    const double qd = floor((double)a * (double)b / (double)m.n);
     const uint64_t q = qd <= 0.0 ? 0ull : (uint64_t)qd;
-    long long r = (long long)(lo - q * n);   // the exact a b - q n, within (-2n, 3n)
+    long long r = (long long)(lo - q * m.n);   // the exact a b - q n, within (-2n, 3n)
 #pragma unroll 1
-    for (int it = 0; it < 4 && r < 0; ++it) r += (long long)n;
+    for (int it = 0; it < 4 && r < 0; ++it) r += (long long)m.n;
 #pragma unroll 1
-    for (int it = 0; it < 4 && r >= (long long)n; ++it) r -= (long long)n;
+    for (int it = 0; it < 4 && r >= (long long)m.n; ++it) r -= (long long)m.n;
     return (uint64_t)r;
 }
 
-__device__ __forceinline__ uint64_t powmod_dev(uint64_t g, uint64_t e, uint64_t n) {
-    uint64_t r = 1 % n, b = g % n;
+__device__ __forceinline__ uint64_t powmod_dev(uint64_t g, uint64_t e, const Modulus &m) {
+    uint64_t r = 1 % m.n, b = g % m.n;
 #pragma unroll 1
     while (e) {
-        if (e & 1) r = mulmod_dev(r, b, n);
-        b = mulmod_dev(b, b, n);
+        if (e & 1) r = mulmod_dev(r, b, m);
+        b = mulmod_dev(b, b, m);
         e >>= 1;
     }
     return r;
@@ -136,16 +150,16 @@ uint64_t primitive_root(uint64_t n) {
 }
 
 // gp[c] = g^c mod n for c < H; thread t fills [t B, t B + B).
-__global__ void cbc_powers_kernel(uint64_t g, uint64_t n, uint64_t H, uint64_t B, uint64_t *gp) {
+__global__ void cbc_powers_kernel(uint64_t g, Modulus m, uint64_t H, uint64_t B, uint64_t *gp) {
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t c0 = t * B;
     if (c0 >= H) return;
-    uint64_t x = powmod_dev(g, c0, n);
+    uint64_t x = powmod_dev(g, c0, m);
     const uint64_t c1 = c0 + B < H ? c0 + B : H;
 #pragma unroll 1
     for (uint64_t c = c0; c < c1; ++c) {
         gp[c] = x;
-        x = mulmod_dev(x, g, n);
+        x = mulmod_dev(x, g, m);
     }
 }
 
@@ -162,14 +176,70 @@ __global__ void cbc_omega_kernel(const uint64_t *gp, uint64_t H, uint64_t L, uin
     }
 }
 
-// p[k] *= beta + gamma omega({k z / n}) for k <= H (p[k] = 1 first when init).
-__global__ void cbc_update_kernel(double *p, uint64_t H, uint64_t n, uint64_t z, double beta,
-                                  double gamma, int init) {
-    for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= H;
-         k += (uint64_t)gridDim.x * blockDim.x) {
-        const double f = fma(gamma, omega_k((double)mulmod_dev(k, z, n) / (double)n), beta);
-        p[k] = init ? f : p[k] * f;
+// Blocks of the block-wise reductions, and what one component leaves for the next.
+constexpr unsigned kCbcBlocks = 152 * 8;
+
+// The choice of the previous component from its blocks' picks: the smallest representative
+// (n when there is none) and its T.  Every thread returns the same.
+__device__ __forceinline__ uint64_t cbc_choice(const uint64_t *rep, const double *t, unsigned blocks,
+                                               uint64_t n, double *t_best) {
+    __shared__ uint64_t sr[kCbcThreads];
+    __shared__ double st[kCbcThreads];
+    uint64_t best = n;
+    double bt = 0.0;
+    for (unsigned b = threadIdx.x; b < blocks; b += kCbcThreads)
+        if (rep[b] < best) {
+            best = rep[b];
+            bt = t[b];
+        }
+    sr[threadIdx.x] = best;
+    st[threadIdx.x] = bt;
+    __syncthreads();
+    for (int w = kCbcThreads / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w && sr[threadIdx.x + w] < sr[threadIdx.x]) {
+            sr[threadIdx.x] = sr[threadIdx.x + w];
+            st[threadIdx.x] = st[threadIdx.x + w];
+        }
+        __syncthreads();
     }
+    *t_best = st[0];
+    return sr[0];
+}
+
+// Component j: z_1 = 1, later ones the choice of the previous picks.  p[k] *= beta + gamma
+// omega({k z / n}) for k <= H (p[k] = the factor for j = 0), and the block sums of p[1..H] (a
+// fixed order within a block; the host adds the blocks in order).  z, its T, p[0] and the
+// block sums of every component stay on the device until the last one.
+__global__ void __launch_bounds__(kCbcThreads)
+    cbc_update_kernel(double *p, uint64_t H, Modulus m, double beta, double gamma, int j,
+                      unsigned pick_blocks, const uint64_t *rep, const double *rep_t,
+                      uint64_t per_block, uint64_t *z_out, double *t_out, double *p0_out, double *sums) {
+    __shared__ double s[kCbcThreads];
+    uint64_t z = 1;
+    double tz = 0.0;
+    if (j) z = cbc_choice(rep, rep_t, pick_blocks, m.n, &tz);
+    auto update = [&](uint64_t k) {
+        const double f = fma(gamma, omega_k((double)mulmod_dev(k, z, m) / (double)m.n), beta);
+        const double v = j ? p[k] * f : f;
+        p[k] = v;
+        return v;
+    };
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        p0_out[j] = update(0);
+        z_out[j] = z;
+        t_out[j] = tz;
+    }
+    const uint64_t lo = 1 + (uint64_t)blockIdx.x * per_block;
+    const uint64_t hi = lo + per_block < H + 1 ? lo + per_block : H + 1;
+    double acc = 0.0;
+    for (uint64_t k = lo + threadIdx.x; k < hi; k += kCbcThreads) acc += update(k);
+    s[threadIdx.x] = acc;
+    __syncthreads();
+    for (int w = kCbcThreads / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) sums[(uint64_t)j * kCbcBlocks + blockIdx.x] = s[0];
 }
 
 // P[b] = p(min(g^-b, n - g^-b)) for b < H (g^-b = n - g^(H - b) for b >= 1, g^0 = 1), zero
@@ -200,30 +270,19 @@ __global__ void cbc_pointwise_kernel(cufftDoubleComplex *a, const cufftDoubleCom
     }
 }
 
-// Block sums of p[1..H] (fixed order within a block, blocks in order on the host).
-__global__ void cbc_sum_kernel(const double *p, uint64_t H, uint64_t per_block, double *out) {
-    __shared__ double s[kCbcThreads];
-    const uint64_t lo = 1 + (uint64_t)blockIdx.x * per_block;
-    const uint64_t hi = lo + per_block < H + 1 ? lo + per_block : H + 1;
-    double acc = 0.0;
-    for (uint64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) acc += p[k];
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = kCbcThreads / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[blockIdx.x] = s[0];
-}
+// T[a] = scale raw[a] + off, a < H, with off = p(0) omega(0) of the current p.
+__device__ __forceinline__ double cbc_offset(const double *p) { return __dmul_rn(p[0], omega_k(0.0)); }
 
-// Per-block minimum of T[a] = scale raw[a] + off over a < H.
-__global__ void cbc_min_kernel(const double *raw, uint64_t H, double scale, double off,
-                               uint64_t per_block, double *out) {
+// Per-block minimum of T.
+__global__ void __launch_bounds__(kCbcThreads)
+    cbc_min_kernel(const double *raw, const double *p, uint64_t H, double scale, uint64_t per_block,
+                   double *out) {
     __shared__ double s[kCbcThreads];
+    const double off = cbc_offset(p);
     const uint64_t lo = (uint64_t)blockIdx.x * per_block;
     const uint64_t hi = lo + per_block < H ? lo + per_block : H;
     double m = INFINITY;
-    for (uint64_t a = lo + threadIdx.x; a < hi; a += blockDim.x) m = fmin(m, fma(scale, raw[a], off));
+    for (uint64_t a = lo + threadIdx.x; a < hi; a += kCbcThreads) m = fmin(m, fma(scale, raw[a], off));
     s[threadIdx.x] = m;
     __syncthreads();
     for (int w = kCbcThreads / 2; w > 0; w >>= 1) {
@@ -233,18 +292,36 @@ __global__ void cbc_min_kernel(const double *raw, uint64_t H, double scale, doub
     if (threadIdx.x == 0) out[blockIdx.x] = s[0];
 }
 
-// Per block: the smallest representative min(g^a, n - g^a) among a with T[a] <= bound,
-// and its T (representative n when none).
-__global__ void cbc_pick_kernel(const double *raw, const uint64_t *gp, uint64_t H, uint64_t n,
-                                double scale, double off, double bound, uint64_t per_block,
-                                uint64_t *rep_out, double *t_out) {
+// Per block: the smallest representative min(g^a, n - g^a) among a with T[a] <= bound, and
+// its T (representative n when none).  The bound is the least of the blocks' minima plus the
+// tie tolerance of sum_k p(k) (psums: block sums of p[1..H]).
+__global__ void __launch_bounds__(kCbcThreads)
+    cbc_pick_kernel(const double *raw, const uint64_t *gp, const double *p, uint64_t H, uint64_t n,
+                    double scale, uint64_t per_block, const double *mins, unsigned min_blocks,
+                    const double *psums, uint64_t *rep_out, double *t_out) {
     __shared__ uint64_t sr[kCbcThreads];
-    __shared__ double st[kCbcThreads];
+    __shared__ double st[kCbcThreads], sm[kCbcThreads];
+    double least = INFINITY, sum = 0.0;
+    for (unsigned b = threadIdx.x; b < min_blocks; b += kCbcThreads) least = fmin(least, mins[b]);
+    for (unsigned b = threadIdx.x; b < kCbcBlocks; b += kCbcThreads) sum += psums[b];
+    sm[threadIdx.x] = least;
+    st[threadIdx.x] = sum;
+    __syncthreads();
+    for (int w = kCbcThreads / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) {
+            sm[threadIdx.x] = fmin(sm[threadIdx.x], sm[threadIdx.x + w]);
+            st[threadIdx.x] += st[threadIdx.x + w];
+        }
+        __syncthreads();
+    }
+    const double bound = sm[0] + kTieRtol * omega_k(0.0) * (p[0] + 2.0 * st[0]);
+    __syncthreads();
+    const double off = cbc_offset(p);
     const uint64_t lo = (uint64_t)blockIdx.x * per_block;
     const uint64_t hi = lo + per_block < H ? lo + per_block : H;
     uint64_t best = n;
     double bt = INFINITY;
-    for (uint64_t a = lo + threadIdx.x; a < hi; a += blockDim.x) {
+    for (uint64_t a = lo + threadIdx.x; a < hi; a += kCbcThreads) {
         const double t = fma(scale, raw[a], off);
         if (t <= bound) {
             const uint64_t v = gp[a];
@@ -271,29 +348,90 @@ __global__ void cbc_pick_kernel(const double *raw, const uint64_t *gp, uint64_t 
     }
 }
 
-struct DeviceBuffers {
-    std::vector<void *> ptrs;
-    ~DeviceBuffers() {
-        for (void *p : ptrs) cudaFree(p);
+// What a call needs besides its inputs: two cuFFT plans of length L, their shared work area
+// and one device buffer.  Making them costs more than a construction of a small size runs
+// for, so up to kKept of them, of at most kKeptBytes each, wait for the next call of the same
+// device and length; a call takes one out for itself (calls from several threads or streams
+// do not share any) and gives it back when its stream has drained.
+struct Workspace {
+    int device = -1;
+    uint64_t L = 0;
+    size_t bytes = 0, fft_bytes = 0;
+    cufftHandle fwd = 0, inv = 0;
+    bool have_fwd = false, have_inv = false;
+    char *base = nullptr;
+    Workspace() = default;
+    Workspace(const Workspace &) = delete;
+    Workspace &operator=(const Workspace &) = delete;
+    ~Workspace() {
+        if (have_fwd) cufftDestroy(fwd);
+        if (have_inv) cufftDestroy(inv);
+        if (base) cudaFree(base);
     }
-    template <class T>
-    bool alloc(T **p, size_t count) {
-        void *q = nullptr;
-        if (cudaMalloc(&q, count * sizeof(T)) != cudaSuccess) return false;
-        ptrs.push_back(q);
-        *p = static_cast<T *>(q);
-        return true;
+    // Plans without their own work areas, then one allocation of `need` bytes and the larger
+    // of the two areas behind it.
+    bool make(uint64_t length, size_t need) {
+        long long len = (long long)length;
+        size_t wf = 0, wi = 0;
+        if (cudaGetDevice(&device) != cudaSuccess) return false;
+        L = length;
+        if (cufftCreate(&fwd) != CUFFT_SUCCESS) return false;
+        have_fwd = true;
+        if (cufftCreate(&inv) != CUFFT_SUCCESS) return false;
+        have_inv = true;
+        if (cufftSetAutoAllocation(fwd, 0) != CUFFT_SUCCESS || cufftSetAutoAllocation(inv, 0) != CUFFT_SUCCESS ||
+            cufftMakePlanMany64(fwd, 1, &len, nullptr, 1, 0, nullptr, 1, 0, CUFFT_D2Z, 1, &wf) != CUFFT_SUCCESS ||
+            cufftMakePlanMany64(inv, 1, &len, nullptr, 1, 0, nullptr, 1, 0, CUFFT_Z2D, 1, &wi) != CUFFT_SUCCESS)
+            return false;
+        bytes = need;
+        fft_bytes = wf > wi ? wf : wi;
+        if (cudaMalloc(&base, bytes + fft_bytes + 256) != cudaSuccess) {
+            base = nullptr;
+            return false;
+        }
+        return cufftSetWorkArea(fwd, base + bytes) == CUFFT_SUCCESS &&
+               cufftSetWorkArea(inv, base + bytes) == CUFFT_SUCCESS;
     }
 };
 
-struct Plans {
-    cufftHandle fwd = 0, inv = 0;
-    bool have_fwd = false, have_inv = false;
-    ~Plans() {
-        if (have_fwd) cufftDestroy(fwd);
-        if (have_inv) cufftDestroy(inv);
+constexpr size_t kKept = 2;
+constexpr size_t kKeptBytes = (size_t)64 << 20;
+std::mutex g_kept_mutex;
+// never destroyed: at process exit the driver may be gone before static destructors run
+std::vector<std::unique_ptr<Workspace>> &kept() {
+    static auto *v = new std::vector<std::unique_ptr<Workspace>>;
+    return *v;
+}
+
+std::unique_ptr<Workspace> take_workspace(uint64_t L, size_t need) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_kept_mutex);
+        auto &v = kept();
+        for (size_t i = 0; i < v.size(); ++i)
+            if (v[i]->device == dev && v[i]->L == L && v[i]->bytes >= need) {
+                std::unique_ptr<Workspace> w = std::move(v[i]);
+                v.erase(v.begin() + i);
+                return w;
+            }
     }
-};
+    std::unique_ptr<Workspace> w(new (std::nothrow) Workspace);
+    if (w && !w->make(L, need)) w.reset();
+    return w;
+}
+
+void give_back(std::unique_ptr<Workspace> w) {
+    if (w->bytes + w->fft_bytes > kKeptBytes) return;
+    std::unique_ptr<Workspace> old;   // destroyed outside the lock
+    std::lock_guard<std::mutex> lock(g_kept_mutex);
+    auto &v = kept();
+    if (v.size() >= kKept) {
+        old = std::move(v.front());
+        v.erase(v.begin());
+    }
+    v.push_back(std::move(w));
+}
 
 // Smallest 2^a 3^b 5^c 7^d >= x.
 uint64_t smooth_at_least(uint64_t x) {
@@ -339,105 +477,74 @@ extern "C" int qmc_cbc_korobov(uint64_t n, int s, double gamma, double beta, uin
     const uint64_t g = primitive_root(n);
     if (!g) return QMC_ERR_ARG;
 
-    DeviceBuffers buf;
-    uint64_t *gp = nullptr;
-    double *p = nullptr, *P = nullptr, *part = nullptr, *tpart = nullptr;
-    uint64_t *rpart = nullptr;
-    cufftDoubleComplex *FP = nullptr, *FW = nullptr;
-    const unsigned nblk = 152 * 8;
-    if (!buf.alloc(&gp, H) || !buf.alloc(&p, H + 1) || !buf.alloc(&P, L) || !buf.alloc(&FP, nc) ||
-        !buf.alloc(&FW, nc) || !buf.alloc(&part, nblk) || !buf.alloc(&tpart, nblk) ||
-        !buf.alloc(&rpart, nblk))
+    // per-component results and the blocks' partials, then the large arrays
+    size_t bytes = 0;
+    auto take = [&](size_t count) {
+        const size_t at = bytes;
+        bytes += (count * 8 + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t o_z = take(s), o_t = take(s), o_p0 = take(s), o_sums = take((size_t)s * kCbcBlocks),
+                 host_bytes = bytes, o_mins = take(kCbcBlocks), o_rep = take(kCbcBlocks),
+                 o_rept = take(kCbcBlocks), o_gp = take(H), o_p = take(H + 1), o_P = take(L),
+                 o_FP = take(2 * nc), o_FW = take(2 * nc);
+    std::unique_ptr<Workspace> ws = take_workspace(L, bytes);
+    if (!ws || cufftSetStream(ws->fwd, st) != CUFFT_SUCCESS || cufftSetStream(ws->inv, st) != CUFFT_SUCCESS)
         return QMC_ERR_CUDA;
+    auto at = [&](size_t off) { return ws->base + off; };
+    uint64_t *z_d = (uint64_t *)at(o_z), *rep = (uint64_t *)at(o_rep), *gp = (uint64_t *)at(o_gp);
+    double *t_d = (double *)at(o_t), *p0_d = (double *)at(o_p0), *sums = (double *)at(o_sums);
+    double *mins = (double *)at(o_mins), *rep_t = (double *)at(o_rept), *p = (double *)at(o_p), *P = (double *)at(o_P);
+    cufftDoubleComplex *FP = (cufftDoubleComplex *)at(o_FP), *FW = (cufftDoubleComplex *)at(o_FW);
 
-    Plans plans;
-    long long len = (long long)L;
-    size_t work = 0;
-    if (cufftCreate(&plans.fwd) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
-    plans.have_fwd = true;
-    if (cufftCreate(&plans.inv) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
-    plans.have_inv = true;
-    if (cufftMakePlanMany64(plans.fwd, 1, &len, nullptr, 1, 0, nullptr, 1, 0, CUFFT_D2Z, 1, &work) !=
-            CUFFT_SUCCESS ||
-        cufftMakePlanMany64(plans.inv, 1, &len, nullptr, 1, 0, nullptr, 1, 0, CUFFT_Z2D, 1, &work) !=
-            CUFFT_SUCCESS ||
-        cufftSetStream(plans.fwd, st) != CUFFT_SUCCESS || cufftSetStream(plans.inv, st) != CUFFT_SUCCESS)
-        return QMC_ERR_CUDA;
-
-    // powers of g, the transformed omega sequence (P is scratch here)
-    const uint64_t B = 64;
+    // powers of g (threads of B powers each: enough threads for the chip first), the
+    // transformed omega sequence (P is scratch here)
+    const Modulus mod{n, n >> 32 ? 0 : ~0ull / n};   // floor((2^64 - 1) / n) = floor(2^64 / n), n odd
+    const uint64_t B = std::max<uint64_t>(1, std::min<uint64_t>(64, H / (152 * 2048)));
     const uint64_t nthr = (H + B - 1) / B;
-    cbc_powers_kernel<<<(unsigned)((nthr + kCbcThreads - 1) / kCbcThreads), kCbcThreads, 0, st>>>(g, n, H, B, gp);
+    cbc_powers_kernel<<<(unsigned)((nthr + kCbcThreads - 1) / kCbcThreads), kCbcThreads, 0, st>>>(g, mod, H, B, gp);
     cbc_omega_kernel<<<grid_for(L), kCbcThreads, 0, st>>>(gp, H, L, n, P);
     if (cudaGetLastError() != cudaSuccess) return QMC_ERR_CUDA;
-    if (cufftExecD2Z(plans.fwd, P, FW) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
+    if (cufftExecD2Z(ws->fwd, P, FW) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
 
-    // component 1: z_1 = 1
-    cbc_update_kernel<<<grid_for(H + 1), kCbcThreads, 0, st>>>(p, H, n, 1, beta, gamma, 1);
-    const uint64_t per_sum = (H + nblk - 1) / nblk;
-    const uint64_t per_min = (H + nblk - 1) / nblk;
-    std::vector<double> hpart(nblk), htp(nblk);
-    std::vector<uint64_t> hrp(nblk);
-
-    auto total = [&](double &tot) -> bool {
-        double p0 = 0.0;
-        cbc_sum_kernel<<<nblk, kCbcThreads, 0, st>>>(p, H, per_sum, part);
-        if (cudaMemcpyAsync(hpart.data(), part, nblk * sizeof(double), cudaMemcpyDeviceToHost, st) !=
-                cudaSuccess ||
-            cudaMemcpyAsync(&p0, p, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return false;
-        double acc = 0.0;
-        for (unsigned b = 0; b < nblk; ++b) acc += hpart[b];
-        tot = p0 + 2.0 * acc;
-        return true;
-    };
-    double tot = 0.0;
-    if (!total(tot)) return QMC_ERR_CUDA;
-    z_out[0] = 1;
-    if (e2_out) e2_out[0] = -1.0 + tot / (double)n;
-    const double w0 = omega_k(0.0);
-
-    for (int j = 1; j < s; ++j) {
-        double p0 = 0.0;
-        if (cudaMemcpyAsync(&p0, p, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-            return QMC_ERR_CUDA;
-        cbc_gather_kernel<<<grid_for(L), kCbcThreads, 0, st>>>(gp, p, H, L, n, P);
-        if (cufftExecD2Z(plans.fwd, P, FP) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
-        cbc_pointwise_kernel<<<grid_for(nc), kCbcThreads, 0, st>>>(FP, FW, nc);
-        if (cufftExecZ2D(plans.inv, FP, P) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
-        if (cudaStreamSynchronize(st) != cudaSuccess) return QMC_ERR_CUDA;
-        // T[a] = 2 raw[a + H] / L + p(0) omega(0)  (the inverse transform is unnormalised)
-        const double scale = 2.0 / (double)L, off = p0 * w0;
-        const double *raw = P + H;
-        cbc_min_kernel<<<nblk, kCbcThreads, 0, st>>>(raw, H, scale, off, per_min, part);
-        if (cudaMemcpyAsync(hpart.data(), part, nblk * sizeof(double), cudaMemcpyDeviceToHost, st) !=
-                cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return QMC_ERR_CUDA;
-        double tmin = INFINITY;
-        for (unsigned b = 0; b < nblk; ++b) tmin = std::fmin(tmin, hpart[b]);
-        const double bound = tmin + kTieRtol * w0 * tot;
-        cbc_pick_kernel<<<nblk, kCbcThreads, 0, st>>>(raw, gp, H, n, scale, off, bound, per_min, rpart,
-                                                      tpart);
-        if (cudaMemcpyAsync(hrp.data(), rpart, nblk * sizeof(uint64_t), cudaMemcpyDeviceToHost, st) !=
-                cudaSuccess ||
-            cudaMemcpyAsync(htp.data(), tpart, nblk * sizeof(double), cudaMemcpyDeviceToHost, st) !=
-                cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return QMC_ERR_CUDA;
-        uint64_t zj = n;
-        double tj = 0.0;
-        for (unsigned b = 0; b < nblk; ++b)
-            if (hrp[b] < zj) {
-                zj = hrp[b];
-                tj = htp[b];
-            }
-        if (zj >= n) return QMC_ERR_CUDA;   // non-finite sums
-        z_out[j] = zj;
-        if (e2_out) e2_out[j] = -1.0 + (beta * tot + gamma * tj) / (double)n;
-        cbc_update_kernel<<<grid_for(H + 1), kCbcThreads, 0, st>>>(p, H, n, zj, beta, gamma, 0);
-        if (!total(tot)) return QMC_ERR_CUDA;
+    const uint64_t per_sum = (H + kCbcBlocks - 1) / kCbcBlocks;
+    // the minimum and the pick do not depend on the order: blocks of at least 2048 candidates
+    const uint64_t per_min = std::max<uint64_t>(2048, per_sum);
+    const unsigned blocks = (unsigned)((H + per_min - 1) / per_min);
+    // T[a] = 2 raw[a + H] / L + p(0) omega(0)  (the inverse transform is unnormalised)
+    const double scale = 2.0 / (double)L;
+    const double *raw = P + H;
+    for (int j = 0; j < s; ++j) {
+        if (j) {
+            cbc_gather_kernel<<<grid_for(L), kCbcThreads, 0, st>>>(gp, p, H, L, n, P);
+            if (cufftExecD2Z(ws->fwd, P, FP) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
+            cbc_pointwise_kernel<<<grid_for(nc), kCbcThreads, 0, st>>>(FP, FW, nc);
+            if (cufftExecZ2D(ws->inv, FP, P) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
+            cbc_min_kernel<<<blocks, kCbcThreads, 0, st>>>(raw, p, H, scale, per_min, mins);
+            cbc_pick_kernel<<<blocks, kCbcThreads, 0, st>>>(raw, gp, p, H, n, scale, per_min, mins, blocks,
+                                                            sums + (size_t)(j - 1) * kCbcBlocks, rep, rep_t);
+        }
+        cbc_update_kernel<<<kCbcBlocks, kCbcThreads, 0, st>>>(p, H, mod, beta, gamma, j, blocks, rep, rep_t,
+                                                              per_sum, z_d, t_d, p0_d, sums);
+        if (cudaGetLastError() != cudaSuccess) return QMC_ERR_CUDA;
     }
-    return cudaStreamSynchronize(st) == cudaSuccess ? QMC_OK : QMC_ERR_CUDA;
+    std::vector<char> host(host_bytes);
+    if (cudaMemcpyAsync(host.data(), ws->base, host_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return QMC_ERR_CUDA;
+    give_back(std::move(ws));
+    const uint64_t *hz = (const uint64_t *)(host.data() + o_z);
+    const double *ht = (const double *)(host.data() + o_t), *hp0 = (const double *)(host.data() + o_p0);
+    const double *hs = (const double *)(host.data() + o_sums);
+    double tot = 0.0;   // sum_k p(k) of the components so far
+    for (int j = 0; j < s; ++j) {
+        if (hz[j] >= n) return QMC_ERR_CUDA;   // non-finite sums
+        z_out[j] = hz[j];
+        const double before = tot;
+        double acc = 0.0;
+        for (unsigned b = 0; b < kCbcBlocks; ++b) acc += hs[(size_t)j * kCbcBlocks + b];
+        tot = hp0[j] + 2.0 * acc;
+        if (e2_out) e2_out[j] = -1.0 + (j ? beta * before + gamma * ht[j] : tot) / (double)n;
+    }
+    return QMC_OK;
 }
