@@ -23,13 +23,26 @@ struct Arena {
     int device = -1;
     char *base = nullptr;
     size_t cap = 0;
+    char *pin = nullptr;   // page-locked staging for the one upload and the one download
+    size_t pin_cap = 0;
+};
+
+// Waits for the stream when a call leaves early with work enqueued: the arena and its staging
+// buffer serve the next call.
+struct DrainOnExit {
+    cudaStream_t s;
+    bool busy = false;
+    ~DrainOnExit() {
+        if (busy) cudaStreamSynchronize(s);
+    }
 };
 
 std::mutex g_mutex;
 std::vector<Arena> g_arenas;
 
-// Returns a device buffer of at least `bytes` for the current device (caller holds g_mutex).
-char *arena_get(size_t bytes, int *status) {
+// Returns the current device's buffer, of at least `bytes`, and `pin_bytes` of page-locked
+// staging (caller holds g_mutex).
+char *arena_get(size_t bytes, size_t pin_bytes, char **pin, int *status) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         *status = QMC_ERR_NO_DEVICE;
@@ -53,6 +66,17 @@ char *arena_get(size_t bytes, int *status) {
         }
         a->cap = want;
     }
+    if (a->pin_cap < pin_bytes) {
+        if (a->pin) cudaFreeHost(a->pin);
+        a->pin = nullptr;
+        a->pin_cap = 0;
+        if (cudaMallocHost(&a->pin, pin_bytes) != cudaSuccess) {
+            *status = QMC_ERR_CUDA;
+            return nullptr;
+        }
+        a->pin_cap = pin_bytes;
+    }
+    *pin = a->pin;
     *status = QMC_OK;
     return a->base;
 }
@@ -118,11 +142,14 @@ extern "C" int qmc_integrate(const qmc_integrand *f, const qmc_genvec_table *tab
     L.off_fc = take((size_t)std::max(f->nf, 0) * sizeof(double));
     L.off_ue = take((size_t)std::max(f->nu, 0) * d * sizeof(int32_t));
     L.off_fe = take((size_t)std::max(f->nf, 0) * d * sizeof(int32_t));
-    L.off_shift = take(m_cap * d * sizeof(uint64_t));
-    L.off_fit = take(6 * d * sizeof(double));
-    L.off_sums = take(4 * m_cap * sizeof(double));
+    // results and counters side by side (one download), the shifts behind them (one upload of
+    // everything up to the shifts in use)
     L.off_res = take(4 * sizeof(double));
     L.off_cnt = take(2 * sizeof(unsigned long long));
+    L.off_shift = take(m_cap * d * sizeof(uint64_t));
+    const size_t pin_bytes = o;
+    L.off_fit = take(6 * d * sizeof(double));
+    L.off_sums = take(4 * m_cap * sizeof(double));
     L.off_hist = take(use_fit ? (size_t)d * bins * sizeof(double) : 8);
     L.off_hws = take(use_fit ? qmc_histogram_workspace_bytes(n_fit, d, bins) : 8);
     // lattice-sum workspace: the largest over the (n, m) pairs the loop may visit, i.e. n
@@ -148,23 +175,36 @@ extern "C" int qmc_integrate(const qmc_integrand *f, const qmc_genvec_table *tab
     L.total = o;
 
     std::lock_guard<std::mutex> lock(g_mutex);
-    char *base = arena_get(L.total, &st);
+    char *pin = nullptr;
+    char *base = arena_get(L.total, pin_bytes, &pin, &st);
     if (st) return st;
+    DrainOnExit drain{s};
 
-    qmc_integrand df = *f;   // device copy of the description
-    auto up = [&](size_t off, const void *src, size_t bytes) -> cudaError_t {
-        if (!src || !bytes) return cudaSuccess;
-        return cudaMemcpyAsync(base + off, src, bytes, cudaMemcpyHostToDevice, s);
+    // device copy of the description: packed in the staging buffer with zeroed counters, sent
+    // with the first shifts (each array apart was a copy call of its own, and so were the
+    // counters' reset and the two result reads: 5 calls more on an 80 us integral)
+    qmc_integrand df = *f;
+    auto pack = [&](size_t off, const void *src, size_t bytes) -> const void * {
+        if (!src) return nullptr;
+        std::memcpy(pin + off, src, bytes);
+        return base + off;
     };
-    cudaError_t e = cudaSuccess;
-    if (f->c) { e = up(L.off_c, f->c, d * sizeof(double)); df.c = (const double *)(base + L.off_c); }
-    if (e == cudaSuccess && f->w) { e = up(L.off_w, f->w, d * sizeof(double)); df.w = (const double *)(base + L.off_w); }
-    if (e == cudaSuccess && f->h) { e = up(L.off_h, f->h, d * sizeof(int64_t)); df.h = (const int64_t *)(base + L.off_h); }
-    if (e == cudaSuccess && f->ucoef) { e = up(L.off_uc, f->ucoef, f->nu * sizeof(double)); df.ucoef = (const double *)(base + L.off_uc); }
-    if (e == cudaSuccess && f->fcoef) { e = up(L.off_fc, f->fcoef, f->nf * sizeof(double)); df.fcoef = (const double *)(base + L.off_fc); }
-    if (e == cudaSuccess && f->uexp) { e = up(L.off_ue, f->uexp, (size_t)f->nu * d * sizeof(int32_t)); df.uexp = (const int32_t *)(base + L.off_ue); }
-    if (e == cudaSuccess && f->fexp) { e = up(L.off_fe, f->fexp, (size_t)f->nf * d * sizeof(int32_t)); df.fexp = (const int32_t *)(base + L.off_fe); }
-    if (e != cudaSuccess) return QMC_ERR_CUDA;
+    const size_t nu = (size_t)std::max(f->nu, 0), nf = (size_t)std::max(f->nf, 0);
+    df.c = (const double *)pack(L.off_c, f->c, d * sizeof(double));
+    df.w = (const double *)pack(L.off_w, f->w, d * sizeof(double));
+    df.h = (const int64_t *)pack(L.off_h, f->h, d * sizeof(int64_t));
+    df.ucoef = (const double *)pack(L.off_uc, f->ucoef, nu * sizeof(double));
+    df.fcoef = (const double *)pack(L.off_fc, f->fcoef, nf * sizeof(double));
+    df.uexp = (const int32_t *)pack(L.off_ue, f->uexp, nu * d * sizeof(int32_t));
+    df.fexp = (const int32_t *)pack(L.off_fe, f->fexp, nf * d * sizeof(int32_t));
+    std::memset(pin + L.off_res, 0, L.off_shift - L.off_res);
+    // uploads the staging buffer from `from` on, with `count` shift values
+    auto upload = [&](size_t from, size_t count) {
+        drain.busy = true;
+        return cudaMemcpyAsync(base + from, pin + from, L.off_shift + count * sizeof(uint64_t) - from,
+                               cudaMemcpyHostToDevice, s) == cudaSuccess;
+    };
+    uint64_t *h_shifts = (uint64_t *)(pin + L.off_shift);
 
     // generating vector of a table size
     auto zrow = [&](uint64_t nn, uint64_t *z) -> int {
@@ -181,11 +221,11 @@ extern "C" int qmc_integrate(const qmc_integrand *f, const qmc_genvec_table *tab
     // seeded with seed + 1.
     double *d_fit = nullptr;
     if (use_fit) {
-        uint64_t zf[QMC_MAX_DIM], sh[QMC_MAX_DIM];
+        uint64_t zf[QMC_MAX_DIM];
         if ((st = zrow(n_fit, zf))) return st;
-        qmc_make_shifts(seed + 1, 1, d, sh);
+        qmc_make_shifts(seed + 1, 1, d, h_shifts);
+        if (!upload(0, d)) return QMC_ERR_CUDA;
         uint64_t *d_sh = (uint64_t *)(base + L.off_shift);
-        if (cudaMemcpyAsync(d_sh, sh, d * sizeof(uint64_t), cudaMemcpyHostToDevice, s) != cudaSuccess) return QMC_ERR_CUDA;
         double *d_hist = (double *)(base + L.off_hist);
         st = qmc_histogram(&df, n_fit, zf, d, d_sh, bins, d_hist, base + L.off_hws,
                            qmc_histogram_workspace_bytes(n_fit, d, bins), stream);
@@ -204,8 +244,8 @@ extern "C" int qmc_integrate(const qmc_integrand *f, const qmc_genvec_table *tab
     uint64_t evals = 0, iters = 0;
     unsigned long long counters_total[2] = {0, 0};
     double res[4] = {0, 0, 0, 0};
-    std::vector<uint64_t> sh;
     uint64_t shifts_m = 0;
+    bool described = use_fit;   // whether the description is on the device
     for (;;) {
         qmc_rule rule;
         std::memset(&rule, 0, sizeof(rule));
@@ -216,28 +256,29 @@ extern "C" int qmc_integrate(const qmc_integrand *f, const qmc_genvec_table *tab
         rule.transform = transform;
         rule.fit = d_fit;
         if (shifts_m != cur_m) {
-            sh.resize(cur_m * d);
-            qmc_make_shifts(seed, cur_m, d, sh.data());
-            if (cudaMemcpyAsync(base + L.off_shift, sh.data(), sh.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s) != cudaSuccess)
-                return QMC_ERR_CUDA;
+            // (the stream has drained since the last use of the staging buffer)
+            qmc_make_shifts(seed, cur_m, d, h_shifts);
+            if (!upload(described ? L.off_shift : 0, cur_m * d)) return QMC_ERR_CUDA;
+            described = true;
             shifts_m = cur_m;
         }
         rule.shifts = (const uint64_t *)(base + L.off_shift);
         unsigned long long *d_cnt = (unsigned long long *)(base + L.off_cnt);
-        if (cudaMemsetAsync(d_cnt, 0, 2 * sizeof(unsigned long long), s) != cudaSuccess) return QMC_ERR_CUDA;
         double *d_sums = (double *)(base + L.off_sums);
+        drain.busy = true;
         // the reservation, so that qmc_sums' size check guards it
         st = qmc_sums(&df, &rule, 0, n, base + L.off_ws, ws_bytes, d_sums, d_cnt, stream);
         if (st) return st;
         double *d_res = (double *)(base + L.off_res);
         if ((st = qmc_finalize(d_sums, cur_m, n, cplx, d_res, nullptr, stream))) return st;
-        unsigned long long cnt[2];
-        if (cudaMemcpyAsync(res, d_res, 4 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaMemcpyAsync(cnt, d_cnt, sizeof(cnt), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        // results and counters (which add up over the iterations)
+        if (cudaMemcpyAsync(pin + L.off_res, base + L.off_res, L.off_cnt + 16 - L.off_res,
+                            cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
             return QMC_ERR_CUDA;
-        counters_total[0] += cnt[0];
-        counters_total[1] += cnt[1];
+        drain.busy = false;
+        std::memcpy(res, pin + L.off_res, sizeof(res));
+        std::memcpy(counters_total, pin + L.off_cnt, sizeof(counters_total));
         evals += n * cur_m;
         ++iters;
         if (!opts || goal_met(res, cplx, opts) || evals >= opts->maxeval) break;

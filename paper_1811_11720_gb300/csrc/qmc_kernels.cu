@@ -7,6 +7,7 @@
 #include "qmc_integrands.cuh"
 #include "qmc_internal.h"
 #include "qmc_lattice.cuh"
+#include "qmc_reduce.cuh"
 #include "qmc_transforms.cuh"
 
 namespace qmc {
@@ -85,52 +86,18 @@ cudaError_t launch_points(PointsParams p, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// ---- fixed-order double-double reductions ----------------------------------------------
-struct dd {
-    double hi, lo;
-};
-
-__device__ __forceinline__ dd two_sum(double a, double b) {
-    double s = a + b;
-    double bp = s - a;
-    double e = (a - (s - bp)) + (b - bp);
-    return {s, e};
-}
-
-__device__ __forceinline__ dd dd_add(dd a, dd b) {
-    dd s = two_sum(a.hi, b.hi);
-    double e = s.lo + a.lo + b.lo;
-    double hi = s.hi + e;
-    double lo = e - (hi - s.hi);
-    return {hi, lo};
-}
-
-constexpr int kRedThreads = 256;
-
-// One block per (shift, component): thread t folds tiles t, t+256, ... in order, then a
-// fixed binary tree over the block.
+// ---- fixed-order reductions -------------------------------------------------------------
+// One block per (shift, component).
 __global__ void __launch_bounds__(kRedThreads) reduce_tiles_kernel(const double *partials,
                                                                    uint64_t tiles, int m,
                                                                    double *sums) {
-    __shared__ dd red[kRedThreads];
     const int col = blockIdx.x;           // k + m * component
     const int comp = col / m, k = col % m;
-    const double *base = partials + 2 * (uint64_t)comp * tiles * m;
-    dd acc = {0.0, 0.0};
-    for (uint64_t t = threadIdx.x; t < tiles; t += kRedThreads) {
-        const double *pp = base + 2 * (t * (uint64_t)m + k);
-        acc = dd_add(acc, dd{pp[0], pp[1]});
-    }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] = dd_add(red[threadIdx.x], red[threadIdx.x + w]);
-        __syncthreads();
-    }
+    const SumPair acc = fold_tiles(partials + 2 * (uint64_t)comp * tiles * m, tiles, m, k);
     if (threadIdx.x == 0) {
         double *o = sums + 2 * (uint64_t)comp * m + 2 * k;
-        o[0] = red[0].hi;
-        o[1] = red[0].lo;
+        o[0] = acc.hi;
+        o[1] = acc.lo;
     }
 }
 
@@ -140,10 +107,8 @@ cudaError_t launch_reduce_tiles(const double *partials, uint64_t tiles, int m, i
     return cudaGetLastError();
 }
 
-// Eq. (lattice) and Eq. (lattice-error): Q_k = S_k / n, Qbar, sigma, per component.
-// The m divisions run in parallel (one thread per shift and component); the mean and the
-// variance are then summed by one thread per component in fixed order k = 0..m-1, the
-// order the batched form uses, so both give the same bits.
+// Eq. (lattice) and Eq. (lattice-error): Q_k = S_k / n, one thread per shift and component,
+// then Qbar and sigma, one warp per component.
 constexpr int kFinThreads = 256;
 
 __global__ void __launch_bounds__(kFinThreads)
@@ -159,34 +124,20 @@ __global__ void __launch_bounds__(kFinThreads)
         q_s[i] = q;
         if (Q) Q[i] = q;
     }
+    if (!is_complex && threadIdx.x < 2) result[2 + threadIdx.x] = 0.0;
     __syncthreads();
-    const int comp = threadIdx.x;
+    const int comp = threadIdx.x >> 5;
     if (comp >= ncomp) return;
     const double *qc = q_s + (size_t)comp * m;
-    double mean = 0.0;
-#pragma unroll 8
-    for (int k = 0; k < m; ++k) mean += qc[k];
-    mean /= (double)m;
-    double var = 0.0;
-#pragma unroll 8
-    for (int k = 0; k < m; ++k) {
-        const double dq = qc[k] - mean;
-        var = fma(dq, dq, var);
-    }
-    var /= (double)m * (double)(m - 1);
-    result[2 * comp] = mean;
-    result[2 * comp + 1] = sqrt(var);
-    if (!is_complex) {
-        result[2] = 0.0;
-        result[3] = 0.0;
-    }
+    shift_stats(m, [&](int k) { return qc[k]; }, result + 2 * comp);
 }
 
 cudaError_t launch_finalize(const double *sums, int m, uint64_t n, int is_complex,
                             double *result, double *Q, cudaStream_t s) {
     const int work = m * (is_complex ? 2 : 1);
+    const int least = is_complex ? 64 : 32;   // a warp per component
     const int threads = work >= kFinThreads ? kFinThreads : ((work + 31) / 32) * 32;
-    finalize_kernel<<<1, threads, 0, s>>>(sums, m, n, is_complex, result, Q);
+    finalize_kernel<<<1, threads < least ? least : threads, 0, s>>>(sums, m, n, is_complex, result, Q);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,81 @@
+// qmc_reduce.cuh -- fixed-order reductions shared by the single-integral and the batched forms
+// (both give the same bits): tile partials to per-shift sums, per-shift sums to mean and error.
+#pragma once
+#include <cstdint>
+
+namespace qmc {
+
+// A sum as an unnormalized pair: hi is the running double sum, lo collects the rounding errors
+// of its additions (TwoSum) and the partials' own compensations.  Eight FP64 operations per
+// addition of which only hi's is on the chain from one addition to the next; renormalizing
+// after each (double-double addition) costs eleven, nine of them in a chain.
+struct SumPair {
+    double hi = 0.0, lo = 0.0;
+    __device__ __forceinline__ void add(double h, double l) {
+        const double s = hi + h;
+        const double b = s - hi;
+        lo += ((hi - (s - b)) + (h - b)) + l;
+        hi = s;
+    }
+};
+
+constexpr int kRedThreads = 256;
+
+// Folds column `col`'s (sum, compensation) pairs of `tiles` tiles, pair t at base[2 (t m + col)]:
+// thread t takes tiles t, t + 256, ... in order, then a fixed tree within each warp and one over
+// the warps.  Block of kRedThreads; the result is valid in thread 0.
+__device__ __forceinline__ SumPair fold_tiles(const double *base, uint64_t tiles, int m, int col) {
+    __shared__ SumPair part[kRedThreads / 32];
+    const double *p = base + 2 * col;   // 8-byte aligned, no more is asked of the caller
+    SumPair acc;
+#pragma unroll 4
+    for (uint64_t t = threadIdx.x; t < tiles; t += kRedThreads) {
+        const double *v = p + 2 * t * (uint64_t)m;
+        acc.add(v[0], v[1]);
+    }
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto tree = [&](int width) {
+        for (int w = width / 2; w > 0; w >>= 1) {
+            const double h = __shfl_down_sync(0xFFFFFFFFu, acc.hi, w);
+            const double l = __shfl_down_sync(0xFFFFFFFFu, acc.lo, w);
+            acc.add(h, l);
+        }
+    };
+    tree(32);
+    if (lane == 0) part[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        acc = lane < kRedThreads / 32 ? part[lane] : SumPair{};
+        tree(kRedThreads / 32);
+        const double s = acc.hi + acc.lo;   // normalized: |lo| is far below |hi|
+        acc.lo = acc.lo - (s - acc.hi);
+        acc.hi = s;
+    }
+    return acc;
+}
+
+// Mean and standard error of Q_0..Q_(m-1), value(k) each, by one warp: lane l takes k = l,
+// l + 32, ... in order, then a fixed tree.  (Eq. (lattice), Eq. (lattice-error).)
+template <class Value>
+__device__ __forceinline__ void shift_stats(int m, Value value, double *result) {
+    const int lane = threadIdx.x & 31;
+    auto all = [](double v) {
+        for (int w = 16; w > 0; w >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, w);
+        return v;
+    };
+    double s = 0.0;
+    for (int k = lane; k < m; k += 32) s += value(k);
+    const double mean = all(s) / (double)m;
+    double var = 0.0;
+    for (int k = lane; k < m; k += 32) {
+        const double dq = value(k) - mean;
+        var = fma(dq, dq, var);
+    }
+    var = all(var) / ((double)m * (double)(m - 1));
+    if (lane == 0) {
+        result[0] = mean;
+        result[1] = sqrt(var);
+    }
+}
+
+}  // namespace qmc
