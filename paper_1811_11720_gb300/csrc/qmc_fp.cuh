@@ -39,6 +39,31 @@ __device__ __forceinline__ double ipow_u(double x, int e) {
     return r;
 }
 
+// 1/a within one unit of 2^-53: the hardware's ~20-bit estimate and one cubic step, three FP64
+// instructions instead of a full division.  Outside the exponents where estimate and result are
+// normal (zero, infinities and NaN among them) the division itself.
+static __device__ __noinline__ double recip_any(double a) { return 1.0 / a; }
+__device__ __forceinline__ bool mid_range(double a) {   // 2^-1020 <= |a| < 2^1020
+    return ((uint32_t)__double2hiint(a) << 1 >> 21) - 3u < 2040u;
+}
+__device__ __forceinline__ double recip_cubic(double a) {
+    if (!mid_range(a)) return recip_any(a);
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+    const double e = fma(-a, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// 1/sqrt(a) for a > 0 likewise: y + y e (1/2 + 3/8 e), e = 1 - a y^2, five instructions.
+static __device__ __noinline__ double rsqrt_any(double a) { return rsqrt(a); }
+__device__ __forceinline__ double rsqrt_cubic(double a) {
+    if (!mid_range(a)) return rsqrt_any(a);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
 // Select between two doubles on the integer pipe.
 __device__ __forceinline__ double sel(bool p, double a, double b) { return p ? a : b; }
 

@@ -30,11 +30,15 @@ namespace qmc {
 // forms run on the integer pipe when the coordinate arrives in 0.64 fixed point:
 //   linear (1, 3, 5, 6): cl_j = c_j 2^S with S = 62 - floor(log2 sum_j c_j), so every
 //     partial sum of c_j x_j (or c_j |x_j - w_j|) stays below 2^63;
-//   Gaussian (4) and product peak (2): cq_j = c_j 2^S with S = 61 - floor(log2 max_j c_j),
-//     so |c_j (x_j - w_j)| 2^S < 2^62 and each square (2^(2S - 64) scale) is below 2^60.
-//     A square keeps only 2S - 64 fractional bits, so these forms need S >= 57 (max c < 32,
-//     at least 50 fractional bits); the product peak also caps S at 62, so that 1 at the
-//     square's scale, one = 2^(2S - 64), is at most 2^60 and 1 + q_j^2 fits below 2^61.
+//   Gaussian (4): cq_j = c_j 2^S with S = 61 - floor(log2 max_j c_j), so
+//     |c_j (x_j - w_j)| 2^S < 2^62 and each square (2^(2S - 64) scale) is below 2^60.
+//     A square keeps only 2S - 64 fractional bits, so this form needs S >= 57 (max c < 32,
+//     at least 50 fractional bits).
+//   product peak (2): the same with the largest S that keeps 1 + q_j^2, q_j <= max c, below
+//     2^64 at the square's scale (one = 2^(2S - 64) is 1 there): S = 61 and one = 2^58 for
+//     c = 5, S = 58 for max c just below 32, the same limit.  With one that large a factor
+//     1 + q^2 enters the running product as it is; scaled like the Gaussian's (one = 2^54) it
+//     had to be normalized first.
 // S is capped at 64 otherwise (small c keep 2^-64 absolute precision), so that the
 // exponential's argument scale, S or 2S - 64, lies in [2, 64] (exp_fixed).
 // Each term truncates by at most three units (2^-S, or 2^(64 - 2S) for squares); the forms
@@ -115,8 +119,8 @@ __device__ __forceinline__ void stage_fixed_forms(const P &p, FixedForms &fx) {
         S = cmax > 0.0 ? min(61 - ilogb(cmax), 64) : 64;
         ok = ok && S >= 57;
     } else if constexpr (FAM == QMC_GENZ_PRODUCT_PEAK) {
-        S = cmax > 0.0 ? min(61 - ilogb(cmax), 62) : 62;
-        ok = ok && S >= 57;
+        S = (127 - ilogb(fma(cmax, cmax, 1.0))) / 2;   // 2^(2S - 64) (1 + cmax^2) < 2^64
+        ok = ok && cmax < 32.0;
     } else {
         S = csum > 0.0 ? min(62 - ilogb(csum), 64) : 64;
     }
@@ -156,7 +160,7 @@ __device__ __forceinline__ void stage_fixed_forms(const P &p, FixedForms &fx) {
             ok = ok && (num == 0.0 || num >= 0x1p-1022);   // Fx takes zero or normal values
             fx.num = num;
             fx.numx = fx_of_double(ok ? num : 0.0);
-            fx.one = ok ? 1ull << (2 * S - 64) : 0ull;
+            fx.one = ok ? (1ull << (2 * S - 64)) + 1ull : 0ull;   // (and the square's mean loss)
         }
         fx.S = S;
         fx.ok = ok;
@@ -217,8 +221,21 @@ __device__ __forceinline__ void stage_family(const P &p, FamilyShared<FAM> &fs) 
     }
 }
 
+// What the fixed-point forms' truncated products lose on average, which their sums start from: a
+// high product 1.25 units (mulhi_trunc: half a unit for each cross product's dropped half, a
+// quarter for the low product), a square of one about 1.5 (its own 1.25 and the product's loss
+// times 2 q).  Without it the Gaussian's exponent was ~1.5 d 2^-56 low, and a d = 5 integral
+// 1e-16 high in all its shifts alike.
+__device__ __forceinline__ uint64_t linear_loss(int d) { return (uint64_t)(d + (d >> 2)); }
+__device__ __forceinline__ uint64_t square_loss(int d) { return (uint64_t)(d + (d >> 1)); }
+
+// finish_fixed<kInt> forms the family's value as a double; where the integer finish is a positive
+// number in the format Fx (all but the oscillatory family), finish_fx gives that instead, so that
+// the weight joins it before the one rounding to double.
 template <int FAM>
 struct FamilyAcc;
+template <int FAM>
+constexpr bool kFxFinish = kHasFixedForm<FAM> && FAM != QMC_GENZ_OSCILLATORY;
 
 // sum of c_j over reflected dimensions
 __device__ __forceinline__ double reflected_c_sum(uint32_t mask, int d, const SeparableShared &fs) {
@@ -247,7 +264,7 @@ struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
     // fixed point: sum c_j x_j on the integer pipe, either scaled by 2^S (then cos in FP64)
     // or, for the integer finish, as the phase in turns mod 1 (FixedForms)
     uint64_t sl;
-    __device__ __forceinline__ void init_fixed() { sl = 0; }
+    __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); }
     template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         if constexpr (kInt) {
@@ -284,23 +301,24 @@ struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
         im = 0.0;
     }
     // fixed point: f = prod c_j^2 / prod (1 + q_j^2), q_j = c_j |x_j - w_j|; each factor
-    // 1 + q_j^2 at scale 2^(2S - 64) (below 2^61, at least 2^50), the product in Fx
+    // 1 + q_j^2 at scale 2^(2S - 64) (below 2^64, at least 2^52), the product in Fx
     Fx pf;
-    __device__ __forceinline__ void init_fixed() { pf = {0x8000000000000000ull, 1}; }
+    __device__ __forceinline__ void init_fixed(int) { pf = {0x8000000000000000ull, 1}; }
     template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
         const uint64_t a = x >= w ? x - w : w - x;                       // |x - w| 2^64
         const uint64_t q = mulhi_trunc(a, fs.fx.cq[j]);                 // c |x - w| 2^S
         const uint64_t s = fs.fx.one + sqhi_trunc(q);               // (1 + q^2) 2^(2S-64)
-        pf = fx_norm(fx_mul(pf, fx_norm({s, 128 - 2 * fs.fx.S})));
+        pf = fx_norm(fx_mul(pf, Fx{s, 128 - 2 * fs.fx.S}));
     }
     template <bool kInt>
     __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        // prod c_j^2 times the reciprocal of the product (Newton on the integer pipe), or
-        // one FP64 division
-        if constexpr (kInt) re = fx_to_double(fx_mul(fs.fx.numx, fx_recip(pf)));
-        else re = fs.fx.num / fx_to_double(pf);
+        re = fs.fx.num / fx_to_double(pf);
+    }
+    // prod c_j^2 times the reciprocal of the product (Newton on the integer pipe)
+    __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
+        return fx_mul(fs.fx.numx, fx_recip(pf));
     }
 };
 
@@ -323,23 +341,22 @@ struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
         im = 0.0;
     }
     uint64_t sl;
-    __device__ __forceinline__ void init_fixed() { sl = 0; }
+    __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); }
     template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         sl += mulhi_trunc(x, fs.fx.cl[j]);
     }
     template <bool kInt>
     __device__ __forceinline__ void finish_fixed(int d, const SeparableShared &fs, double &re) {
-        if constexpr (kInt) {
-            // 1 + s as Fx (s = sl 2^-S, sl < 2^63; S = 64 drops sl's lowest bit), its
-            // (d+1)-th power and the reciprocal, all on the integer pipe
-            const int S = fs.fx.S;
-            const Fx b = S <= 63 ? fx_norm_any((1ull << S) + sl, 64 - S)
-                                 : Fx{0x8000000000000000ull + (sl >> 1), 1};
-            re = fx_to_double(fx_recip(fx_powi(b, d + 1)));
-        } else {
-            re = 1.0 / ipow_u(1.0 + scaled_fixed(sl, fs.fx.S), d + 1);
-        }
+        re = 1.0 / ipow_u(1.0 + scaled_fixed(sl, fs.fx.S), d + 1);
+    }
+    __device__ __forceinline__ Fx finish_fx(int d, const SeparableShared &fs) {
+        // 1 + s as Fx (s = sl 2^-S, sl < 2^63; S = 64 drops sl's lowest bit), its (d+1)-th
+        // power and the reciprocal, all on the integer pipe
+        const int S = fs.fx.S;
+        const Fx b = S <= 63 ? fx_norm_any((1ull << S) + sl, 64 - S)
+                             : Fx{0x8000000000000000ull + (sl >> 1), 1};
+        return fx_recip(fx_powi(b, d + 1));
     }
 };
 
@@ -362,7 +379,7 @@ struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
     }
     // fixed point: q = c |x - w| 2^S < 2^62, q^2 2^(2S - 64) < 2^60, summed in 64 bits
     uint64_t sq;
-    __device__ __forceinline__ void init_fixed() { sq = 0; }
+    __device__ __forceinline__ void init_fixed(int d) { sq = square_loss(d); }
     template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
@@ -372,8 +389,10 @@ struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
     }
     template <bool kInt>
     __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        if constexpr (kInt) re = fx_to_double_sat(exp_fixed(sq, 2 * fs.fx.S - 64, true, fs.exp2q));
-        else re = exp_table(-scaled_fixed(sq, 2 * fs.fx.S - 64), fs.exp2t);
+        re = exp_table(-scaled_fixed(sq, 2 * fs.fx.S - 64), fs.exp2t);
+    }
+    __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
+        return exp_fixed(sq, 2 * fs.fx.S - 64, true, fs.exp2q);
     }
 };
 
@@ -394,7 +413,7 @@ struct FamilyAcc<QMC_GENZ_C0> {
         im = 0.0;
     }
     uint64_t sl;
-    __device__ __forceinline__ void init_fixed() { sl = 0; }
+    __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); }
     template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
@@ -403,8 +422,10 @@ struct FamilyAcc<QMC_GENZ_C0> {
     }
     template <bool kInt>
     __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        if constexpr (kInt) re = fx_to_double_sat(exp_fixed(sl, fs.fx.S, true, fs.exp2q));
-        else re = exp_table(-scaled_fixed(sl, fs.fx.S), fs.exp2t);
+        re = exp_table(-scaled_fixed(sl, fs.fx.S), fs.exp2t);
+    }
+    __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
+        return exp_fixed(sl, fs.fx.S, true, fs.exp2q);
     }
 };
 
@@ -430,7 +451,7 @@ struct FamilyAcc<QMC_GENZ_DISCONTINUOUS> {
         im = 0.0;
     }
     uint64_t sl;
-    __device__ __forceinline__ void init_fixed() { sl = 0; zero = false; }
+    __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); zero = false; }
     template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         if (j < 2) zero |= x > fs.fx.w64[j];
@@ -438,8 +459,12 @@ struct FamilyAcc<QMC_GENZ_DISCONTINUOUS> {
     }
     template <bool kInt>
     __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        if constexpr (kInt) re = zero ? 0.0 : fx_to_double_sat(exp_fixed(sl, fs.fx.S, false, fs.exp2q));
-        else re = zero ? 0.0 : exp_table(scaled_fixed(sl, fs.fx.S), fs.exp2t);
+        re = zero ? 0.0 : exp_table(scaled_fixed(sl, fs.fx.S), fs.exp2t);
+    }
+    __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
+        Fx f = exp_fixed(sl, fs.fx.S, false, fs.exp2q);
+        if (zero) f.m = 0;
+        return f;
     }
 };
 

@@ -161,19 +161,37 @@ __device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableSha
     Weight W[NP];
     FamilyAcc<FAM> fa[NP];
 #pragma unroll
-    for (int u = 0; u < NP; ++u) fa[u].init_fixed();
-#pragma unroll 1
-    for (int j = 0; j < p.d; ++j) {
+    for (int u = 0; u < NP; ++u) fa[u].init_fixed(p.d);
+    auto dim = [&](int j, auto norm) {
         const uint64_t D = dsh(j);
 #pragma unroll
         for (int u = 0; u < NP; ++u)
-            fa[u].template add_fixed<kIntFinish>(j, transform_fixed<TK, R>(st[u].hi(j) + D, p.t, W[u]), fsh);
+            fa[u].template add_fixed<kIntFinish>(
+                j, transform_fixed<TK, R, true, decltype(norm)::value>(st[u].hi(j) + D, p.t, W[u]), fsh);
+    };
+    if constexpr (TK == kTKorobovInt) {
+        // pairs of dimensions: the weight's product is renormalized once a pair
+        int j = 0;
+        if (p.d & 1) dim(j++, std::true_type{});
+#pragma unroll 1
+        for (; j < p.d; j += 2) {
+            dim(j, std::false_type{});
+            dim(j + 1, std::true_type{});
+        }
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < p.d; ++j) dim(j, std::true_type{});
     }
 #pragma unroll
     for (int u = 0; u < NP; ++u) {
-        const double wt = weight_finish<TK, R>(W[u], p.t, cd);
-        fa[u].template finish_fixed<kIntFinish>(p.d, fsh, g[u]);
-        g[u] *= wt;
+        if constexpr (kIntFinish && kFxFinish<FAM>) {
+            Fx f = fa[u].finish_fx(p.d, fsh);
+            if constexpr (kIntKorobov<TK>) f = fx_mul(f, weight_fx<TK, R>(W[u], p.t, cd, p.d));
+            g[u] = fx_to_double_sat(fx_norm(f));
+        } else {
+            fa[u].template finish_fixed<kIntFinish>(p.d, fsh, g[u]);
+            g[u] *= weight_finish<TK, R>(W[u], p.t, cd, p.d);
+        }
     }
 }
 

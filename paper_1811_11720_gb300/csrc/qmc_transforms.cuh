@@ -89,13 +89,30 @@ __device__ __forceinline__ Mapped apply_transform(double u, const TransformParam
     }
 }
 
+// korobov_phi_fixed of order R, or for R = 0 of the order at run time (uniform).
+template <int R>
+__device__ __forceinline__ uint64_t korobov_phi_of(uint64_t V, int r, Fx &Wp) {
+    if constexpr (R > 0) {
+        return korobov_phi_fixed<R>(V, Wp);
+    } else {
+        switch (r) {
+        case 1: return korobov_phi_fixed<1>(V, Wp);
+        case 2: return korobov_phi_fixed<2>(V, Wp);
+        case 3: return korobov_phi_fixed<3>(V, Wp);
+        case 4: return korobov_phi_fixed<4>(V, Wp);
+        case 5: return korobov_phi_fixed<5>(V, Wp);
+        default: return korobov_phi_fixed<6>(V, Wp);
+        }
+    }
+}
+
 // The integer-pipe Korobov maps take the lattice state's top word X = x 2^64 instead of the
 // rounded u: v = min(x, 1 - x) in 0.64 fixed point.
 template <int TK, int R>
 __device__ __forceinline__ Mapped korobov_int_x(uint64_t X, const TransformParams &t, Weight &W) {
     const bool lo = !(X >> 63);
     if constexpr (TK == kTKorobovGen) return {fixed_to_double64(korobov_gen_phi(X, t, W.wp, W.wq)), !lo};
-    else return {fixed_to_double64(korobov_phi_fixed<R>(lo ? X : ~X, W.wp)), !lo};
+    else return {fixed_to_double64(korobov_phi_of<R>(lo ? X : ~X, t.r0, W.wp)), !lo};
 }
 
 // Transforms that are exact or fixed-point on the integer pipe can hand the integrand the
@@ -107,7 +124,8 @@ constexpr bool kIntKorobov = TK == kTKorobovInt || TK == kTKorobovGen;
 template <int TK>
 constexpr bool kFixedTransform = TK == QMC_T_NONE || TK == QMC_T_BAKER || kIntKorobov<TK>;
 
-template <int TK, int R>
+// kOdd: the form of Korobov<R,R> for the separable families (korobov_odd_fixed).
+template <int TK, int R, bool kOdd = false, bool kNorm = true>
 __device__ __forceinline__ uint64_t transform_fixed(uint64_t X, const TransformParams &t, Weight &W) {
     if constexpr (TK == QMC_T_NONE) {
         return X;
@@ -118,23 +136,31 @@ __device__ __forceinline__ uint64_t transform_fixed(uint64_t X, const TransformP
         return X >> 63 ? ~F : F;
     } else {
         static_assert(TK == kTKorobovInt, "no fixed-point form");
+        if constexpr (kOdd) return korobov_odd_fixed<R, kNorm>(X, W.wp);
         const bool lo = !(X >> 63);
-        const uint64_t F = korobov_phi_fixed<R>(lo ? X : ~X, W.wp);
+        const uint64_t F = korobov_phi_of<R>(lo ? X : ~X, t.r0, W.wp);
         return lo ? F : ~F;
     }
+}
+
+// The weight of the integer-pipe Korobov maps (cd = C^d); odd_dims: d where Korobov<R,R> ran in
+// its odd form, else 0.
+template <int TK, int R>
+__device__ __forceinline__ Fx weight_fx(const Weight &W, const TransformParams &t, double cd, int odd_dims) {
+    if constexpr (TK == kTKorobovGen) return korobov_gen_weight(W.wp, W.wq, t, fx_of_double(cd));
+    else if constexpr (R == 0) return fx_norm(fx_mul(fx_powi(W.wp, t.r0), fx_of_double(cd)));
+    else return korobov_weight_fixed<R>(W.wp, fx_of_double(cd), odd_dims);
 }
 
 // cd = C^d for Korobov (folded once per launch).
 template <int TK, int R = 0>
 __device__ __forceinline__ double weight_finish(const Weight &W, const TransformParams &t,
-                                                double cd) {
+                                                double cd, int odd_dims = 0) {
     if constexpr (TK == QMC_T_KOROBOV) {
         if (t.r0 == t.r1) return cd * ipow_u(W.wu, t.r0) * W.w;
         return cd * ipow_u(W.wu, t.r0) * ipow_u(W.w1, t.r1) * W.w;
-    } else if constexpr (TK == kTKorobovInt) {
-        return korobov_weight_fixed<R>(W.wp, fx_of_double(cd)) * W.w;
-    } else if constexpr (TK == kTKorobovGen) {
-        return korobov_gen_weight(W.wp, W.wq, t, fx_of_double(cd)) * W.w;
+    } else if constexpr (kIntKorobov<TK>) {
+        return fx_to_double(weight_fx<TK, R>(W, t, cd, odd_dims)) * W.w;
     } else {
         return W.w;
     }
@@ -146,15 +172,6 @@ __device__ __forceinline__ double weight_finish(const Weight &W, const Transform
 //   [6] a6 = 1 - |a2| - |a3| - a4 - a5, [7] |a2| (a0 - 1) a0, [8] |a3| (a1 - 1) a1,
 //   [9] 2 a5, [10] 3 a6 (the derivative's coefficients).
 constexpr int kFitStride = 11;
-
-// 1/a within one unit of 2^-53 for a normal a with a normal reciprocal: the hardware's ~20-bit
-// estimate and one cubic step, three FP64 instructions instead of a full division.
-__device__ __forceinline__ double recip_cubic(double a) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = fma(-a, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
 
 __device__ __forceinline__ double apply_fit(double x, const double *fp, double &jac) {
     const double d0 = fp[0] - x;
