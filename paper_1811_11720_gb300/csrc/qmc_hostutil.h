@@ -237,8 +237,8 @@ inline cudaError_t launch_sums_any(int family, int tkind, const LatticeLaunch &l
         return launch_sums_genz(family, tkind, lp, max_d, s);
     case QMC_GENZ_C0: case QMC_GENZ_DISCONTINUOUS: case QMC_MONOMIAL: case QMC_TRIG:
         return launch_sums_other(family, tkind, lp, max_d, s);
-    case QMC_SECTOR: case QMC_FEYNMAN:
-        return launch_sums_poly(family, tkind, lp, max_d, s);
+    case QMC_SECTOR: return launch_sums_sector(tkind, lp, max_d, s);
+    case QMC_FEYNMAN: return launch_sums_feynman(tkind, lp, max_d, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -13,7 +13,9 @@ namespace qmc {
 // Returns cudaErrorInvalidValue when (family, transform) is not in that group.
 cudaError_t launch_sums_genz(int family, int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
 cudaError_t launch_sums_other(int family, int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
-cudaError_t launch_sums_poly(int family, int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
+cudaError_t launch_sums_sector(int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
+cudaError_t launch_sums_feynman(int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
+cudaError_t launch_sums_feynman_large(int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s);
 
 struct PointsParams {
     uint64_t n, i_begin, count;

@@ -55,6 +55,8 @@ struct PolyShared {
     // as round(c 2^sf) at u[3 kMaxTerms + e], U's as round(c 2^su) at u[kMaxTerms + e];
     // the nested-form coefficients of F and U after their FP64 tensors (feyn_add_horner)
     int feyn_fixed, sf, su;
+    // the values at z in fixed point as well (stage_feynman_full): scales
+    int feyn_full, sv, svu, s3, s2u, sg, sh, sgu;
     // real family, dense F with non-negative coefficients and a positive constant term
     // whose error bound passes (stage_poly): the dense coefficients in place as
     // round(c 2^sfix) (unsigned), evaluated by dense_eval_fixed
@@ -210,13 +212,6 @@ __device__ __forceinline__ bool feyn_tensor_cheaper(const PolyShared &ps, const 
     return dense < sparse;
 }
 
-// Partial sum l of a list of non-negative coefficients; -infinity when one is negative (NaN).
-__device__ __forceinline__ double sum_nonneg(const double *c, int n, int l) {
-    double s = 0.0;
-    for (int e = l; e < n; e += kSumLanes) s += c[e] >= 0.0 ? c[e] : -INFINITY;
-    return s;
-}
-
 // What the products of dense_eval_fixed truncate on average, in units of 2^-s, as added to the
 // constant term: a high product is 1.25 units low on average (mulhi_trunc: half a unit for
 // each cross product's dropped low half and a quarter for the low product), the loss of an
@@ -224,6 +219,153 @@ __device__ __forceinline__ double sum_nonneg(const double *c, int n, int l) {
 __device__ __forceinline__ uint64_t dense_truncation(int d, int D) {
     const double n1 = d, n2 = d * (d + 1) / 2, n3 = d * (d + 1) * (d + 2) / 6;
     return (uint64_t)(1.25 * (n1 + 0.5 * n2 + (D == 3 ? 0.25 * n3 : 0.0)));
+}
+
+// Sums of products of signed fixed-point numbers in three multiplies each.  A 64-bit integer is
+// written as h 2^32 + l with signed 32-bit digits (l its low word as signed, h the high word
+// plus l's sign bit), so the high word of a product is h h' + (h l' + l h') 2^-32 with every
+// partial product signed: one wide multiply-add into a 64-bit sum and two high multiply-adds
+// into a 32-bit one, where the unsigned high product with its sign corrections and 64-bit adds
+// takes 11 to 15 instructions.  The l l' product (below one unit, mean zero) is dropped, and
+// each high multiply drops its fraction, half a unit on average: the 32-bit sum starts at the
+// number of products, which makes it up.  That sum must not overflow: callers bound
+// (sum |h| + sum |h'|) / 2 below 2^31 - 16, or with kSplit, two 32-bit sums, each half of it.
+__device__ __forceinline__ uint64_t signed_digits(long long v) {
+    return (uint64_t)v + ((uint64_t)((uint32_t)v >> 31) << 32);
+}
+struct Digits {
+    int h, l;
+    __device__ __forceinline__ Digits() {}
+    __device__ __forceinline__ Digits(uint64_t packed) : h((int)(packed >> 32)), l((int)packed) {}
+};
+__device__ __forceinline__ Digits digits_of(int64_t v) { return Digits(signed_digits(v)); }
+template <bool kSplit = false>
+struct DigitDot {
+    int64_t wide = 0;
+    int cross, cross2 = 0;
+    __device__ __forceinline__ explicit DigitDot(int products) : cross(products) {}
+    __device__ __forceinline__ void add(const Digits &a, const Digits &b) {
+        wide += (int64_t)a.h * b.h;
+        asm("mad.hi.s32 %0, %1, %2, %0;" : "+r"(cross) : "r"(a.h), "r"(b.l));
+        int &c = kSplit ? cross2 : cross;
+        asm("mad.hi.s32 %0, %1, %2, %0;" : "+r"(c) : "r"(a.l), "r"(b.h));
+    }
+    __device__ __forceinline__ int64_t value() const {   // sum a b 2^-64
+        return kSplit ? wide + cross + cross2 : wide + cross;
+    }
+};
+
+// Where the complex family's values F(z), U(z) may be formed in fixed point too
+// (feyn_full_values), and the scales.  Every quantity there carries an absolute error of a few
+// units of 2^-57 of its bound, where FP64's rounding is relative; so the form is taken when F
+// has a constant term c0 and all bounds stay near it: no FP64 evaluation of F is better than
+// 2^-54 |c0| either, as its terms are added to c0.  (Without c0, F(x) near a corner of the cube
+// is many orders below its coefficients, and a fixed-point F(x) missed the oracle by 1e-8.)
+// U enters as a factor, so its absolute error counts against its coefficients' sum.
+template <class PS>
+__device__ __forceinline__ void stage_feynman_full(PS &ps, int d) {
+    const int tid = threadIdx.x;
+    const int nU = 1 + d + d * d, nF = nU + d * d * (d + 1) / 2;
+    const double *ub = ps.buf.v, *fb = ps.buf.v + 2 * kMaxTerms;
+    const double *hu = ub + nU, *hf = fb + nF;
+    const int n2 = d * (d + 1) / 2, n3 = d * (d + 1) * (d + 2) / 6;
+    // row bounds over the cube: |dF/dx_i|, |H_ij|, |dU/dx_i|
+    for (int i = tid; i < d; i += blockDim.x) {
+        const double *f1 = fb + 1, *F2 = f1 + d, *F3 = F2 + d * d, *u1 = ub + 1, *U2 = u1 + d;
+        double g = fabs(f1[i]), hmax = 0.0, gu = fabs(u1[i]);
+        for (int j = 0; j < d; ++j) {
+            double h = 2.0 * fabs(F2[i * d + j]);
+            const double *t = F3 + (i <= j ? feyn_pair(i, j, d) : feyn_pair(j, i, d)) * d;
+            double s = 0.0;
+            for (int k = 0; k < d; ++k) s += fabs(t[k]);
+            h += s;
+            hmax = fmax(hmax, h);
+            g += 2.0 * fabs(F2[i * d + j]) + 0.5 * s;
+            gu += 2.0 * fabs(U2[i * d + j]);
+        }
+        ps.part[0][i] = g;
+        ps.part[1][i] = hmax;
+        ps.part[0][8 + i] = gu;
+    }
+    if (tid == blockDim.x - 1) {
+        double bf = 0.0, bu = 0.0;
+        for (int e = 0; e < 1 + d + n2 + n3; ++e) bf += fabs(hf[e]);
+        for (int e = 0; e < 1 + d + n2; ++e) bu += fabs(hu[e]);
+        ps.part[1][8] = bf;
+        ps.part[1][9] = bu;
+        double b3 = 0.0, b2 = 0.0;
+        for (int e = 0; e < n3; ++e) b3 += fabs(hf[1 + d + n2 + e]);
+        for (int e = 0; e < n2; ++e) b2 += fabs(hu[1 + d + e]);
+        ps.part[1][10] = b3;
+        ps.part[1][11] = b2;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double g = 0.0, h = 0.0, gu = 0.0;
+        for (int i = 0; i < d; ++i) {
+            g = fmax(g, ps.part[0][i]);
+            h = fmax(h, ps.part[1][i]);
+            gu = fmax(gu, ps.part[0][8 + i]);
+        }
+        const double bf = ps.part[1][8], bu = ps.part[1][9], b3 = ps.part[1][10], b2 = ps.part[1][11];
+        const double c0 = fabs(hf[0]), lam = fabs(ps.lam), y = 0.25 * g;   // |y_k| <= lam y
+        int ok = g > 0.0 && h > 0.0 && gu > 0.0 && lam < 1e3 && bf <= 16.0 * c0 &&
+                 lam * d * g * y <= 64.0 * c0 && lam * lam * d * d * h * y * y <= 64.0 * c0 &&
+                 lam * lam * lam * b3 * y * y * y <= c0 && lam * lam * b2 * y * y <= bu &&
+                 lam * d * gu * y <= 64.0 * bu && bf < 1e30 && bu < 1e30 && bf > 1e-30 && bu > 1e-30 &&
+                 h > 1e-30 && g > 1e-30 && gu > 1e-30;
+        if (ok) {
+            ps.sv = 60 - ilogb(bf);                       // partial sums of F(x) below 2^61
+            ps.svu = 60 - ilogb(bu);
+            ps.s3 = b3 > 0.0 ? 60 - max(ilogb(b3), -100) : 0;
+            ps.s2u = b2 > 0.0 ? 60 - max(ilogb(b2), -100) : 0;
+            ps.sg = 60 - ilogb(g);                        // |g| 2^sg, |H| 2^sh, |grad U| 2^sgu < 2^61
+            ps.sh = 60 - ilogb(h);
+            ps.sgu = 60 - ilogb(gu);
+            ok = abs(ps.sg - ps.sh) < 40;
+        }
+        ps.feyn_full = ok;
+    }
+    __syncthreads();
+    if (!ps.feyn_full) return;
+    // in signed digits behind the fixed-point tensors (FeynFull): the Hessian's, the gradients',
+    // the nested forms of the values at 2^sv (2^svu), and their top-degree coefficients again at
+    // 2^s3 (2^s2u) for the terms at y
+    const int nHu = 1 + d + n2, nHf = nHu + n3, nT = d * n2;
+    const double *f1 = fb + 1, *F2 = f1 + d, *F3 = F2 + d * d, *u1 = ub + 1, *U2 = u1 + d;
+    uint64_t *qf = ps.buf.u + 3 * kMaxTerms + nF, *qu = ps.buf.u + kMaxTerms + nU;
+    auto digits = [](double c, int e) { return signed_digits(llrint(ldexp(c, e))); };
+    for (int e = tid; e < nT; e += blockDim.x) qf[e] = digits(F3[e], ps.sh);
+    for (int e = tid; e < d * d; e += blockDim.x) {
+        qf[nT + e] = (uint64_t)llrint(ldexp(2.0 * F2[e], ps.sh));
+        qu[e] = digits(2.0 * U2[e], ps.sgu);
+    }
+    qf += nT + d * d;
+    qu += d * d;
+    for (int e = tid; e < d; e += blockDim.x) {
+        qf[e] = (uint64_t)llrint(ldexp(f1[e], ps.sg));
+        qu[e] = (uint64_t)llrint(ldexp(u1[e], ps.sgu));
+    }
+    qf += d;
+    qu += d;
+    // (linear and lower coefficients are added, not multiplied: plain integers)
+    for (int e = tid; e < nHf; e += blockDim.x) {
+        const long long c = llrint(ldexp(hf[e], ps.sv));
+        qf[e] = e < nHu ? (uint64_t)c : signed_digits(c);
+    }
+    for (int e = tid; e < n3; e += blockDim.x) qf[nHf + e] = digits(hf[1 + d + n2 + e], ps.s3);
+    for (int e = tid; e < nHu; e += blockDim.x) {
+        const long long c = llrint(ldexp(hu[e], ps.svu));
+        qu[e] = e < 1 + d ? (uint64_t)c : signed_digits(c);
+    }
+    for (int e = tid; e < n2; e += blockDim.x) qu[nHu + e] = digits(hu[1 + d + e], ps.s2u);
+}
+
+// Partial sum l of a list of non-negative coefficients; -infinity when one is negative (NaN).
+__device__ __forceinline__ double sum_nonneg(const double *c, int n, int l) {
+    double s = 0.0;
+    for (int e = l; e < n; e += kSumLanes) s += c[e] >= 0.0 ? c[e] : -INFINITY;
+    return s;
 }
 
 // allow_dense: the real sector family evaluates through the dense Horner form when
@@ -242,6 +384,7 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
         ps.maxdeg_u = 0;
         ps.maxdeg_f = 0;
         ps.feyn_fixed = 0;
+        ps.feyn_full = 0;
         ps.fixed_f = 0;
         ps.fixed_u = 0;
         const double tb = 2.0 * p.pb;
@@ -327,6 +470,8 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
                 for (int q = 0; q < p.nu; ++q) feyn_add_horner(hu, p.uexp + (size_t)q * d, d, p.ucoef[q]);
                 for (int q = 0; q < p.nf; ++q) feyn_add_horner(hf, p.fexp + (size_t)q * d, d, p.fcoef[q]);
             }
+            __syncthreads();
+            stage_feynman_full(ps, d);
         }
         return;
     }
@@ -416,6 +561,12 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
 __device__ __forceinline__ int64_t smulhi_x(int64_t c, uint64_t X) {
     const uint64_t h = mulhi_trunc((uint64_t)c, X);
     return (int64_t)(c < 0 ? h - X : h);
+}
+// a b / 2^64 for signed a and b, up to 3 units low: the unsigned high word of their residues,
+// minus the other factor for each negative one.
+__device__ __forceinline__ int64_t smulhi(int64_t a, int64_t b) {
+    const uint64_t h = mulhi_trunc((uint64_t)a, (uint64_t)b);
+    return (int64_t)(h - ((uint64_t)(a >> 63) & (uint64_t)b) - ((uint64_t)(b >> 63) & (uint64_t)a));
 }
 // x in [0, 1] to x 2^64, truncated (x = 1 saturates to 2^64 - 1).  For 0 < x < 1 with
 // biased exponent E <= 1022, x 2^64 is the 64-bit mantissa shifted right by 1022 - E.
@@ -678,8 +829,9 @@ __device__ __forceinline__ cplx cmul(cplx a, cplx b) {
     return {fma(a.re, b.re, -a.im * b.im), fma(a.re, b.im, a.im * b.re)};
 }
 __device__ __forceinline__ cplx crecip(cplx a) {
-    // scaled to avoid overflow of |a|^2 for the magnitudes met here (|a| in 1e-150..1e150)
-    double s = 1.0 / fma(a.re, a.re, a.im * a.im);
+    // no scaling: |a|^2 neither overflows nor underflows for the magnitudes met here (|a| in
+    // 1e-150..1e150)
+    double s = recip_cubic(fma(a.re, a.re, a.im * a.im));
     return {a.re * s, -a.im * s};
 }
 
@@ -764,13 +916,9 @@ __device__ __forceinline__ cplx feynman_jacobian_det(const double *x, const doub
 // those of the elimination above up to rounding.  In the first step K is purely
 // imaginary and K_rc K_cq = -H_rc H_cq is real.
 template <int D>
-__device__ __forceinline__ cplx feynman_jacobian_det_sym(const double *x, const double *lx,
-                                                         const double *g, const double *H,
-                                                         double lam) {
+__device__ __forceinline__ cplx feynman_jacobian_det_sym(const double *lx, const double *lamb,
+                                                         const double *H) {
     double Kr[D * D], Ki[D * D];   // upper triangle, K_rq at r * D + q for q >= r
-    double lamb[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) lamb[k] = -lam * fma(-2.0, x[k], 1.0) * g[k];
     cplx det = {1.0, fma(lx[0], H[0], lamb[0])};   // A_00 = 1 + i (Λ_0 + p_0 H_00)
     if constexpr (D == 1) return det;
     {
@@ -814,16 +962,20 @@ __device__ __forceinline__ cplx feynman_jacobian_det_sym(const double *x, const 
 __device__ __forceinline__ cplx csqrt_principal(cplx a) {
     // |a| without the library's rescaling where the squares can neither overflow nor
     // underflow (both exponents within (2^-500, 2^500): a test on the bit patterns, off the
-    // FP64 pipe; relative error within 1.5 ulp)
+    // FP64 pipe; relative error within 2 ulp)
     const uint64_t br = (uint64_t)__double_as_longlong(a.re), bi = (uint64_t)__double_as_longlong(a.im);
     const uint32_t er = (uint32_t)(br >> 52) & 0x7FFu, ei = (uint32_t)(bi >> 52) & 0x7FFu;
-    const double r = (er - 524u < 998u && ei - 524u < 998u)   // 524 <= E <= 1521
-                         ? sqrt(fma(a.re, a.re, a.im * a.im))
-                         : hypot(a.re, a.im);
+    double r;
+    if (er - 524u < 998u && ei - 524u < 998u) {   // 524 <= E <= 1521
+        const double n2 = fma(a.re, a.re, a.im * a.im);
+        r = n2 * rsqrt_cubic(n2);
+    } else {
+        r = hypot(a.re, a.im);
+    }
     if (((br | bi) << 1) == 0) return {0.0, a.im};            // a = 0
     // t = sqrt(s) and a.im / (2 t) from one reciprocal square root
     const double s = 0.5 * (r + fabs(a.re));
-    const double q = rsqrt(s);
+    const double q = rsqrt_cubic(s);
     const double t = s * q;
     const double o = a.im * (0.5 * q);
     if (!(br >> 63) || !(br << 1)) return {t, o};             // a.re >= 0 (and -0)
@@ -1087,8 +1239,129 @@ static __device__ __noinline__ void feynman_value_dense(const IN *xin, int d_rt,
     }
     if (Fz.im > 0.0) ++signfail;
     cplx det;
-    if constexpr (FX) det = feynman_jacobian_det_sym<DT>(x, xo, g, H, lam);
-    else det = feynman_jacobian_det<DT>(x, xo, g, H, d, lam);
+    if constexpr (FX) {
+        double lamb[DA];
+#pragma unroll
+        for (int k = 0; k < DA; ++k) lamb[k] = -lam * fma(-2.0, x[k], 1.0) * g[k];
+        det = feynman_jacobian_det_sym<DT>(xo, lamb, H);
+    } else det = feynman_jacobian_det<DT>(x, xo, g, H, d, lam);
+    feynman_combine(Uz, Fz, det, ps.pa, ps.pb, ps.pow_half, re, im);
+}
+
+// The whole integrand but det J and the power in fixed point (stage_feynman_full): F(x), U(x)
+// by the nested form, and at z = x - i lam yh, yh_k = x_k (1 - x_k) g_k,
+//   F(z) = F(x) - lam^2 yh.H yh / 2 - i (lam g.yh - lam^3 F3[yh, yh, yh]),
+//   U(z) = U(x) - lam^2 yh.U2 yh - i lam grad U.yh.
+// All sums of products run in signed digits (DigitDot): x as x 2^61 (its high digit at most
+// 2^29, so six terms' cross products stay below 2^31; a sum comes back 8 times too small and is
+// shifted up), yh as Y = 4 yh 2^sg, |Y| < 2^61, and g, H and grad U below 2^61.  What is left
+// in FP64 (~215 instructions for d = 5 instead of ~450) is det J, the power and one
+// multiply-add per value.  n = 1,072,187, m = 32: 29.8 ms with F(z), U(z) in FP64 (FP64 pipe
+// 81 % busy), 24.4 in fixed point with unsigned products, 23.3 in signed digits, and 19.1 with
+// two blocks per SM (kSumsMinBlocks).
+template <int D>
+static __device__ __noinline__ void feynman_value_full(const uint64_t *Xin, const PolyShared &ps,
+                                                       double &re, double &im,
+                                                       unsigned long long &signfail) {
+    constexpr int n2 = D * (D + 1) / 2, n3 = D * (D + 1) * (D + 2) / 6;
+    constexpr int nU = 1 + D + D * D, nF = nU + D * n2, nHu = 1 + D + n2, nHf = nHu + n3;
+    const uint64_t *h3 = ps.buf.u + 3 * kMaxTerms + nF, *h2 = h3 + D * n2, *f1 = h2 + D * D;
+    const uint64_t *qf = f1 + D, *c3y = qf + nHf;
+    const uint64_t *g2u = ps.buf.u + kMaxTerms + nU, *u1 = g2u + D * D, *qu = u1 + D, *c2y = qu + nHu;
+    const int sg = ps.sg, sh = ps.sh;
+    const double lam = ps.lam;
+    Digits x[D], Y[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) x[k] = digits_of((int64_t)(Xin[k] >> 3));
+    int64_t Hq[D * D];
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = i; j < D; ++j) {
+            DigitDot<> t(D);
+#pragma unroll
+            for (int k = 0; k < D; ++k) t.add(h3[feyn_pair(i, j, D) * D + k], x[k]);
+            Hq[i * D + j] = Hq[j * D + i] = (int64_t)h2[i * D + j] + (t.value() << 3);
+        }
+    // gradients, g = f1 + (2 F2 + H) x / 2 and grad U = u1 + 2 U2 x; Y, and the first-order terms
+    double lx[D], lamb[D];
+    int64_t gy = 0, gUy = 0;
+    const int eg = sg - sh + 2;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        DigitDot<true> t(D);   // H is bounded by entries, not by rows
+        DigitDot<> u(D);
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            t.add(digits_of((Hq[i * D + j] >> 1) + ((int64_t)h2[i * D + j] >> 1)), x[j]);
+            u.add(g2u[i * D + j], x[j]);
+        }
+        const int64_t v = t.value();   // (2 F2 + H) x / 2 at 2^(sh - 3)
+        const int64_t gq = (int64_t)f1[i] + (eg >= -1 ? v << (eg + 1) : v >> (-1 - eg));
+        const uint64_t X = Xin[i];
+        const uint64_t T = mulhi_trunc(X, ~X);   // x (1 - x) 2^64, below 2^62
+        Y[i] = digits_of(smulhi_x(gq, T << 2));
+        DigitDot<> s(1), r(1);
+        s.add(digits_of(gq), Y[i]);
+        r.add(digits_of((int64_t)u1[i] + (u.value() << 3)), Y[i]);
+        gy += s.value();
+        gUy += r.value();
+        // -lam x (1 - x) and -lam (1 - 2 x) g for det J; (1 - 2 x) 2^63 = 2^63 - X, less one
+        // unit so that X = 0 stays positive
+        lx[i] = -lam * fixed_u64_to_double(T, 64);
+        lamb[i] = -lam * fixed_s64_to_double(smulhi(gq, (int64_t)(0x7FFFFFFFFFFFFFFFull - X)), sg - 1);
+    }
+    // the higher terms at y, and the values at x
+    DigitDot<true> yHy(D);
+    DigitDot<> dF(D), dU(D), cF(D), qU(D);
+    {
+        const uint64_t *c2f = qf + 1 + D, *c3f = c2f + n2, *c2u = qu + 1 + D;
+        int p2 = 0, p3 = 0;
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            DigitDot<true> off(D - 1 - i);
+            DigitDot<> diag(1), tf(D - i), tu(D - i), ty(D - i), tuy(D - i);
+#pragma unroll
+            for (int j = i; j < D; ++j) {
+                if (j == i) diag.add(digits_of(Hq[i * D + j]), Y[j]);
+                else off.add(digits_of(Hq[i * D + j]), Y[j]);
+                DigitDot<> a(D - j), b(D - j);
+#pragma unroll
+                for (int k = j; k < D; ++k) {
+                    a.add(c3f[p3], x[k]);
+                    b.add(c3y[p3], Y[k]);
+                    ++p3;
+                }
+                tf.add(digits_of((int64_t)c2f[p2] + (a.value() << 3)), x[j]);
+                ty.add(digits_of(b.value()), Y[j]);
+                tu.add(c2u[p2], x[j]);
+                tuy.add(c2y[p2], Y[j]);
+                ++p2;
+            }
+            yHy.add(digits_of(diag.value() + 2 * off.value()), Y[i]);
+            dF.add(digits_of((int64_t)qf[1 + i] + (tf.value() << 3)), x[i]);
+            dU.add(digits_of((int64_t)qu[1 + i] + (tu.value() << 3)), x[i]);
+            cF.add(digits_of(ty.value()), Y[i]);
+            qU.add(digits_of(tuy.value()), Y[i]);
+        }
+    }
+    const int64_t Fq = (int64_t)qf[0] + (dF.value() << 3), Uq = (int64_t)qu[0] + (dU.value() << 3);
+    gy = gy < 0 ? 0 : gy;   // a sum of squares, truncated
+    const int sy = sg + 2;
+    const double l2 = lam * lam;
+    const cplx Fz = {fma(-0.5 * l2, fixed_s64_to_double(yHy.value(), sh + 2 * sy - 128),
+                         fixed_s64_to_double(Fq, ps.sv)),
+                     fma(l2 * lam, fixed_s64_to_double(cF.value(), ps.s3 + 3 * (sy - 64)),
+                         -lam * fixed_s64_to_double(gy, sg + sy - 64))};
+    const cplx Uz = {fma(-l2, fixed_s64_to_double(qU.value(), ps.s2u + 2 * (sy - 64)), fixed_s64_to_double(Uq, ps.svu)),
+                     -lam * fixed_s64_to_double(gUy, ps.sgu + sy - 64)};
+    if (Fz.im > 0.0) ++signfail;
+    double H[D * D];
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int j = i; j < D; ++j) H[i * D + j] = fixed_s64_to_double(Hq[i * D + j], sh);
+    const cplx det = feynman_jacobian_det_sym<D>(lx, lamb, H);
     feynman_combine(Uz, Fz, det, ps.pa, ps.pb, ps.pow_half, re, im);
 }
 
@@ -1101,6 +1374,14 @@ __device__ __forceinline__ bool feyn_fixed_ok(const PolyShared &ps, int d) {
 __device__ __forceinline__ void feynman_value_x(const uint64_t *X, int d, const PolyShared &ps,
                                                 double &re, double &im,
                                                 unsigned long long &signfail) {
+    if (ps.feyn_full) {
+        switch (d) {
+        case 3: feynman_value_full<3>(X, ps, re, im, signfail); return;
+        case 4: feynman_value_full<4>(X, ps, re, im, signfail); return;
+        case 5: feynman_value_full<5>(X, ps, re, im, signfail); return;
+        default: feynman_value_full<6>(X, ps, re, im, signfail); return;
+        }
+    }
     switch (d) {
     case 3: feynman_value_dense<3, true>(X, d, ps, re, im, signfail); return;
     case 4: feynman_value_dense<4, true>(X, d, ps, re, im, signfail); return;

@@ -41,10 +41,10 @@ __device__ __forceinline__ void neumaier_add(double &s, double &c, double v) {
 // Fit constants per dimension in shared memory (see apply_fit).
 __device__ __forceinline__ void prepare_fit(const double *fit, int d, double *s_fit) {
     const int tid = threadIdx.x;
-    if (fit && tid < d) {
-        const double *a = fit + 6 * tid;
+    for (int j = tid; fit && j < d; j += blockDim.x) {
+        const double *a = fit + 6 * j;
         double a2 = fabs(a[2]), a3 = fabs(a[3]);
-        double *o = s_fit + kFitStride * tid;
+        double *o = s_fit + kFitStride * j;
         o[0] = a[0];
         o[1] = a[1];
         o[2] = a2 * (a[0] - 1.0);
@@ -389,10 +389,11 @@ __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilySha
                          });
 }
 
-// The integer Korobov is compiled once per order r (uniform branch per tile).
+// The integer Korobov is compiled once per order r (uniform branch per tile) for the separable
+// families, whose time it is; the polynomial families choose the order at each use.
 template <int FAM, int TK, class... A>
 __device__ __forceinline__ void stream_sums(const Integral &p, A &&...a) {
-    if constexpr (TK == kTKorobovInt) {
+    if constexpr (TK == kTKorobovInt && !kPolyFamily<FAM>) {
         switch (p.t.r0) {
         case 1: stream_sums_r<FAM, TK, 1>(p, a...); return;
         case 2: stream_sums_r<FAM, TK, 2>(p, a...); return;
@@ -433,16 +434,17 @@ __device__ __forceinline__ void tile_partial(const StreamSum &acc, double *s_red
 }
 
 // Blocks per SM the register allocation must allow: five for the separable families (48
-// registers; their throughput depends on hiding integer latency), two for the sector family
-// (128 registers; left to itself the compiler takes more and one block runs alone: 9.0 ms
-// instead of 5.9 at d = 8, n = 1,072,187, m = 32), no constraint for the complex family (its
-// working set needs the registers).
+// registers; their throughput depends on hiding integer latency), three for the sector family
+// (85 registers; d = 8, n = 1,072,187, m = 32: 4.55 ms with two blocks, 4.43 with three, 9.0
+// with the one the compiler leaves room for by itself), two for the complex family with the
+// dimension compiled in (128 registers with a few spills; d = 5 at the same size: 23.3 ms with
+// one, 19.1 with two) and one without (d = 8 with two blocks was 15 % slower).
 template <int FAM>
-constexpr int kSumsMinBlocks = FAM == QMC_FEYNMAN ? 1 : FAM == QMC_SECTOR ? 2 : 5;
+constexpr int kSumsMinBlocks = FAM == QMC_FEYNMAN ? 2 : FAM == QMC_SECTOR ? 3 : 5;
 
 // Dynamic shared memory: the shifts, [kMaxDim or d][m].
-template <int FAM, int TK>
-__global__ void __launch_bounds__(kSumsThreads, kSumsMinBlocks<FAM>)
+template <int FAM, int TK, int MINB>
+__global__ void __launch_bounds__(kSumsThreads, MINB)
     lattice_kernel(const __grid_constant__ LatticeLaunch lp) {
     extern __shared__ uint64_t s_dsh[];
     __shared__ FamilyShared<FAM> fsh;
@@ -477,7 +479,7 @@ __global__ void __launch_bounds__(kSumsThreads, kSumsMinBlocks<FAM>)
             const int k = i / d, j = i - k * d;
             s_dsh[j * m + k] = it.shifts[i] << 11;
         }
-        if (tid < d) s_step.set(tid, it.dc[tid], it.n);
+        for (int j = tid; j < d; j += blockDim.x) s_step.set(j, it.dc[j], it.n);
         stage_family<FAM, false>(it, fsh);
         prepare_fit(it.fit, d, s_fit);
         __syncthreads();
