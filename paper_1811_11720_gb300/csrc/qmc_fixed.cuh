@@ -80,6 +80,16 @@ __device__ __forceinline__ uint64_t sqhi_trunc(uint64_t a) {
     return (uint64_t)ah * ah + ((uint64_t)__umulhi(ah, al) << 1);
 }
 
+// Fixed point for polynomial work on the integer multiply pipe: a value v is held as the
+// integer round(v 2^s) with one scale s per polynomial (signed for the complex family's
+// tensors, unsigned for the real family's non-negative dense forms), a coordinate x in
+// [0, 1] as the uint64 X = x 2^64.
+//   c X / 2^64 for signed c: the unsigned high word of (c mod 2^64) X, minus X when c < 0.
+__device__ __forceinline__ int64_t smulhi_x(int64_t c, uint64_t X) {
+    const uint64_t h = mulhi_trunc((uint64_t)c, X);
+    return (int64_t)(c < 0 ? h - X : h);
+}
+
 // ---------------------------------------------------------------------------------------
 // value = m 2^(e - 64); m == 0 encodes zero.  Normalized: m >= 2^63.
 struct Fx {

@@ -553,15 +553,6 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
     }
 }
 
-// Fixed point for polynomial work on the integer multiply pipe: a value v is held as the
-// integer round(v 2^s) with one scale s per polynomial (signed for the complex family's
-// tensors, unsigned for the real family's non-negative dense forms), a coordinate x in
-// [0, 1] as the uint64 X = x 2^64.
-//   c X / 2^64 for signed c: the unsigned high word of (c mod 2^64) X, minus X when c < 0.
-__device__ __forceinline__ int64_t smulhi_x(int64_t c, uint64_t X) {
-    const uint64_t h = mulhi_trunc((uint64_t)c, X);
-    return (int64_t)(c < 0 ? h - X : h);
-}
 // a b / 2^64 for signed a and b, up to 3 units low: the unsigned high word of their residues,
 // minus the other factor for each negative one.
 __device__ __forceinline__ int64_t smulhi(int64_t a, int64_t b) {

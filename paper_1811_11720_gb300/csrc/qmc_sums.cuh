@@ -18,6 +18,7 @@
 #pragma once
 #include <cstdint>
 
+#include "qmc_fitmap.cuh"
 #include "qmc_integrands.cuh"
 #include "qmc_transforms.cuh"
 
@@ -198,35 +199,41 @@ __device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableSha
 // One evaluation of g at a point with lattice state `st`.
 template <int FAM, int TK, int R, class St>
 __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared<FAM> &fsh,
-                                           const double *s_fit, bool use_fit, Shifts dsh, double cd,
-                                           const St &st, double &g_re, double &g_im,
+                                           const double *s_fit, const FitFixed *fit_fixed, bool use_fit,
+                                           Shifts dsh, double cd, const St &st, double &g_re, double &g_im,
                                            unsigned long long &signfail) {
     Weight W;
     FamilyAcc<FAM> fa;
-    if constexpr (kFixedTransform<TK> && FAM == QMC_SECTOR) {
-        // the real family with F in fixed point takes the coordinates as x 2^64 from the
-        // integer-pipe transform (no fit map)
-        if (!use_fit && sector_fixed_ok(fsh.poly, p.d)) {
+    if constexpr (kFixedTransform<TK> && kPolyFamily<FAM>) {
+        // the polynomial families' fixed-point forms take the coordinates as x 2^64 from the
+        // integer-pipe transform, through the integer fit map where there is one
+        bool fixed = !use_fit || fit_fixed->ok;
+        if constexpr (FAM == QMC_SECTOR) fixed = fixed && sector_fixed_ok(fsh.poly, p.d);
+        else fixed = fixed && feyn_fixed_ok(fsh.poly, p.d);
+        if (fixed) {   // uniform over the block
+            Weight V;
+            Fx J;
             uint64_t X[8];
 #pragma unroll 1
-            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), p.t, W);
-            const double wt = weight_finish<TK, R>(W, p.t, cd);
-            g_re = sector_value_x(X, p.d, fsh.poly) * wt;
-            g_im = 0.0;
-            return;
-        }
-    }
-    if constexpr (kFixedTransform<TK> && FAM == QMC_FEYNMAN) {
-        // the complex family's fixed-point form likewise takes x 2^64 from the map
-        if (!use_fit && feyn_fixed_ok(fsh.poly, p.d)) {
-            uint64_t X[kFeynFixedMaxDim];
-#pragma unroll 1
-            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), p.t, W);
-            const double wt = weight_finish<TK, R>(W, p.t, cd);
-            feynman_value_x(X, p.d, fsh.poly, g_re, g_im, signfail);
-            g_re *= wt;
-            g_im *= wt;
-            return;
+            for (int j = 0; j < p.d; ++j) X[j] = transform_fixed<TK, R>(st.hi(j) + dsh(j), p.t, V);
+            if (!use_fit || fit_fixed->apply_all(X, p.d, &J)) {
+                double wt;
+                if (use_fit) {
+                    if constexpr (kIntKorobov<TK>) J = fx_mul(J, weight_fx<TK, R>(V, p.t, cd, 0));
+                    wt = fx_to_double(J);
+                } else {
+                    wt = weight_finish<TK, R>(V, p.t, cd);
+                }
+                if constexpr (FAM == QMC_SECTOR) {
+                    g_re = sector_value_x(X, p.d, fsh.poly) * wt;
+                    g_im = 0.0;
+                } else {
+                    feynman_value_x(X, p.d, fsh.poly, g_re, g_im, signfail);
+                    g_re *= wt;
+                    g_im *= wt;
+                }
+                return;
+            }
         }
     }
     fa.init(fsh);
@@ -366,8 +373,8 @@ __device__ __forceinline__ void run_stream(const Integral &p, const BlockSteps &
 
 template <int FAM, int TK, int R>
 __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilyShared<FAM> &fsh,
-                                              const double *s_fit, bool use_fit, Shifts dsh,
-                                              const BlockSteps &steps, const WarpStreams &ws,
+                                              const double *s_fit, const FitFixed *fit_fixed,
+                                              bool use_fit, Shifts dsh, const BlockSteps &steps, const WarpStreams &ws,
                                               WarpLattice<TK> &lat, uint64_t w0, uint32_t cnt,
                                               StreamSum &acc) {
     constexpr bool kCplx = FamilyAcc<FAM>::kComplex;
@@ -384,8 +391,8 @@ __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilySha
     run_stream<kCplx, 1>(p, steps, ws, lat, w0, cnt, acc,
                          [&](auto &st, auto &g_re, auto &g_im, unsigned long long &signfail) {
                              g_im[0] = 0.0;
-                             eval_point<FAM, TK, R>(p, fsh, s_fit, use_fit, dsh, cd, st[0], g_re[0],
-                                                    g_im[0], signfail);
+                             eval_point<FAM, TK, R>(p, fsh, s_fit, fit_fixed, use_fit, dsh, cd, st[0],
+                                                    g_re[0], g_im[0], signfail);
                          });
 }
 
@@ -453,6 +460,11 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
     __shared__ WarpLattice<TK> s_lat[kSumsThreads / 32];
     __shared__ Integral s_item;
     __shared__ BlockSteps s_step;
+    FitFixed *fit_fixed = nullptr;
+    if constexpr (kFixedTransform<TK> && kPolyFamily<FAM>) {
+        __shared__ FitFixed s_fitq;
+        fit_fixed = &s_fitq;
+    }
     __shared__ int s_q;
     constexpr bool kCplx = FamilyAcc<FAM>::kComplex;
 
@@ -472,6 +484,8 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
         }
         for (int w = tid; w < (int)(sizeof(Integral) / 8); w += blockDim.x)
             reinterpret_cast<uint64_t *>(&s_item)[w] = reinterpret_cast<const uint64_t *>(src)[w];
+        if constexpr (kFixedTransform<TK> && kPolyFamily<FAM>)
+            if (tid == 0) fit_fixed->ok = 1;
         __syncthreads();
         const Integral &it = s_item;
         const int d = it.d;
@@ -482,6 +496,8 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
         for (int j = tid; j < d; j += blockDim.x) s_step.set(j, it.dc[j], it.n);
         stage_family<FAM, false>(it, fsh);
         prepare_fit(it.fit, d, s_fit);
+        if constexpr (kFixedTransform<TK> && kPolyFamily<FAM>)
+            for (int j = tid; it.fit && j < d; j += blockDim.x) fit_fixed->stage(it.fit, j);
         __syncthreads();
         if constexpr (kHasFixedForm<FAM>) {
             // the FP64 forms' subset-sum tables (256 FP64 sums per block), only when the
@@ -497,7 +513,7 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
         uint32_t cnt = 0;
         if (i0 < it.i_end) cnt = it.i_end - i0 < it.L ? (uint32_t)(it.i_end - i0) : it.L;
         StreamSum acc;
-        stream_sums<FAM, TK>(it, fsh, s_fit, it.fit != nullptr, Shifts{s_dsh + tid % m, m}, s_step, ws,
+        stream_sums<FAM, TK>(it, fsh, s_fit, (const FitFixed *)fit_fixed, it.fit != nullptr, Shifts{s_dsh + tid % m, m}, s_step, ws,
                              s_lat[tid >> 5], w0, cnt, acc);
         double *base = lp.partials + it.partial_off;
         tile_partial<kCplx>(acc, s_red, m, spb, base + 2 * (local * (uint64_t)m),
