@@ -23,21 +23,6 @@
 
 namespace qmc {
 
-// 2^127 / m for m in [2^63, 2^64), at most 2^-59 low: a single-precision estimate made slightly
-// low, r0 = 2^63 / m 2^32 (1 - e) with 0 < e < 2^-20, and r0 (1 + e + e^2).  (The estimate, the
-// conversion to single precision and two products err by less than 2^-21.6 in all.)
-__device__ __forceinline__ uint64_t recip_fixed(uint64_t m) {
-    const uint32_t mh = (uint32_t)(m >> 32), ml = (uint32_t)m;
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint2float_rn(mh)));
-    const uint32_t r0 = __float2uint_rz(r * (0x1p63f * (1.0f - 0x1p-21f)));   // below 2^32
-    // e 2^63 < 2^43, less one for the dropped fraction, so that R never exceeds 2^127 / m
-    const uint64_t E = 0x7FFFFFFFFFFFFFFFull - ((uint64_t)mh * r0 + __umulhi(ml, r0));
-    const uint32_t e22 = (uint32_t)(E >> 20);                                  // e 2^43
-    const uint64_t E2 = E + (((uint64_t)e22 * e22) >> 23);                     // (e + e^2) 2^63
-    return ((uint64_t)r0 << 32) + (((uint64_t)r0 * (uint32_t)E2) >> 31) + ((uint64_t)r0 * (uint32_t)(E2 >> 32) << 1);
-}
-
 struct FitFixed {
     struct Dim {
         uint64_t a0, b;              // a0 2^(64 - k0), b 2^(64 - k1)

@@ -163,37 +163,24 @@ __device__ __forceinline__ Fx fx_powi(Fx a, int p) {
     return r;
 }
 
-// 1/a for a normalized a = m 2^(e - 64): R = 2^127 / m (R < 2^64 for m > 2^63) by Newton's
-// iteration R <- R + R (2^127 - m R) 2^-127 from a single-precision seed (rcp.approx of
-// the top 32 bits, relative error ~2^-22), two steps (2^-44, then below 2^-61: at most 4
-// units low).  m within 2^32 of 2^63 takes the first-order value 2^64 - 2 (m - 2^63)
-// (exact to 4 units there), m = 2^63 the exact power of two.  The result may fall a few
-// units below 2^63; fx_to_double renormalizes.
-__device__ __forceinline__ Fx fx_recip(Fx a) {
-    const uint64_t m = a.m;
-    const uint32_t mh = (uint32_t)(m >> 32);
-    if (mh == 0x80000000u) {
-        const uint64_t dl = m - 0x8000000000000000ull;
-        if (!dl) return Fx{0x8000000000000000ull, 2 - a.e};
-        return Fx{0 - 2 * dl, 1 - a.e};
-    }
+// 2^127 / m for m in [2^63, 2^64), at most 2^-59 low: a single-precision estimate made slightly
+// low, r0 = 2^63 / m 2^32 (1 - e) with 0 < e < 2^-20, and r0 (1 + e + e^2).  (The estimate, the
+// conversion to single precision and two products err by less than 2^-21.6 in all.)
+__device__ __forceinline__ uint64_t recip_fixed(uint64_t m) {
+    const uint32_t mh = (uint32_t)(m >> 32), ml = (uint32_t)m;
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint2float_rn(mh)));
-    const uint32_t rb = __float_as_uint(r);                 // r = 2^E (1 + f), E = -32 or -31
-    const int E = (int)(rb >> 23) - 127;
-    const uint64_t mant = (uint64_t)((rb & 0x7FFFFFu) | 0x800000u);
-    uint64_t R = E >= -31 ? 0xFFFFFFFFFFFFFFFFull : mant << (72 + E);   // r 2^95
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const uint64_t plo = m * R, phi = __umul64hi(m, R);
-        // high word of 2^127 - m R (two's complement; |2^127 - m R| < 2^107)
-        const uint64_t ehi = 0x8000000000000000ull - phi - (plo != 0 ? 1ull : 0ull);
-        const bool neg = (long long)ehi < 0;
-        const uint64_t c = __umul64hi(R, neg ? 0 - ehi : ehi) << 1;
-        R = neg ? R - c : R + c;
-    }
-    return Fx{R, 1 - a.e};
+    const uint32_t r0 = __float2uint_rz(r * (0x1p63f * (1.0f - 0x1p-21f)));   // below 2^32
+    // e 2^63 < 2^43, less one for the dropped fraction, so that R never exceeds 2^127 / m
+    const uint64_t E = 0x7FFFFFFFFFFFFFFFull - ((uint64_t)mh * r0 + __umulhi(ml, r0));
+    const uint32_t e22 = (uint32_t)(E >> 20);                                  // e 2^43
+    const uint64_t E2 = E + (((uint64_t)e22 * e22) >> 23);                     // (e + e^2) 2^63
+    return ((uint64_t)r0 << 32) + (((uint64_t)r0 * (uint32_t)E2) >> 31) + ((uint64_t)r0 * (uint32_t)(E2 >> 32) << 1);
 }
+
+// 1/a for a normalized a = m 2^(e - 64), at most 2^-59 low (~25 instructions; two Newton steps
+// with full 64-bit products, to 2^-61, took ~60).
+__device__ __forceinline__ Fx fx_recip(Fx a) { return Fx{recip_fixed(a.m), 1 - a.e}; }
 
 // x 2^-64 for a 0.64 fixed-point x, rounded to nearest.
 __device__ __forceinline__ double fixed_to_double64(uint64_t x) {
@@ -371,15 +358,18 @@ __device__ __forceinline__ uint64_t korobov_odd_fixed(uint64_t X, Fx &Wp) {
     return (h ^ low) + 0x8000000000000000ull;
 }
 
-// Wp^E for a normalized Wp, normalized (binary powering).
+// Wp^E for a normalized Wp by binary powering.  Up to E = 4 the products stay unnormalized (at
+// least 2^61 of 2^64): the few bits lost are below 2^-59 of the value, and the result is
+// normalized once where it is used.
 template <int E>
 __device__ __forceinline__ Fx fx_pow(Fx Wp) {
     if constexpr (E == 1) {
         return Wp;
     } else {
-        const Fx h = fx_pow<E / 2>(Wp);
-        const Fx sq = fx_norm(fx_sq(h));
-        if constexpr (E % 2) return fx_norm(fx_mul(sq, Wp));
+        auto step = [](Fx v) { return E <= 4 ? v : fx_norm(v); };
+        const Fx h = step(fx_pow<E / 2>(Wp));
+        const Fx sq = step(fx_sq(h));
+        if constexpr (E % 2) return step(fx_mul(sq, Wp));
         else return sq;
     }
 }
@@ -388,7 +378,7 @@ __device__ __forceinline__ Fx fx_pow(Fx Wp) {
 // this many dimensions.
 template <int R>
 __device__ __forceinline__ Fx korobov_weight_fixed(Fx Wp, Fx cdx, int quarters = 0) {
-    Fx w = fx_norm(fx_mul(fx_pow<R>(Wp), cdx));
+    Fx w = fx_mul(fx_pow<R>(Wp), cdx);   // unnormalized, at least 2^59
     w.e -= 2 * R * quarters;
     return w;
 }
