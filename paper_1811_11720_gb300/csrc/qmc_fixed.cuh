@@ -303,6 +303,29 @@ __device__ __forceinline__ uint64_t korobov_gen_phi(uint64_t X, const TransformP
     return mulhi_trunc(pw, P) << (64 - t.kf);
 }
 
+// The same map for the separable families, which need phi absolutely but not relatively near 1:
+// phi = u^(r0+1) sum_(k <= r1) binom(r0+k, k) (1 - u)^k holds on all of [0, 1], so there are no
+// halves to choose between and r0 + r1 + 1 products instead of 2 max(r0, r1) + 1.  Every product
+// truncates downwards, so phi stays below 1.  kNorm as for korobov_odd_fixed.
+template <bool kNorm>
+__device__ __forceinline__ uint64_t korobov_gen_whole(uint64_t X, const TransformParams &t, Fx &Wu, Fx &W1) {
+    const uint64_t W = ~X;
+    const int r0 = t.r0, r1 = t.r1;
+    uint64_t P = t.KA[r1];
+#pragma unroll 1
+    for (int k = r1 - 1; k >= 0; --k) P = mulhi_trunc(P, W) + t.KA[k];
+    uint64_t pw = mulhi_trunc(X, P);   // u P, then the other r0 powers
+#pragma unroll 1
+    for (int q = 0; q < r0; ++q) pw = mulhi_trunc(pw, X);
+    Wu = fx_mul(Wu, Fx{X, 0});
+    W1 = fx_mul(W1, Fx{W, 0});
+    if constexpr (kNorm) {
+        Wu = fx_norm(Wu);
+        W1 = fx_norm(W1);
+    }
+    return pw << (64 - t.kf);
+}
+
 // C^d Wu^r0 W1^r1; cdx = C^d as Fx.
 __device__ __forceinline__ Fx korobov_gen_weight(Fx Wu, Fx W1, const TransformParams &t, Fx cdx) {
     return fx_norm(fx_mul(fx_norm(fx_mul(fx_powi(Wu, t.r0), fx_powi(W1, t.r1))), cdx));

@@ -124,13 +124,16 @@ constexpr bool kIntKorobov = TK == kTKorobovInt || TK == kTKorobovGen;
 template <int TK>
 constexpr bool kFixedTransform = TK == QMC_T_NONE || TK == QMC_T_BAKER || kIntKorobov<TK>;
 
-// kOdd: the form of Korobov<R,R> for the separable families (korobov_odd_fixed).
+// kOdd: the forms of the Korobov maps for the separable families (korobov_odd_fixed,
+// korobov_gen_whole).
 template <int TK, int R, bool kOdd = false, bool kNorm = true>
 __device__ __forceinline__ uint64_t transform_fixed(uint64_t X, const TransformParams &t, Weight &W) {
     if constexpr (TK == QMC_T_NONE) {
         return X;
     } else if constexpr (TK == QMC_T_BAKER) {
         return ((X >> 63) ? ~X : X) << 1;   // min(X, 2^64 - 1 - X) < 2^63
+    } else if constexpr (TK == kTKorobovGen && kOdd) {
+        return korobov_gen_whole<kNorm>(X, t, W.wp, W.wq);
     } else if constexpr (TK == kTKorobovGen) {
         const uint64_t F = korobov_gen_phi(X, t, W.wp, W.wq);
         return X >> 63 ? ~F : F;

@@ -95,3 +95,26 @@ def test_sums_against_the_oracle(r0, r1):
         if fam == "feynman":
             got, want = s[2 * m:4 * m].reshape(m, 2).sum(1), o["im"].sum(1)
             assert np.all(np.abs(got - want) <= 1e-12 * o["abs"])
+
+
+@pytest.mark.parametrize("r0,r1", ORDERS)
+def test_phi_on_the_whole_interval(r0, r1):
+    """The separable families' form: one polynomial on [0, 1], below 1.  The Horner products and
+    the r0 + 1 powers are at most 3 units of 2^-kf low each (the powers' losses are scaled by
+    u < 1), W one unit of 2^-64: at most 4 (r0 + r1 + 1) units."""
+    rng = random.Random(10 * r0 + r1)
+    deg = max(r0, r1)
+    kf = 63 - int(math.log2(math.comb(r0 + r1 + 1, deg)))
+    for X in [0, 1, M, M - 1, 1 << 63] + [rng.getrandbits(64) >> rng.choice([0, 0, 1, 9, 40]) for _ in range(200)] + \
+             [M ^ (rng.getrandbits(64) >> rng.choice([1, 9, 40])) for _ in range(100)]:
+        P = math.comb(r0 + r1, r1) << kf
+        for k in range(r1 - 1, -1, -1):
+            P = mulhi_trunc(P, M ^ X) + (math.comb(r0 + k, k) << kf)
+            assert P <= M
+        pw = mulhi_trunc(X, P)
+        for _ in range(r0):
+            pw = mulhi_trunc(pw, X)
+        assert pw < 1 << kf
+        u = Fr(X, 1 << 64)
+        exact = u ** (r0 + 1) * sum(math.comb(r0 + k, k) * (1 - u) ** k for k in range(r1 + 1))
+        assert 0 <= exact - Fr(pw, 1 << kf) <= Fr(4 * (r0 + r1 + 1), 1 << kf)
