@@ -31,12 +31,10 @@
 //   Ten FP64 instructions, within about 1 ulp; arguments outside [-708.3, 709] (where 2^m
 //   would leave the normal range) take the library exp.
 //
-// GB300 issues ~2 FP64 fused multiply-adds per clock per SM against ~32x as many integer
-// multiply-adds.  The integer form (~60 integer instructions for ~13 FP64 ones) pays when
-// the rest of the evaluation leaves the integer multiply pipe room (baker, none, Korobov up
-// to r = 3 for the exp families); under the higher Korobov orders that pipe is the
-// bottleneck and the FP64 form, on the otherwise idle FP64 pipe, is faster (the crossover
-// is FamilyAcc::kIntFinishMaxR).
+// GB300 issues ~2 FP64 fused multiply-adds per clock per SM against ~30x as many integer
+// multiply-adds: the integer form (~60 integer instructions for ~13 FP64 ones) serves every
+// fixed-point evaluation, the FP64 form those whose argument is a double (fitted rules,
+// parameters outside the fixed-point ranges), with half the FP64 work of the library exp.
 #pragma once
 #include <cstdint>
 

@@ -57,8 +57,7 @@ struct FixedForms {
     uint64_t t0;             // oscillatory: w_1 2^64 mod 2^64
     bool tk_any;             // oscillatory: some c_j >= 2 pi (a nonzero integer part)
     uint64_t one;            // 2^(2S - 64) (product peak)
-    double num;              // prod_j c_j^2 (product peak)
-    Fx numx;                 // the same as Fx (zero or normal)
+    Fx numx;                 // prod_j c_j^2 (product peak; zero or normal)
     int S;
     bool ok;
 };
@@ -92,12 +91,6 @@ template <int FAM>
 constexpr bool kHasFixedForm = FAM == QMC_GENZ_OSCILLATORY || FAM == QMC_GENZ_PRODUCT_PEAK ||
                                FAM == QMC_GENZ_CORNER_PEAK || FAM == QMC_GENZ_GAUSSIAN ||
                                FAM == QMC_GENZ_C0 || FAM == QMC_GENZ_DISCONTINUOUS;
-
-// v 2^-S for an integer v < 2^64, rounded once (the power of two is exact; v 2^-S is normal).
-__device__ __forceinline__ double scaled_fixed(uint64_t v, int S) {
-    const long long b = __double_as_longlong(__ull2double_rn(v));
-    return __longlong_as_double(b ? b - ((long long)S << 52) : 0ll);
-}
 
 // Per-thread staging of the fixed-point constants (threads tid < d; thread 0 writes S, ok).
 template <int FAM, class P>
@@ -158,7 +151,6 @@ __device__ __forceinline__ void stage_fixed_forms(const P &p, FixedForms &fx) {
             double num = 1.0;
             for (int i = 0; ok && i < p.d; ++i) num *= p.c[i] * p.c[i];
             ok = ok && (num == 0.0 || num >= 0x1p-1022);   // Fx takes zero or normal values
-            fx.num = num;
             fx.numx = fx_of_double(ok ? num : 0.0);
             fx.one = ok ? (1ull << (2 * S - 64)) + 1ull : 0ull;   // (and the square's mean loss)
         }
@@ -229,9 +221,12 @@ __device__ __forceinline__ void stage_family(const P &p, FamilyShared<FAM> &fs) 
 __device__ __forceinline__ uint64_t linear_loss(int d) { return (uint64_t)(d + (d >> 2)); }
 __device__ __forceinline__ uint64_t square_loss(int d) { return (uint64_t)(d + (d >> 1)); }
 
-// finish_fixed<kInt> forms the family's value as a double; where the integer finish is a positive
-// number in the format Fx (all but the oscillatory family), finish_fx gives that instead, so that
-// the weight joins it before the one rounding to double.
+// The fixed-point forms' value: finish_fx as a positive number in the format Fx, so that the weight
+// joins it before the one rounding to double, or finish_fixed as a double (the oscillatory family).
+// These integer finishes once gave way to FP64 ones under the higher Korobov orders; with the odd
+// map, the short reciprocal and two points at a time they are the faster ones up to d = 8 (1.8x at
+// d = 3, Korobov-3: 0.98 -> 0.59 ms for a corner peak at n = 1,072,187, m = 32) and at most 4 %
+// slower at d = 10, for every family and order.
 template <int FAM>
 struct FamilyAcc;
 template <int FAM>
@@ -248,7 +243,6 @@ __device__ __forceinline__ double reflected_c_sum(uint32_t mask, int d, const Se
 template <>
 struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
     static constexpr bool kComplex = false;
-    static constexpr int kIntFinishMaxR = 4;   // integer finish up to this Korobov order
     double s;
     uint32_t mask;
     __device__ __forceinline__ void init(const SeparableShared &fs) { s = fs.s0; mask = 0; }
@@ -261,25 +255,17 @@ struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
         re = cos(mask ? s + reflected_c_sum(mask, d, fs) : s);
         im = 0.0;
     }
-    // fixed point: sum c_j x_j on the integer pipe, either scaled by 2^S (then cos in FP64)
-    // or, for the integer finish, as the phase in turns mod 1 (FixedForms)
+    // fixed point: the phase in turns mod 1 (FixedForms)
     uint64_t sl;
     __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); }
-    template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
-        if constexpr (kInt) {
-            // the integer turns per unit x only when some c_j >= 2 pi (a uniform branch;
-            // the Genz ranges have ||c||_1 = 6)
-            if (fs.fx.tk_any) sl += x * fs.fx.tk[j];
-            sl += mulhi_trunc(x, fs.fx.tg[j]);
-        } else {
-            sl += mulhi_trunc(x, fs.fx.cl[j]);
-        }
+        // the integer turns per unit x only when some c_j >= 2 pi (a uniform branch; the Genz
+        // ranges have ||c||_1 = 6)
+        if (fs.fx.tk_any) sl += x * fs.fx.tk[j];
+        sl += mulhi_trunc(x, fs.fx.tg[j]);
     }
-    template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        if constexpr (kInt) re = cos_turns_fixed(sl + fs.fx.t0, fs.cos256);
-        else re = cos(fs.s0 + scaled_fixed(sl, fs.fx.S));
+    __device__ __forceinline__ double finish_fixed(const SeparableShared &fs) {
+        return cos_turns_fixed(sl + fs.fx.t0, fs.cos256);
     }
 };
 
@@ -287,7 +273,6 @@ struct FamilyAcc<QMC_GENZ_OSCILLATORY> {
 template <>
 struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
     static constexpr bool kComplex = false;
-    static constexpr int kIntFinishMaxR = 6;   // integer finish up to this Korobov order
     double prod;
     __device__ __forceinline__ void init(const SeparableShared &) { prod = 1.0; }
     __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
@@ -304,17 +289,12 @@ struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
     // 1 + q_j^2 at scale 2^(2S - 64) (below 2^64, at least 2^52), the product in Fx
     Fx pf;
     __device__ __forceinline__ void init_fixed(int) { pf = {0x8000000000000000ull, 1}; }
-    template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
         const uint64_t a = x >= w ? x - w : w - x;                       // |x - w| 2^64
         const uint64_t q = mulhi_trunc(a, fs.fx.cq[j]);                 // c |x - w| 2^S
         const uint64_t s = fs.fx.one + sqhi_trunc(q);               // (1 + q^2) 2^(2S-64)
         pf = fx_norm(fx_mul(pf, Fx{s, 128 - 2 * fs.fx.S}));
-    }
-    template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        re = fs.fx.num / fx_to_double(pf);
     }
     // prod c_j^2 times the reciprocal of the product (Newton on the integer pipe)
     __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
@@ -326,7 +306,6 @@ struct FamilyAcc<QMC_GENZ_PRODUCT_PEAK> {
 template <>
 struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
     static constexpr bool kComplex = false;
-    static constexpr int kIntFinishMaxR = 1;   // integer finish up to this Korobov order
     double s;
     uint32_t mask;
     __device__ __forceinline__ void init(const SeparableShared &) { s = 1.0; mask = 0; }
@@ -342,13 +321,8 @@ struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
     }
     uint64_t sl;
     __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); }
-    template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         sl += mulhi_trunc(x, fs.fx.cl[j]);
-    }
-    template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int d, const SeparableShared &fs, double &re) {
-        re = 1.0 / ipow_u(1.0 + scaled_fixed(sl, fs.fx.S), d + 1);
     }
     __device__ __forceinline__ Fx finish_fx(int d, const SeparableShared &fs) {
         // 1 + s as Fx (s = sl 2^-S, sl < 2^63; S = 64 drops sl's lowest bit), its (d+1)-th
@@ -364,7 +338,6 @@ struct FamilyAcc<QMC_GENZ_CORNER_PEAK> {
 template <>
 struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
     static constexpr bool kComplex = false;
-    static constexpr int kIntFinishMaxR = 3;   // integer finish up to this Korobov order
     double s;
     __device__ __forceinline__ void init(const SeparableShared &) { s = 0.0; }
     __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
@@ -372,24 +345,19 @@ struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
         const double q = fma(m.refl ? -fs.c[j] : fs.c[j], m.y, m.refl ? fs.c1w[j] : fs.mcw[j]);
         s = fma(q, q, s);
     }
-    __device__ __forceinline__ void finish(int, const SeparableShared &, double &re, double &im,
+    __device__ __forceinline__ void finish(int, const SeparableShared &fs, double &re, double &im,
                                            unsigned long long &) {
-        re = exp(-s);
+        re = exp_table(-s, fs.exp2t);
         im = 0.0;
     }
     // fixed point: q = c |x - w| 2^S < 2^62, q^2 2^(2S - 64) < 2^60, summed in 64 bits
     uint64_t sq;
     __device__ __forceinline__ void init_fixed(int d) { sq = square_loss(d); }
-    template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
         const uint64_t a = x >= w ? x - w : w - x;                       // |x - w| 2^64
         const uint64_t q = mulhi_trunc(a, fs.fx.cq[j]);                 // c |x - w| 2^S
         sq += sqhi_trunc(q);
-    }
-    template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        re = exp_table(-scaled_fixed(sq, 2 * fs.fx.S - 64), fs.exp2t);
     }
     __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
         return exp_fixed(sq, 2 * fs.fx.S - 64, true, fs.exp2q);
@@ -400,29 +368,23 @@ struct FamilyAcc<QMC_GENZ_GAUSSIAN> {
 template <>
 struct FamilyAcc<QMC_GENZ_C0> {
     static constexpr bool kComplex = false;
-    static constexpr int kIntFinishMaxR = 3;   // integer finish up to this Korobov order
     double s;
     __device__ __forceinline__ void init(const SeparableShared &) { s = 0.0; }
     __device__ __forceinline__ void add(int j, const Mapped &m, const SeparableShared &fs) {
         double t = m.refl ? fs.w1[j] - m.y : m.y - fs.w[j];
         s = fma(fs.c[j], fabs(t), s);
     }
-    __device__ __forceinline__ void finish(int, const SeparableShared &, double &re, double &im,
+    __device__ __forceinline__ void finish(int, const SeparableShared &fs, double &re, double &im,
                                            unsigned long long &) {
-        re = exp(-s);
+        re = exp_table(-s, fs.exp2t);
         im = 0.0;
     }
     uint64_t sl;
     __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); }
-    template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         const uint64_t w = fs.fx.w64[j];
         const uint64_t a = x >= w ? x - w : w - x;                       // |x - w| 2^64
         sl += mulhi_trunc(a, fs.fx.cl[j]);
-    }
-    template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        re = exp_table(-scaled_fixed(sl, fs.fx.S), fs.exp2t);
     }
     __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
         return exp_fixed(sl, fs.fx.S, true, fs.exp2q);
@@ -433,7 +395,6 @@ struct FamilyAcc<QMC_GENZ_C0> {
 template <>
 struct FamilyAcc<QMC_GENZ_DISCONTINUOUS> {
     static constexpr bool kComplex = false;
-    static constexpr int kIntFinishMaxR = 3;   // integer finish up to this Korobov order
     double s;
     uint32_t mask;
     bool zero;
@@ -447,19 +408,14 @@ struct FamilyAcc<QMC_GENZ_DISCONTINUOUS> {
     }
     __device__ __forceinline__ void finish(int d, const SeparableShared &fs, double &re, double &im,
                                            unsigned long long &) {
-        re = zero ? 0.0 : exp(mask ? s + reflected_c_sum(mask, d, fs) : s);
+        re = zero ? 0.0 : exp_table(mask ? s + reflected_c_sum(mask, d, fs) : s, fs.exp2t);
         im = 0.0;
     }
     uint64_t sl;
     __device__ __forceinline__ void init_fixed(int d) { sl = linear_loss(d); zero = false; }
-    template <bool kInt>
     __device__ __forceinline__ void add_fixed(int j, uint64_t x, const SeparableShared &fs) {
         if (j < 2) zero |= x > fs.fx.w64[j];
         sl += mulhi_trunc(x, fs.fx.cl[j]);
-    }
-    template <bool kInt>
-    __device__ __forceinline__ void finish_fixed(int, const SeparableShared &fs, double &re) {
-        re = zero ? 0.0 : exp_table(scaled_fixed(sl, fs.fx.S), fs.exp2t);
     }
     __device__ __forceinline__ Fx finish_fx(int, const SeparableShared &fs) {
         Fx f = exp_fixed(sl, fs.fx.S, false, fs.exp2q);

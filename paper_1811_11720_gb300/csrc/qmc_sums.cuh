@@ -153,12 +153,6 @@ struct Shifts {
 template <int FAM, int TK, int R, int NP, class St>
 __device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableShared &fsh, Shifts dsh,
                                            double cd, const St (&st)[NP], double (&g)[NP]) {
-    // the final function (exp, power, cos) on the integer pipe where the map leaves it room;
-    // under the higher Korobov orders the integer multiply pipe is the bottleneck and the FP64
-    // form, on the otherwise idle FP64 pipe, is faster (the crossover order per family was
-    // measured)
-    constexpr bool kIntFinish = !kIntKorobov<TK> ||
-                                (TK == kTKorobovInt && R <= FamilyAcc<FAM>::kIntFinishMaxR);
     Weight W[NP];
     FamilyAcc<FAM> fa[NP];
 #pragma unroll
@@ -167,8 +161,8 @@ __device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableSha
         const uint64_t D = dsh(j);
 #pragma unroll
         for (int u = 0; u < NP; ++u)
-            fa[u].template add_fixed<kIntFinish>(
-                j, transform_fixed<TK, R, true, decltype(norm)::value>(st[u].hi(j) + D, p.t, W[u]), fsh);
+            fa[u].add_fixed(j, transform_fixed<TK, R, true, decltype(norm)::value>(st[u].hi(j) + D, p.t, W[u]),
+                            fsh);
     };
     if constexpr (TK == kTKorobovInt) {
         // pairs of dimensions: the weight's product is renormalized once a pair
@@ -185,13 +179,12 @@ __device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableSha
     }
 #pragma unroll
     for (int u = 0; u < NP; ++u) {
-        if constexpr (kIntFinish && kFxFinish<FAM>) {
+        if constexpr (kFxFinish<FAM>) {
             Fx f = fa[u].finish_fx(p.d, fsh);
             if constexpr (kIntKorobov<TK>) f = fx_mul(f, weight_fx<TK, R>(W[u], p.t, cd, p.d));
             g[u] = fx_to_double_sat(fx_norm(f));
         } else {
-            fa[u].template finish_fixed<kIntFinish>(p.d, fsh, g[u]);
-            g[u] *= weight_finish<TK, R>(W[u], p.t, cd, p.d);
+            g[u] = fa[u].finish_fixed(fsh) * weight_finish<TK, R>(W[u], p.t, cd, p.d);
         }
     }
 }
