@@ -12,6 +12,13 @@ static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s
     const uint64_t tiles = lp.end_tile - lp.first_tile;
     const uint64_t grid = tiles < 0x7FFFFFFFull ? tiles : 0x7FFFFFFFull;
     const size_t smem = sizeof(uint64_t) * max_d * lp.m;
+    // static and dynamic shared memory together exceed the 48 KB that need no opting in for many
+    // shifts and dimensions (the static part is at most 46.2 KB)
+    if (smem > 2048) {
+        const cudaError_t e = cudaFuncSetAttribute(lattice_kernel<FAM, TK, MINB>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     lattice_kernel<FAM, TK, MINB><<<(unsigned)grid, lp.spb * lp.m, smem, s>>>(lp);
     return cudaGetLastError();
 }
