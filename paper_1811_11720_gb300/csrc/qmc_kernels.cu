@@ -43,13 +43,14 @@ __global__ void __launch_bounds__(kPointThreads) points_kernel(const __grid_cons
     const uint64_t i0 = p.i_begin + off, rows = (uint64_t)p.rows;
     lattice_state_at(i0, c, n, fh, fl, rem);
     if constexpr (kShort) {
-        DimConst step;   // `rows` steps at once
-        lattice_state_at(rows, c, n, step.fz_hi, step.fz_lo, step.rq);
-        step.rq = step.rq ? rows * c.rq : 0;   // (a whole number of periods leaves none)
-        ShortState s{fh, fl, i0 * c.rq};
+        const uint64_t w = short_step_word(c, n);
+        LatticeStep step;   // `rows` steps at once
+        lattice_state_at(rows, c, n, step.fz_hi, step.fz_lo, step.remz);
+        const uint64_t step_w = rows * w;
+        ShortState s{fh, fl, i0 * w};
         for (uint32_t q = 0; q < cnt; ++q) {
             __stcs(o, fixed_to_double(s.f_hi + dsh, s.f_lo, n));
-            s.step(step.fz_hi, step.fz_lo, step.rq);
+            s.step(step.fz_hi, step.fz_lo, step_w);
             o += stride;
         }
     } else {

@@ -94,12 +94,16 @@ __device__ __forceinline__ void lattice_step(const LatticeStep &c, uint64_t n, u
 }
 
 // The same step for n < 2^32: the fraction is carried to 192 bits, started with the third
-// word i rq mod 2^64 and stepped by one long addition, without an exact remainder.  The third
-// word is low by less than i units, so a carry out of it can be missed only where the true
-// fraction of a unit of 2^-128, rem / n, is below i / 2^64 < 1 / n: only for rem = 0, at
-// multiples of n, and a stream of points 0 <= i < n steps to none (it may start at i = 0,
-// where all three words are exact).
+// word i w mod 2^64 and stepped by one long addition of w = ceil(remz 2^64 / n), without an
+// exact remainder.  After i steps the third word is high by less than i units.  So no carry out
+// of it is missed, and none is spurious: that would take a true fraction of a unit of 2^-128,
+// rem / n <= 1 - 1/n, above 1 - i / 2^64, and i < n < 2^32.  (Rounded down it would be low, and
+// miss the carry wherever rem(i) = 0: at multiples of n's odd part, inside the lattice of an
+// even n that is no power of two.)
 constexpr int kShortBits = 32;
+__device__ __forceinline__ uint64_t short_step_word(const DimConst &c, uint64_t n) {
+    return c.rq + (c.rq * n != 0);   // remz 2^64 mod n = -rq n modulo 2^64
+}
 struct ShortState {
     uint64_t f_hi, f_lo, f_2;
     __device__ __forceinline__ void step(uint64_t z_hi, uint64_t z_lo, uint64_t z_2) {

@@ -95,19 +95,19 @@ template <int TK>
 constexpr bool kTopWordOnly = kIntKorobov<TK>;
 
 // The step constants of the d coordinates in shared memory (a warp's lanes read different j).
-// z2: the third fraction word for n < 2^32 (ShortState), else the exact remainder.
+// z2: the third word's step for n < 2^32 (ShortState), else the exact remainder.
 struct BlockSteps {
     uint64_t zh[kMaxDim], zl[kMaxDim], z2[kMaxDim];
     __device__ __forceinline__ void set(int j, const DimConst &c, uint64_t n) {
         const LatticeStep st = lattice_step_of(c, n);
         zh[j] = st.fz_hi;
         zl[j] = st.fz_lo;
-        z2[j] = n >> kShortBits ? st.remz : c.rq;
+        z2[j] = n >> kShortBits ? st.remz : short_step_word(c, n);
     }
     __device__ __forceinline__ void start(int j, uint64_t i, const DimConst &c, uint64_t n,
                                           ShortState &s) const {
         lattice_state_at(i, c, n, s.f_hi, s.f_lo, s.f_2);
-        if (!(n >> kShortBits)) s.f_2 = i * c.rq;
+        if (!(n >> kShortBits)) s.f_2 = i * z2[j];
     }
     __device__ __forceinline__ void step(int j, uint64_t n, ShortState &s) const {
         if (n >> kShortBits) lattice_step(LatticeStep{zh[j], zl[j], z2[j]}, n, s.f_hi, s.f_lo, s.f_2);
