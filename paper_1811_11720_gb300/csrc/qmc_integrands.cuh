@@ -92,7 +92,8 @@ constexpr bool kHasFixedForm = FAM == QMC_GENZ_OSCILLATORY || FAM == QMC_GENZ_PR
                                FAM == QMC_GENZ_CORNER_PEAK || FAM == QMC_GENZ_GAUSSIAN ||
                                FAM == QMC_GENZ_C0 || FAM == QMC_GENZ_DISCONTINUOUS;
 
-// Per-thread staging of the fixed-point constants (threads tid < d; thread 0 writes S, ok).
+// Staging of the fixed-point constants, thread t's dimensions t, t + blockDim, ... (a block may
+// have fewer threads than dimensions); thread 0 writes S, ok.
 template <int FAM, class P>
 __device__ __forceinline__ void stage_fixed_forms(const P &p, FixedForms &fx) {
     const int tid = threadIdx.x;
@@ -118,12 +119,12 @@ __device__ __forceinline__ void stage_fixed_forms(const P &p, FixedForms &fx) {
         S = csum > 0.0 ? min(62 - ilogb(csum), 64) : 64;
     }
     ok = ok && S >= 2;
-    if (ok) {
-        const double c = p.c[tid];
-        const double w = p.w ? p.w[tid] : 0.0;
-        fx.cl[tid] = __double2ull_rz(ldexp(c, S));
-        fx.cq[tid] = __double2ull_rz(ldexp(c, S));
-        fx.w64[tid] = w >= 1.0 ? 0xFFFFFFFFFFFFFFFFull : __double2ull_rz(ldexp(w, 64));
+    for (int j = tid; ok && j < p.d; j += blockDim.x) {
+        const double c = p.c[j];
+        const double w = p.w ? p.w[j] : 0.0;
+        fx.cl[j] = __double2ull_rz(ldexp(c, S));
+        fx.cq[j] = __double2ull_rz(ldexp(c, S));
+        fx.w64[j] = w >= 1.0 ? 0xFFFFFFFFFFFFFFFFull : __double2ull_rz(ldexp(w, 64));
         if constexpr (FAM == QMC_GENZ_OSCILLATORY) {
             // c / (2 pi) = hi + lo (double-double), then integer part and 64-bit fraction
             constexpr double kInv2PiHi = 0x1.45f306dc9c883p-3;
@@ -137,8 +138,8 @@ __device__ __forceinline__ void stage_fixed_forms(const P &p, FixedForms &fx) {
             // a carry out of (or borrow into) the fraction moves the integer part
             if (g_lo < 0 && g > __double2ull_rz(ldexp(f, 64))) k -= 1.0;
             if (g_lo > 0 && g < __double2ull_rz(ldexp(f, 64))) k += 1.0;
-            fx.tg[tid] = g;
-            fx.tk[tid] = (uint64_t)(long long)k;
+            fx.tg[j] = g;
+            fx.tk[j] = (uint64_t)(long long)k;
         }
     }
     if (tid == 0) {
@@ -188,16 +189,16 @@ __device__ __forceinline__ void stage_family(const P &p, FamilyShared<FAM> &fs) 
     if constexpr (kPolyFamily<FAM>) {
         stage_poly(p, fs.poly, FAM == QMC_SECTOR);
     } else {
-        if (tid < p.d) {
-            double c = p.c ? p.c[tid] : 0.0;
-            double w = p.w ? p.w[tid] : 0.0;
-            fs.c[tid] = c;
-            fs.w[tid] = w;
-            fs.mcw[tid] = -(c * w);
-            fs.c1w[tid] = c * (1.0 - w);
-            fs.w1[tid] = 1.0 - w;
-            if constexpr (FAM == QMC_GENZ_PRODUCT_PEAK) fs.aux[tid] = 1.0 / (c * c);
-            fs.h[tid] = p.h ? p.h[tid] : 0;
+        for (int j = tid; j < p.d; j += blockDim.x) {
+            double c = p.c ? p.c[j] : 0.0;
+            double w = p.w ? p.w[j] : 0.0;
+            fs.c[j] = c;
+            fs.w[j] = w;
+            fs.mcw[j] = -(c * w);
+            fs.c1w[j] = c * (1.0 - w);
+            fs.w1[j] = 1.0 - w;
+            if constexpr (FAM == QMC_GENZ_PRODUCT_PEAK) fs.aux[j] = 1.0 / (c * c);
+            fs.h[j] = p.h ? p.h[j] : 0;
         }
         if (tid == 0) fs.s0 = (FAM == QMC_GENZ_OSCILLATORY && p.w) ? 6.283185307179586476925 * p.w[0] : 0.0;
         if constexpr (kSubsets) stage_subset_sums<FAM>(p, fs);
