@@ -13,10 +13,13 @@ static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s
     const uint64_t grid = tiles < 0x7FFFFFFFull ? tiles : 0x7FFFFFFFull;
     const size_t smem = sizeof(uint64_t) * max_d * lp.m;
     // static and dynamic shared memory together exceed the 48 KB that need no opting in for many
-    // shifts and dimensions (the static part is at most 46.2 KB)
+    // shifts and dimensions (the static part is at most 46,160 bytes).  The limit is state of the
+    // function that all threads share: always the largest table's size, so that no call lowers it
+    // under another one's launch.
     if (smem > 2048) {
         const cudaError_t e = cudaFuncSetAttribute(lattice_kernel<FAM, TK, MINB>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)sizeof(uint64_t) * kMaxDim * kSumsThreads);
         if (e != cudaSuccess) return e;
     }
     lattice_kernel<FAM, TK, MINB><<<(unsigned)grid, lp.spb * lp.m, smem, s>>>(lp);
