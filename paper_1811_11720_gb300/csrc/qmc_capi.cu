@@ -282,7 +282,7 @@ int qmc_histogram(const qmc_integrand *f, uint64_t n, const uint64_t *z, int dim
     if (!z || !shift || !hist || !workspace) return QMC_ERR_ARG;
     if (dim != f->dim) return QMC_ERR_DIM;
     if (n < 2 || n >= kNMax) return QMC_ERR_N;
-    if (bins < 1 || (size_t)dim * bins > 20480) return QMC_ERR_RANGE;
+    if (bins < 1 || (size_t)dim * bins > kHistCells) return QMC_ERR_RANGE;
     for (int j = 0; j < dim; ++j)
         if (z[j] % n == 0 || gcd_u64(z[j] % n, n) != 1) return QMC_ERR_GENVEC;
     // a smaller workspace, down to one block per 4096 points, takes fewer and longer blocks

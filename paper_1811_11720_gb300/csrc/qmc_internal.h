@@ -37,6 +37,7 @@ cudaError_t launch_finalize(const double *sums, int m, uint64_t n, int is_comple
                             double *result, double *Q, cudaStream_t s);
 
 cudaError_t launch_evaluate(int family, const Integral &p, double *out, cudaStream_t s);
+constexpr int kHistCells = 20480;   // most dim * bins: 160 KB of shared memory
 cudaError_t launch_histogram(int family, const Integral &p, int bins, double *hist, double *work,
                              uint32_t nblocks, cudaStream_t s);
 

@@ -321,9 +321,11 @@ static cudaError_t eval_dispatch_one(const Integral &p, double *out, cudaStream_
 template <int FAM>
 static cudaError_t hist_dispatch_one(const Integral &p, int bins, double *hist, double *work,
                                      uint32_t nblocks, cudaStream_t s) {
-    size_t smem = (size_t)p.d * bins * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(histogram_kernel<FAM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is state of the function that all threads share: always the largest histogram's
+    // size, so that no call lowers it under another one's launch
+    const size_t smem = (size_t)p.d * bins * sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(histogram_kernel<FAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kHistCells * sizeof(double)));
     if (e != cudaSuccess) return e;
     histogram_kernel<FAM><<<nblocks, kHistThreads, smem, s>>>(p, bins, work);
     e = cudaGetLastError();

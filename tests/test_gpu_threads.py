@@ -54,3 +54,27 @@ def test_sums_from_several_threads(fam, shapes):
     torch.cuda.synchronize()
     for out, want in checks:
         assert torch.equal(out, want)
+
+
+def test_histograms_from_several_threads():
+    import torch
+
+    import paper_1811_11720_gb300 as q
+    import workloads as W
+    n = 257
+    workers, checks = [], []
+    for d, bins in [(16, 1280), (4, 100), (8, 1000)]:
+        f = q.Integrand.genz(4, *W.genz_params(4, d, 1)).device_struct("cuda")
+        sh = torch.from_numpy(q.make_shifts(d, 1, d)[0].astype(np.int64)).cuda()
+        z = np.array([v * 2 + 1 for v in range(d)], dtype=np.uint64)
+        ws = torch.empty(q.histogram_workspace_bytes(n, d, bins), dtype=torch.uint8, device="cuda")
+        out, want = (torch.zeros(d, bins, dtype=torch.float64, device="cuda") for _ in range(2))
+        q.histogram(f, n, z, sh, bins, want, ws)
+        torch.cuda.synchronize()
+        stream = torch.cuda.Stream()
+        workers.append(lambda a=(f, n, z, sh, bins, out, ws), s=stream: q.histogram(*a, stream=s))
+        checks.append((out, want))
+    _run(workers, 2000)
+    torch.cuda.synchronize()
+    for out, want in checks:
+        assert torch.equal(out, want)
