@@ -288,9 +288,9 @@ __device__ __forceinline__ uint64_t korobov_gen_phi(uint64_t X, const TransformP
                                                     Fx &W1) {
     const bool lo = !(X >> 63);
     const uint64_t V = lo ? X : ~X, W = ~V;
-    uint64_t P = lo ? t.KA[t.deg] : t.KB[t.deg];
+    uint64_t P = lo ? t.KA[t.deg] : (uint64_t)t.KB[t.deg] << t.kf;
 #pragma unroll 1
-    for (int k = t.deg - 1; k >= 0; --k) P = mulhi_trunc(P, W) + (lo ? t.KA[k] : t.KB[k]);
+    for (int k = t.deg - 1; k >= 0; --k) P = mulhi_trunc(P, W) + (lo ? t.KA[k] : (uint64_t)t.KB[k] << t.kf);
     const int e = lo ? t.r0 : t.r1;   // v^(e + 1)
     uint64_t pw = V;
 #pragma unroll 1

@@ -76,12 +76,10 @@ inline TransformParams make_transform(const qmc_transform &t) {
         if (r0 != r1 && std::min(r0, r1) >= 1 && tp.deg <= kMaxKorobovInt) {
             // so has the asymmetric map; the largest partial sum is binom(r0+r1+1, max)
             tp.kind = kTKorobovGen;
-            std::memset(tp.A, 0, sizeof(tp.A));
-            std::memset(tp.B, 0, sizeof(tp.B));
             const double top = std::max(binom(r0 + r1 + 1, r0), binom(r0 + r1 + 1, r1));
-            tp.kf = 63 - std::ilogb(top);   // top 2^kf < 2^64
+            tp.kf = (uint8_t)(63 - std::ilogb(top));   // top 2^kf < 2^64
             for (int k = 0; k <= r1; ++k) tp.KA[k] = (uint64_t)std::llround(binom(r0 + k, k)) << tp.kf;
-            for (int k = 0; k <= r0; ++k) tp.KB[k] = (uint64_t)std::llround(binom(r1 + k, k)) << tp.kf;
+            for (int k = 0; k <= r0; ++k) tp.KB[k] = (uint16_t)std::llround(binom(r1 + k, k));
         }
     } else if (t.kind == QMC_T_SIDI) {
         const int r = t.r0;

@@ -26,19 +26,17 @@ constexpr int kTKorobovGen = 5;
 // (B: r0 and r1 exchanged).  The weight is C u^r0 (1-u)^r1, C = (r0+r1+1) binom(r0+r1,r0).
 struct TransformParams {
     int kind, r0, r1, deg;        // deg = max(r0, r1): Horner length (zero-padded)
+    double A[kMaxKorobov + 1];
+    double B[kMaxKorobov + 1];
+    double C;                     // Korobov constant, or Sidi (pi/2^r) Gamma(r+1)/Gamma((r+1)/2)^2
     union {
-        struct {
-            double A[kMaxKorobov + 1];
-            double B[kMaxKorobov + 1];
-        };
-        struct {   // kTKorobovGen: binom(r0 + k, k) 2^kf and binom(r1 + k, k) 2^kf, k <= deg
+        double sidi_c[kMaxSidi + 1];  // Sidi: phi = cr * I_r, I_r via the sin-power reduction
+        struct {   // kTKorobovGen: binom(r0 + k, k) 2^kf, and binom(r1 + k, k) by itself, k <= deg
             uint64_t KA[kMaxKorobovInt + 1];
-            uint64_t KB[kMaxKorobovInt + 1];
-            int kf;
+            uint16_t KB[kMaxKorobovInt + 1];
+            uint8_t kf;
         };
     };
-    double C;                     // Korobov constant, or Sidi (pi/2^r) Gamma(r+1)/Gamma((r+1)/2)^2
-    double sidi_c[kMaxSidi + 1];  // Sidi: phi = cr * I_r, I_r via the sin-power reduction
 };
 
 // One integral as the kernels see it: of a launch of its own (passed as a kernel parameter)

@@ -89,10 +89,10 @@ __device__ __forceinline__ WarpStreams warp_streams(int m) {
     return w;
 }
 
-// Words of the state that a transform reads: the maps that take the coordinate as x 2^64
-// read the top word, the others round both to u.
+// Words of the state that a transform reads: Korobov<r,r> takes the coordinate as x 2^64 and
+// reads the top word, the others (may) round both to u.
 template <int TK>
-constexpr bool kTopWordOnly = kIntKorobov<TK>;
+constexpr bool kTopWordOnly = TK == kTKorobovInt;
 
 // The step constants of the d coordinates in shared memory (a warp's lanes read different j).
 // z2: the third word's step for n < 2^32 (ShortState), else the exact remainder.
@@ -189,6 +189,17 @@ __device__ __forceinline__ void eval_fixed(const Integral &p, const SeparableSha
     }
 }
 
+// Whether the fixed-point form serves the integrand under the transform (uniform over the
+// block).  The asymmetric map in FP64 keeps x relative near its ends, the integer one is absolute
+// (~2^-57): a corner peak, or a C0 peak at w = 0, of large coefficients lives near x = 0 and needs
+// sum c < 32 (S >= 58) there.  (A corner peak of d = 1 under Korobov<1,3> with c = 1e3, 1e6, 1e8
+// was 1e-15, 1.5e-12, 2.7e-10 off on integers, 4e-16 in FP64; at c = 31 both 2e-16.)
+template <int FAM, int TK>
+__device__ __forceinline__ bool fixed_form_ok(const FixedForms &fx) {
+    constexpr bool kSharp = TK == kTKorobovGen && (FAM == QMC_GENZ_CORNER_PEAK || FAM == QMC_GENZ_C0);
+    return fx.ok && (!kSharp || fx.S >= 58);
+}
+
 // One evaluation of g at a point with lattice state `st`.
 template <int FAM, int TK, int R, class St>
 __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared<FAM> &fsh,
@@ -197,12 +208,15 @@ __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared
                                            unsigned long long &signfail) {
     Weight W;
     FamilyAcc<FAM> fa;
+    constexpr bool kGen = TK == kTKorobovGen;
     if constexpr (kFixedTransform<TK> && kPolyFamily<FAM>) {
         // the polynomial families' fixed-point forms take the coordinates as x 2^64 from the
-        // integer-pipe transform, through the integer fit map where there is one
+        // integer-pipe transform, through the integer fit map where there is one; from the
+        // asymmetric map only where both polynomials are in fixed point (x is then absolute to
+        // ~2^-57, and in FP64, where it is relative near 0, it may be raised to any power)
         bool fixed = !use_fit || fit_fixed->ok;
-        if constexpr (FAM == QMC_SECTOR) fixed = fixed && sector_fixed_ok(fsh.poly, p.d);
-        else fixed = fixed && feyn_fixed_ok(fsh.poly, p.d);
+        if constexpr (FAM == QMC_SECTOR) fixed = fixed && sector_fixed_ok(fsh.poly, p.d) && (!kGen || fsh.poly.fixed_u);
+        else fixed = fixed && feyn_fixed_ok(fsh.poly, p.d) && (!kGen || fsh.poly.feyn_full);
         if (fixed) {   // uniform over the block
             Weight V;
             Fx J;
@@ -229,11 +243,16 @@ __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared
             }
         }
     }
+    // the asymmetric map in FP64, relative near its ends
+    bool rel = kGen && kPolyFamily<FAM>;
+    if constexpr (kGen && kHasFixedForm<FAM>) rel = !fixed_form_ok<FAM, TK>(fsh.fx);
     fa.init(fsh);
 #pragma unroll 1
     for (int j = 0; j < p.d; ++j) {
         Mapped mx;
-        if constexpr (kIntKorobov<TK> && kPolyFamily<FAM>) {
+        if (kGen && rel) {
+            mx = apply_transform<QMC_T_KOROBOV>(fixed_to_double(st.hi(j) + dsh(j), st.lo(j), p.n), p.t, W);
+        } else if constexpr (kIntKorobov<TK> && kPolyFamily<FAM>) {
             // the polynomial families use x itself: formed from x 2^64 by integer
             // operations instead of an FP64 conversion and reflection
             mx = Mapped{fixed_u64_to_double(transform_fixed<TK, R>(st.hi(j) + dsh(j), p.t, W), 64), false};
@@ -246,7 +265,7 @@ __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared
         if (use_fit) mx = Mapped{apply_fit(reflected(mx), s_fit + kFitStride * j, W.w), false};
         fa.add(j, mx, fsh);
     }
-    const double wt = weight_finish<TK, R>(W, p.t, cd);
+    const double wt = kGen && rel ? weight_finish<QMC_T_KOROBOV>(W, p.t, cd) : weight_finish<TK, R>(W, p.t, cd);
     fa.finish(p.d, fsh, g_re, g_im, signfail);
     g_re *= wt;
     if constexpr (FamilyAcc<FAM>::kComplex) g_im *= wt;
@@ -381,7 +400,7 @@ __device__ __forceinline__ void stream_sums_r(const Integral &p, const FamilySha
     constexpr bool kCplx = FamilyAcc<FAM>::kComplex;
     const double cd = p.cd;
     if constexpr (kFixedTransform<TK> && kHasFixedForm<FAM>) {
-        if (!use_fit && fsh.fx.ok) {   // uniform over the block
+        if (!use_fit && fixed_form_ok<FAM, TK>(fsh.fx)) {   // uniform over the block
             // The tail of its own pays under Korobov<r,r> (streams of 9 points, the d = 4, n =
             // 108,863, m = 16 integral's: 75.8 -> 71.7 us); under baker and the asymmetric map
             // the second copy of the code cost 1 and 3 %.
@@ -517,7 +536,7 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
         if constexpr (kHasFixedForm<FAM>) {
             // the FP64 forms' subset-sum tables (256 FP64 sums per block), only when the
             // fixed-point form does not take every evaluation (uniform over the block)
-            if (!(kFixedTransform<TK> && it.fit == nullptr && fsh.fx.ok)) {
+            if (!(kFixedTransform<TK> && it.fit == nullptr && fixed_form_ok<FAM, TK>(fsh.fx))) {
                 stage_subset_sums<FAM>(it, fsh);
                 __syncthreads();
             }
