@@ -306,7 +306,12 @@ __device__ __forceinline__ uint64_t korobov_gen_phi(uint64_t X, const TransformP
 // The same map for the separable families, which need phi absolutely but not relatively near 1:
 // phi = u^(r0+1) sum_(k <= r1) binom(r0+k, k) (1 - u)^k holds on all of [0, 1], so there are no
 // halves to choose between and r0 + r1 + 1 products instead of 2 max(r0, r1) + 1.  Every product
-// truncates downwards, so phi stays below 1.  kNorm as for korobov_odd_fixed.
+// truncates downwards, so phi stays below 1; the power is formed by itself at 2^-64 and meets P in
+// the last product, the one power that truncates at 2^-kf.  On average phi is 1.7 units of 2^-54 low
+// under the orders 5 and 6 (kf = 54; 0.04 at 1 and 3), where the FP64 form errs by 6 (0.7) either way;
+// with P in the chain from the first power on it was 3.5 low, and a C0 or corner peak under the orders
+// 5 and 6 up to four times as far off as in FP64.  (Setting the bits below 2^-kf would make up one
+// more unit; at d = 8, n = 256,687, m = 20 it cost 2 %.)  kNorm as for korobov_odd_fixed.
 template <bool kNorm>
 __device__ __forceinline__ uint64_t korobov_gen_whole(uint64_t X, const TransformParams &t, Fx &Wu, Fx &W1) {
     const uint64_t W = ~X;
@@ -314,7 +319,7 @@ __device__ __forceinline__ uint64_t korobov_gen_whole(uint64_t X, const Transfor
     uint64_t P = t.KA[r1];
 #pragma unroll 1
     for (int k = r1 - 1; k >= 0; --k) P = mulhi_trunc(P, W) + t.KA[k];
-    uint64_t pw = mulhi_trunc(X, P);   // u P, then the other r0 powers
+    uint64_t pw = X;
 #pragma unroll 1
     for (int q = 0; q < r0; ++q) pw = mulhi_trunc(pw, X);
     Wu = fx_mul(Wu, Fx{X, 0});
@@ -323,7 +328,7 @@ __device__ __forceinline__ uint64_t korobov_gen_whole(uint64_t X, const Transfor
         Wu = fx_norm(Wu);
         W1 = fx_norm(W1);
     }
-    return pw << (64 - t.kf);
+    return mulhi_trunc(pw, P) << (64 - t.kf);
 }
 
 // C^d Wu^r0 W1^r1; cdx = C^d as Fx.
