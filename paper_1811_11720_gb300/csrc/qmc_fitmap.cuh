@@ -6,8 +6,9 @@
 //   p'(x) = |a2| a0/(a0 - 1) v0^2 + |a3| (1 + b)/b v1^2 + a4 + x (2 a5 + 3 a6 x),
 // every factor bounded.  v0 and v1 are held at 2^62, p is formed at 2^58 (from coefficients at
 // 2^60) and p' at 2^em with em from the sum of its coefficients; the Jacobian enters a
-// normalized running product.  Errors are a few units of those scales: below 2^-55 for p, where
-// the FP64 form rounds x near 1 to 2^-53 before a0 - x divides by it.
+// normalized running product.  p's truncations, ~3.2 units of 2^-58 on average, are made up by
+// three; what is left is within 4 units where x is small (7 elsewhere), where the FP64 form rounds
+// x near 1 to 2^-53 before a0 - x divides by it, but is relative near 0 (see eval_point).
 // ~230 integer instructions per dimension against 20 FP64 ones of 17 SM cycles a warp each,
 // which kept fitted sector integrands FP64-bound: a batch of 256 (half of them fitted) took 62 ms
 // and takes 52, the fitted d = 5 call with n = 108,863, m = 32 1090 us and takes 800.
@@ -33,8 +34,11 @@ struct FitFixed {
         int k0, k1, s0, s1, em;      // s: right shift of c R to v at 2^62, less the mantissa's lz
     } dim[kMaxDim];
     int ok;
+    int slope;                       // p' is at most this in every dimension
+    // what 4 units of 2^-58 in every coordinate add to a cubic, in units of 2^-62 of its bound
+    static constexpr int kErrorUnits = 3 * 4 * 32;
 
-    // Stages dimension j from fit[j][6] (one thread each; ok = 1 and a barrier before, one after).
+    // Stages dimension j from fit[j][6] (one thread each; ok = slope = 1 and a barrier before, one after).
     __device__ __forceinline__ void stage(const double *fit, int j) {
         const double *a = fit + 6 * j;
         const double a0 = a[0], b = -a[1], a2 = fabs(a[2]), a3 = fabs(a[3]), a4 = a[4], a5 = a[5];
@@ -47,6 +51,7 @@ struct FitFixed {
             atomicAnd(&ok, 0);
             return;
         }
+        atomicMax(&slope, (int)M + 1);
         Dim &o = dim[j];
         o.k0 = ilogb(a0) + 1;
         o.k1 = ilogb(1.0 + b) + 1;
@@ -81,7 +86,7 @@ struct FitFixed {
         const uint64_t v0 = ratio(o.a0 - (X >> o.k0), o.c0, o.s0);
         const uint64_t v1 = ratio(o.b + (X >> o.k1), o.cb, o.s1);
         int64_t q = smulhi_x(smulhi_x(smulhi_x(o.a6, X) + o.a5, X) + o.a4, X) >> 2;
-        q += (int64_t)(mulhi_trunc(mulhi_trunc(X, v0), o.a2) + mulhi_trunc((1ull << 62) - v1, o.a3b));
+        q += (int64_t)(mulhi_trunc(mulhi_trunc(X, v0), o.a2) + mulhi_trunc((1ull << 62) - v1, o.a3b) + 3);
         const int64_t dp = smulhi_x(smulhi_x(o.d6, X) + o.d5, X) + o.d4 +
                            (int64_t)(mulhi_trunc(sqhi_trunc(v0) << 3, o.k2) + mulhi_trunc(sqhi_trunc(v1) << 3, o.k3));
         // within rounding of [0, 1], and p' not vanishing

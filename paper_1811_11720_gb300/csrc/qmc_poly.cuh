@@ -61,8 +61,10 @@ struct PolyShared {
     // whose error bound passes (stage_poly): the dense coefficients in place as
     // round(c 2^sfix) (unsigned), evaluated by dense_eval_fixed
     int fixed_f, sfix;
-    // the dense U in the same form, where F is (stage_poly), at u[kMaxTerms + e]
-    int fixed_u, sfix_u;
+    // the dense U in the same form, where F is (stage_poly), at u[kMaxTerms + e].  Its error in
+    // units of 2^-sfix_u is below err_u, and below err_u0 + x_max err_u; room_x: what the
+    // coordinates' own error may add (sector_fixed_ok)
+    int fixed_u, sfix_u, err_u, err_u0, room_x;
     // a = 1 and b = n + 1/2 (0 <= n <= 15): n, so that U^a F^-b = U / (F^n sqrt F) needs no
     // per-evaluation tests of the exponents; -1 otherwise
     int pow_half;
@@ -506,10 +508,9 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
         // and N products at under 4.5 units of 2^-s each (dense_eval_fixed) give a
         // relative error below 4.5 N (B / c0) 2^-62, required <= 2^-42.
         // Then U too, when a = 1 with b = n + 1/2 and its dense coefficients are non-negative.
-        // Its error is absolute, below 4.5 N 2^-62 of its coefficients' sum (measured: a
-        // tenth of that), where FP64's is relative; U enters the integrand as a factor, so
-        // what counts is that error against the mean of U where F^-b is large, and F's own
-        // bound (B / c0 times as much) is the larger one wherever that is.
+        // U has no constant term to bound it away from zero, and F^-b may sit where U vanishes, so
+        // each value is checked: where its error may pass 2^-42 of it (err_u 2^42 units, fewer for
+        // small x) U is evaluated in FP64 (sector_u_small).
         __syncthreads();
         const double *cf = ps.buf.v + 2 * kMaxTerms;
         for (int l = tid; l < kSumLanes; l += blockDim.x) {
@@ -532,6 +533,10 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
             ps.sfix = ok ? 62 - ilogb(B) : 0;
             ps.fixed_u = ok_u;
             ps.sfix_u = ok_u ? 62 - ilogb(Bu) : 0;
+            ps.err_u = (9 * (dense_size(V, use_u) + (use_u == 3 ? dense_size(V, 2) : 0) + V) + 1) / 2;
+            // the compensation, and the outermost product of each variable
+            ps.err_u0 = use_u ? (int)dense_truncation(d, use_u) + 4 * d + 1 : 0;
+            ps.room_x = ok ? (int)(fmin(ldexp(c0, ps.sfix - 42) - 4.5 * N, 0x1p30) / fmax(p.pb, 1.0)) : 0;
         }
         __syncthreads();
         if (ps.fixed_f)
@@ -735,21 +740,39 @@ __device__ __forceinline__ double sector_power(double U, double F, const PolySha
     return pow_pos(U, ps.pa) * pow_pos(F, -ps.pb);
 }
 
+// Whether U = Uq 2^-sfix_u from fixed point may be off by more than 2^-42 of itself, the bound
+// that stage_poly sets for F.
+template <int D>
+__device__ __forceinline__ bool sector_u_small(uint64_t Uq, const uint64_t *X, const PolyShared &ps) {
+    const uint32_t q = (uint32_t)(Uq >> 42);
+    if (q >= (uint32_t)ps.err_u) return false;
+    uint32_t top = 0;   // x_max 2^32 is at most top + 1
+#pragma unroll
+    for (int k = 0; k < D; ++k) top |= (uint32_t)(X[k] >> 32);
+    return q <= (uint32_t)ps.err_u0 + __umulhi((uint32_t)ps.err_u, top);
+}
+
 // The real family with F in fixed point, both forms dense and d compiled in (d = 3..8):
-// the coordinates, X = x 2^64, and the unrolled loops stay in registers; U in fixed point
-// with F, else in FP64 at x formed from X by integer operations (truncated).
-// With U in FP64 (its 45 + 9 fused multiply-adds at d = 8 and the power) the FP64 pipe was
-// 70 % busy and the multiply pipe 51 %: n = 1,072,187, m = 32 took 5.88 ms, with U here 4.50.
+// the coordinates, X = x 2^64, and the unrolled loops stay in registers; U in fixed point with F,
+// unless it is too small for that, else in FP64 at x formed from X by integer operations
+// (truncated).
+// With U in FP64 throughout (45 + 9 fused multiply-adds at d = 8 and the power) the FP64 pipe was
+// 70 % busy and the multiply pipe 51 %: n = 1,072,187, m = 32 took 5.88 ms, with U here 4.53 (4.46 without the check).
 template <int D>
 static __device__ __noinline__ double sector_value_fixed_x(const uint64_t *Xin, const PolyShared &ps) {
     uint64_t X[D];
 #pragma unroll
     for (int k = 0; k < D; ++k) X[k] = Xin[k];
     constexpr int V = D + 1;
-    double U;
+    uint64_t Uq = 0;
+    bool small = true;
     if (ps.fixed_u) {
         const uint64_t *Cu = ps.buf.u + kMaxTerms;
-        const uint64_t Uq = ps.dense_u == 3 ? dense_eval_fixed<V>(X, V, 3, Cu) : dense_eval_fixed<V>(X, V, 2, Cu);
+        Uq = ps.dense_u == 3 ? dense_eval_fixed<V>(X, V, 3, Cu) : dense_eval_fixed<V>(X, V, 2, Cu);
+        small = sector_u_small<D>(Uq, X, ps);
+    }
+    double U;
+    if (!small) {
         U = fixed_u64_to_double(Uq, ps.sfix_u);
     } else {
         double x[D];
@@ -761,20 +784,42 @@ static __device__ __noinline__ double sector_value_fixed_x(const uint64_t *Xin, 
     const uint64_t Fq = ps.dense_f == 3 ? dense_eval_fixed<V>(X, V, 3, C) : dense_eval_fixed<V>(X, V, 2, C);
     return sector_power(U, fixed_u64_to_double(Fq, ps.sfix), ps);   // F >= c0 > 0
 }
-// Whether sector_value_fixed_x serves this integrand (uniform over the block).
-__device__ __forceinline__ bool sector_fixed_ok(const PolyShared &ps, int d) {
-    return ps.fixed_f && ps.dense_u && d >= 3 && d <= 8;
+
+// The same with U in FP64 at xin itself.
+template <int D>
+static __device__ __noinline__ double sector_value_fixed_f(const uint64_t *Xin, const double *xin, const PolyShared &ps) {
+    uint64_t X[D];
+    double x[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        X[k] = Xin[k];
+        x[k] = xin[k];
+    }
+    constexpr int V = D + 1;
+    const double U = ps.dense_u == 3 ? dense_eval_t<V, 3>(x, ps.buf.v) : dense_eval_t<V, 2>(x, ps.buf.v);
+    const uint64_t *C = ps.buf.u + 2 * kMaxTerms;
+    const uint64_t Fq = ps.dense_f == 3 ? dense_eval_fixed<V>(X, V, 3, C) : dense_eval_fixed<V>(X, V, 2, C);
+    return sector_power(U, fixed_u64_to_double(Fq, ps.sfix), ps);
 }
 
+// Whether sector_value_x serves this integrand (uniform over the block).  extra: what an absolute
+// error of the coordinates adds to a cubic, in units of 2^-62 of its bound (0: they are exact).
+// Where F^-b sits in a corner, at x ~ c0 / (b B), that error is U's relative one too, and b times
+// F's: room_x bounds both by 2^-42.  (Other powers of U are not bounded by it.)
+__device__ __forceinline__ bool sector_fixed_ok(const PolyShared &ps, int d, int extra) {
+    return ps.fixed_f && ps.dense_u && d >= 3 && d <= 8 && (!extra || (ps.fixed_u && extra <= ps.room_x));
+}
+
+#define QMC_SECTOR_DIM(FN, ...)                                                                                      \
+    (d == 3   ? FN<3>(__VA_ARGS__)                                                                                   \
+     : d == 4 ? FN<4>(__VA_ARGS__)                                                                                   \
+     : d == 5 ? FN<5>(__VA_ARGS__)                                                                                   \
+     : d == 6 ? FN<6>(__VA_ARGS__)                                                                                   \
+     : d == 7 ? FN<7>(__VA_ARGS__)                                                                                   \
+              : FN<8>(__VA_ARGS__))
+
 __device__ __forceinline__ double sector_value_x(const uint64_t *X, int d, const PolyShared &ps) {
-    switch (d) {
-    case 3: return sector_value_fixed_x<3>(X, ps);
-    case 4: return sector_value_fixed_x<4>(X, ps);
-    case 5: return sector_value_fixed_x<5>(X, ps);
-    case 6: return sector_value_fixed_x<6>(X, ps);
-    case 7: return sector_value_fixed_x<7>(X, ps);
-    default: return sector_value_fixed_x<8>(X, ps);
-    }
+    return QMC_SECTOR_DIM(sector_value_fixed_x, X, ps);
 }
 
 __device__ __forceinline__ double sector_value(const double *xin, int d, const PolyShared &ps) {
@@ -783,18 +828,18 @@ __device__ __forceinline__ double sector_value(const double *xin, int d, const P
 #pragma unroll 1
     for (int k = 0; k < d; ++k)
         inside &= (unsigned long long)__double_as_longlong(xin[k]) <= 0x3FF0000000000000ull;
-    if (sector_fixed_ok(ps, d)) {
+    if (sector_fixed_ok(ps, d, 0)) {
         uint64_t X[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) X[k] = k < d ? unit_to_fixed64(xin[k]) : 0;
-        if (inside) return sector_value_x(X, d, ps);
+        if (inside) return ps.fixed_u ? sector_value_x(X, d, ps) : QMC_SECTOR_DIM(sector_value_fixed_f, X, xin, ps);
     }
     double x[kMaxDim + 1];
 #pragma unroll 1
     for (int k = 0; k < d; ++k) x[k] = xin[k];
     x[d] = 1.0;
-    double U, F;
-    uint64_t X[kMaxDim];
+    double F;
+    uint64_t X[kMaxDim], Uq = 0;
     if (ps.fixed_f) {
 #pragma unroll 1
         for (int k = 0; k < d; ++k) X[k] = unit_to_fixed64(x[k]);
@@ -804,8 +849,10 @@ __device__ __forceinline__ double sector_value(const double *xin, int d, const P
         F = ps.dense_f ? dense_eval(x, d + 1, ps.dense_f, ps.buf.v + 2 * kMaxTerms)
                        : poly_real(x, ps.nf, ps.buf.v + 2 * kMaxTerms, ps.buf.u + 3 * kMaxTerms);
     }
-    if (ps.fixed_u && inside)
-        U = fixed_u64_to_double(dense_eval_fixed<0>(X, d + 1, ps.dense_u, ps.buf.u + kMaxTerms), ps.sfix_u);
+    if (ps.fixed_u && inside) Uq = dense_eval_fixed<0>(X, d + 1, ps.dense_u, ps.buf.u + kMaxTerms);
+    double U;
+    if (ps.fixed_u && (Uq >> 42) >= (uint64_t)ps.err_u)
+        U = fixed_u64_to_double(Uq, ps.sfix_u);
     else
         U = ps.dense_u ? dense_eval(x, d + 1, ps.dense_u, ps.buf.v)
                        : poly_real(x, ps.nu, ps.buf.v, ps.buf.u + kMaxTerms);

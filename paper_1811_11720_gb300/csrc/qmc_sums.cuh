@@ -211,12 +211,16 @@ __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared
     constexpr bool kGen = TK == kTKorobovGen;
     if constexpr (kFixedTransform<TK> && kPolyFamily<FAM>) {
         // the polynomial families' fixed-point forms take the coordinates as x 2^64 from the
-        // integer-pipe transform, through the integer fit map where there is one; from the
-        // asymmetric map only where both polynomials are in fixed point (x is then absolute to
-        // ~2^-57, and in FP64, where it is relative near 0, it may be raised to any power)
+        // integer-pipe transform, through the integer fit map where there is one.  The asymmetric
+        // map and the fit leave x absolute to a few units of 2^-kf and 2^-58, where in FP64 it is
+        // relative near 0 and may be raised to any power: they serve where both polynomials are in
+        // fixed point with room for it (extra: what the error, 4 units, adds to a cubic, in units of
+        // 2^-62 of its bound)
         bool fixed = !use_fit || fit_fixed->ok;
-        if constexpr (FAM == QMC_SECTOR) fixed = fixed && sector_fixed_ok(fsh.poly, p.d) && (!kGen || fsh.poly.fixed_u);
-        else fixed = fixed && feyn_fixed_ok(fsh.poly, p.d) && (!kGen || fsh.poly.feyn_full);
+        int extra = use_fit ? FitFixed::kErrorUnits : 0;
+        if constexpr (kGen) extra += (use_fit ? fit_fixed->slope : 1) * (3 * 4) << (63 - p.t.kf);
+        if constexpr (FAM == QMC_SECTOR) fixed = fixed && sector_fixed_ok(fsh.poly, p.d, extra);
+        else fixed = fixed && feyn_fixed_ok(fsh.poly, p.d) && (!extra || fsh.poly.feyn_full);
         if (fixed) {   // uniform over the block
             Weight V;
             Fx J;
@@ -519,7 +523,7 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
         for (int w = tid; w < (int)(sizeof(Integral) / 8); w += blockDim.x)
             reinterpret_cast<uint64_t *>(&s_item)[w] = reinterpret_cast<const uint64_t *>(src)[w];
         if constexpr (kFixedTransform<TK> && kPolyFamily<FAM>)
-            if (tid == 0) fit_fixed->ok = 1;
+            if (tid == 0) fit_fixed->ok = fit_fixed->slope = 1;
         __syncthreads();
         const Integral &it = s_item;
         const int d = it.d;
