@@ -263,7 +263,8 @@ struct DigitDot {
 // has a constant term c0 and all bounds stay near it: no FP64 evaluation of F is better than
 // 2^-54 |c0| either, as its terms are added to c0.  (Without c0, F(x) near a corner of the cube
 // is many orders below its coefficients, and a fixed-point F(x) missed the oracle by 1e-8.)
-// U enters as a factor, so its absolute error counts against its coefficients' sum.
+// U to a positive power enters as a factor, so its absolute error counts against its coefficients'
+// sum; to any other power it needs a constant term too (U^-1 without one, d = 3: 4e-10 off).
 template <class PS>
 __device__ __forceinline__ void stage_feynman_full(PS &ps, int d) {
     const int tid = threadIdx.x;
@@ -312,6 +313,7 @@ __device__ __forceinline__ void stage_feynman_full(PS &ps, int d) {
         const double bf = ps.part[1][8], bu = ps.part[1][9], b3 = ps.part[1][10], b2 = ps.part[1][11];
         const double c0 = fabs(hf[0]), lam = fabs(ps.lam), y = 0.25 * g;   // |y_k| <= lam y
         int ok = g > 0.0 && h > 0.0 && gu > 0.0 && lam < 1e3 && bf <= 16.0 * c0 &&
+                 (ps.pa > 0.0 || bu <= 16.0 * fabs(hu[0])) &&
                  lam * d * g * y <= 64.0 * c0 && lam * lam * d * d * h * y * y <= 64.0 * c0 &&
                  lam * lam * lam * b3 * y * y * y <= c0 && lam * lam * b2 * y * y <= bu &&
                  lam * d * gu * y <= 64.0 * bu && bf < 1e30 && bu < 1e30 && bf > 1e-30 && bu > 1e-30 &&
