@@ -702,6 +702,30 @@ __device__ __forceinline__ double dense_eval(const double *x, int V, int D, cons
     return F;
 }
 
+// The same from the fixed-point coefficients of F (stage_poly), for points outside the cube, where
+// dense_eval_fixed does not follow: c = C 2^-s, the constant term less its compensation.
+__device__ __forceinline__ double dense_eval_outside(const double *x, int V, int D, const uint64_t *C, int s) {
+    const int last = dense_size(V, D) - 1;
+    auto coef = [&](int idx) {
+        return ldexp(__ull2double_rn(idx < last ? C[idx] : C[idx] - dense_truncation(V - 1, D)), -s);
+    };
+    double F = 0.0;
+    int idx = 0;
+#pragma unroll 1
+    for (int a = 0; a < V; ++a) {
+        double sa = 0.0;
+#pragma unroll 1
+        for (int b = a; b < V; ++b) {
+            double t = D == 3 ? 0.0 : coef(idx++);
+#pragma unroll 1
+            for (int c = b; D == 3 && c < V; ++c) t = fma(coef(idx++), x[c], t);
+            sa = fma(x[b], t, sa);
+        }
+        F = fma(x[a], sa, F);
+    }
+    return F;
+}
+
 // Real polynomial value at x (x indexed at run time: x lives in local memory).
 __device__ __forceinline__ double poly_real(const double *x, int nterm, const double *coef,
                                             const uint64_t *mono) {
@@ -824,8 +848,8 @@ __device__ __forceinline__ double sector_value_x(const uint64_t *X, int d, const
     return QMC_SECTOR_DIM(sector_value_fixed_x, X, ps);
 }
 
-__device__ __forceinline__ double sector_value(const double *xin, int d, const PolyShared &ps) {
-    // a fit map that is not monotone leaves the cube: U in fixed point does not follow it there
+static __device__ __noinline__ double sector_value(const double *xin, int d, const PolyShared &ps) {
+    // a fit map that is not monotone leaves the cube: the fixed-point forms do not follow it there
     bool inside = true;
 #pragma unroll 1
     for (int k = 0; k < d; ++k)
@@ -842,7 +866,9 @@ __device__ __forceinline__ double sector_value(const double *xin, int d, const P
     x[d] = 1.0;
     double F;
     uint64_t X[kMaxDim], Uq = 0;
-    if (ps.fixed_f) {
+    if (ps.fixed_f && !inside) {
+        F = dense_eval_outside(x, d + 1, ps.dense_f, ps.buf.u + 2 * kMaxTerms, ps.sfix);
+    } else if (ps.fixed_f) {
 #pragma unroll 1
         for (int k = 0; k < d; ++k) X[k] = unit_to_fixed64(x[k]);
         F = fixed_u64_to_double(dense_eval_fixed<0>(X, d + 1, ps.dense_f, ps.buf.u + 2 * kMaxTerms),
