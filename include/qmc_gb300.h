@@ -423,7 +423,9 @@ int qmc_merge_sums(const double *parts, uint64_t nparts, uint64_t len, double *o
  * beta = 1.
  * z_out: host, s entries.  e2_out: host, s entries (the squared worst-case error after each
  * component), or NULL.  stream: NULL = default.  Device memory (about qmc_cbc_device_bytes(n)
- * plus cuFFT's work area) is allocated here and freed before returning.
+ * and 10 KB per component, plus cuFFT's work area) is allocated here and freed before returning.
+ * Up to two pairs of cuFFT plans, without work areas, stay with the library for the next call of the
+ * same length; after cudaDeviceReset() they are stale and the function must not be called again.
  * Errors: QMC_ERR_ARG (n not a prime in [5, 2^53), s outside 1..1024, beta <= 0,
  * gamma < 0), QMC_ERR_CUDA (allocation, FFT or launch failure), QMC_ERR_NO_DEVICE. */
 size_t qmc_cbc_device_bytes(uint64_t n);

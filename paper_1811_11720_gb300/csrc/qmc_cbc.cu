@@ -348,29 +348,26 @@ __global__ void __launch_bounds__(kCbcThreads)
     }
 }
 
-// What a call needs besides its inputs: two cuFFT plans of length L, their shared work area
-// and one device buffer.  Making them costs more than a construction of a small size runs
-// for, so up to kKept of them, of at most kKeptBytes each, wait for the next call of the same
-// device and length; a call takes one out for itself (calls from several threads or streams
-// do not share any) and gives it back when its stream has drained.
-struct Workspace {
+// Two cuFFT plans of length L, without work areas.  Making them takes two to four milliseconds,
+// more than a construction of a middle size runs for (n = 108,863, s = 10: 2.0 ms, of which 0.13
+// allocating and freeing), so up to kKept
+// pairs wait for the next call of the same device and length; a call takes one out for itself (calls
+// from several threads or streams do not share any) and gives it back when its stream has drained.
+// The buffers, work area included, are the call's own.
+struct Plans {
     int device = -1;
     uint64_t L = 0;
-    size_t bytes = 0, fft_bytes = 0;
+    size_t work_bytes = 0;   // the larger of the two plans' work areas
     cufftHandle fwd = 0, inv = 0;
     bool have_fwd = false, have_inv = false;
-    char *base = nullptr;
-    Workspace() = default;
-    Workspace(const Workspace &) = delete;
-    Workspace &operator=(const Workspace &) = delete;
-    ~Workspace() {
+    Plans() = default;
+    Plans(const Plans &) = delete;
+    Plans &operator=(const Plans &) = delete;
+    ~Plans() {
         if (have_fwd) cufftDestroy(fwd);
         if (have_inv) cufftDestroy(inv);
-        if (base) cudaFree(base);
     }
-    // Plans without their own work areas, then one allocation of `need` bytes and the larger
-    // of the two areas behind it.
-    bool make(uint64_t length, size_t need) {
+    bool make(uint64_t length) {
         long long len = (long long)length;
         size_t wf = 0, wi = 0;
         if (cudaGetDevice(&device) != cudaSuccess) return false;
@@ -383,55 +380,58 @@ struct Workspace {
             cufftMakePlanMany64(fwd, 1, &len, nullptr, 1, 0, nullptr, 1, 0, CUFFT_D2Z, 1, &wf) != CUFFT_SUCCESS ||
             cufftMakePlanMany64(inv, 1, &len, nullptr, 1, 0, nullptr, 1, 0, CUFFT_Z2D, 1, &wi) != CUFFT_SUCCESS)
             return false;
-        bytes = need;
-        fft_bytes = wf > wi ? wf : wi;
-        if (cudaMalloc(&base, bytes + fft_bytes + 256) != cudaSuccess) {
-            base = nullptr;
-            return false;
-        }
-        return cufftSetWorkArea(fwd, base + bytes) == CUFFT_SUCCESS &&
-               cufftSetWorkArea(inv, base + bytes) == CUFFT_SUCCESS;
+        work_bytes = wf > wi ? wf : wi;
+        return true;
+    }
+    bool use(char *work, cudaStream_t st) {
+        return cufftSetWorkArea(fwd, work) == CUFFT_SUCCESS && cufftSetWorkArea(inv, work) == CUFFT_SUCCESS &&
+               cufftSetStream(fwd, st) == CUFFT_SUCCESS && cufftSetStream(inv, st) == CUFFT_SUCCESS;
     }
 };
 
 constexpr size_t kKept = 2;
-constexpr size_t kKeptBytes = (size_t)64 << 20;
 std::mutex g_kept_mutex;
 // never destroyed: at process exit the driver may be gone before static destructors run
-std::vector<std::unique_ptr<Workspace>> &kept() {
-    static auto *v = new std::vector<std::unique_ptr<Workspace>>;
+struct Kept {
+    std::unique_ptr<Plans> plans[kKept];   // oldest first
+};
+Kept &kept() {
+    static auto *v = new Kept;
     return *v;
 }
 
-std::unique_ptr<Workspace> take_workspace(uint64_t L, size_t need) {
+std::unique_ptr<Plans> take_plans(uint64_t L) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     {
         std::lock_guard<std::mutex> lock(g_kept_mutex);
-        auto &v = kept();
-        for (size_t i = 0; i < v.size(); ++i)
-            if (v[i]->device == dev && v[i]->L == L && v[i]->bytes >= need) {
-                std::unique_ptr<Workspace> w = std::move(v[i]);
-                v.erase(v.begin() + i);
-                return w;
-            }
+        for (auto &p : kept().plans)
+            if (p && p->device == dev && p->L == L) return std::move(p);
     }
-    std::unique_ptr<Workspace> w(new (std::nothrow) Workspace);
-    if (w && !w->make(L, need)) w.reset();
-    return w;
+    std::unique_ptr<Plans> p(new (std::nothrow) Plans);
+    if (p && !p->make(L)) p.reset();
+    return p;
 }
 
-void give_back(std::unique_ptr<Workspace> w) {
-    if (w->bytes + w->fft_bytes > kKeptBytes) return;
-    std::unique_ptr<Workspace> old;   // destroyed outside the lock
+void give_back(std::unique_ptr<Plans> p) {
+    std::unique_ptr<Plans> old;   // destroyed outside the lock
     std::lock_guard<std::mutex> lock(g_kept_mutex);
-    auto &v = kept();
-    if (v.size() >= kKept) {
-        old = std::move(v.front());
-        v.erase(v.begin());
+    auto &v = kept().plans;
+    size_t at = 0;
+    while (at < kKept && v[at]) ++at;
+    if (at == kKept) {
+        old = std::move(v[0]);
+        for (at = 0; at + 1 < kKept; ++at) v[at] = std::move(v[at + 1]);
     }
-    v.push_back(std::move(w));
+    v[at] = std::move(p);
 }
+
+struct DeviceBuffer {
+    char *base = nullptr;
+    ~DeviceBuffer() {
+        if (base) cudaFree(base);
+    }
+};
 
 // Smallest 2^a 3^b 5^c 7^d >= x.
 uint64_t smooth_at_least(uint64_t x) {
@@ -488,10 +488,13 @@ extern "C" int qmc_cbc_korobov(uint64_t n, int s, double gamma, double beta, uin
                  host_bytes = bytes, o_mins = take(kCbcBlocks), o_rep = take(kCbcBlocks),
                  o_rept = take(kCbcBlocks), o_gp = take(H), o_p = take(H + 1), o_P = take(L),
                  o_FP = take(2 * nc), o_FW = take(2 * nc);
-    std::unique_ptr<Workspace> ws = take_workspace(L, bytes);
-    if (!ws || cufftSetStream(ws->fwd, st) != CUFFT_SUCCESS || cufftSetStream(ws->inv, st) != CUFFT_SUCCESS)
+    // (declared before the buffer: freeing that waits for whatever is still enqueued)
+    std::unique_ptr<Plans> plans = take_plans(L);
+    DeviceBuffer buf;
+    if (!plans || cudaMalloc(&buf.base, bytes + plans->work_bytes + 256) != cudaSuccess ||
+        !plans->use(buf.base + bytes, st))
         return QMC_ERR_CUDA;
-    auto at = [&](size_t off) { return ws->base + off; };
+    auto at = [&](size_t off) { return buf.base + off; };
     uint64_t *z_d = (uint64_t *)at(o_z), *rep = (uint64_t *)at(o_rep), *gp = (uint64_t *)at(o_gp);
     double *t_d = (double *)at(o_t), *p0_d = (double *)at(o_p0), *sums = (double *)at(o_sums);
     double *mins = (double *)at(o_mins), *rep_t = (double *)at(o_rept), *p = (double *)at(o_p), *P = (double *)at(o_P);
@@ -505,7 +508,7 @@ extern "C" int qmc_cbc_korobov(uint64_t n, int s, double gamma, double beta, uin
     cbc_powers_kernel<<<(unsigned)((nthr + kCbcThreads - 1) / kCbcThreads), kCbcThreads, 0, st>>>(g, mod, H, B, gp);
     cbc_omega_kernel<<<grid_for(L), kCbcThreads, 0, st>>>(gp, H, L, n, P);
     if (cudaGetLastError() != cudaSuccess) return QMC_ERR_CUDA;
-    if (cufftExecD2Z(ws->fwd, P, FW) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
+    if (cufftExecD2Z(plans->fwd, P, FW) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
 
     const uint64_t per_sum = (H + kCbcBlocks - 1) / kCbcBlocks;
     // the minimum and the pick do not depend on the order: blocks of at least 2048 candidates
@@ -517,9 +520,9 @@ extern "C" int qmc_cbc_korobov(uint64_t n, int s, double gamma, double beta, uin
     for (int j = 0; j < s; ++j) {
         if (j) {
             cbc_gather_kernel<<<grid_for(L), kCbcThreads, 0, st>>>(gp, p, H, L, n, P);
-            if (cufftExecD2Z(ws->fwd, P, FP) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
+            if (cufftExecD2Z(plans->fwd, P, FP) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
             cbc_pointwise_kernel<<<grid_for(nc), kCbcThreads, 0, st>>>(FP, FW, nc);
-            if (cufftExecZ2D(ws->inv, FP, P) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
+            if (cufftExecZ2D(plans->inv, FP, P) != CUFFT_SUCCESS) return QMC_ERR_CUDA;
             cbc_min_kernel<<<blocks, kCbcThreads, 0, st>>>(raw, p, H, scale, per_min, mins);
             cbc_pick_kernel<<<blocks, kCbcThreads, 0, st>>>(raw, gp, p, H, n, scale, per_min, mins, blocks,
                                                             sums + (size_t)(j - 1) * kCbcBlocks, rep, rep_t);
@@ -528,14 +531,14 @@ extern "C" int qmc_cbc_korobov(uint64_t n, int s, double gamma, double beta, uin
                                                               per_sum, z_d, t_d, p0_d, sums);
         if (cudaGetLastError() != cudaSuccess) return QMC_ERR_CUDA;
     }
-    std::vector<char> host(host_bytes);
-    if (cudaMemcpyAsync(host.data(), ws->base, host_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    std::unique_ptr<char[]> host(new (std::nothrow) char[host_bytes]);
+    if (!host || cudaMemcpyAsync(host.get(), buf.base, host_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return QMC_ERR_CUDA;
-    give_back(std::move(ws));
-    const uint64_t *hz = (const uint64_t *)(host.data() + o_z);
-    const double *ht = (const double *)(host.data() + o_t), *hp0 = (const double *)(host.data() + o_p0);
-    const double *hs = (const double *)(host.data() + o_sums);
+    give_back(std::move(plans));
+    const uint64_t *hz = (const uint64_t *)(host.get() + o_z);
+    const double *ht = (const double *)(host.get() + o_t), *hp0 = (const double *)(host.get() + o_p0);
+    const double *hs = (const double *)(host.get() + o_sums);
     double tot = 0.0;   // sum_k p(k) of the components so far
     for (int j = 0; j < s; ++j) {
         if (hz[j] >= n) return QMC_ERR_CUDA;   // non-finite sums
