@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kBatchFinThreads)
 }
 
 cudaError_t launch_batch(int family, int tkind, int max_d, const Integral *items, const uint64_t *tb,
-                         int count, uint64_t first_tile, uint64_t end_tile, int m, int spb,
+                         int count, uint64_t first_tile, uint64_t end_tile, int m, int spb, int chain,
                          double *partials, unsigned long long *counters, cudaStream_t s) {
     LatticeLaunch lp{};
     lp.items = items;
@@ -63,6 +63,7 @@ cudaError_t launch_batch(int family, int tkind, int max_d, const Integral *items
     lp.count = count;
     lp.m = m;
     lp.spb = spb;
+    lp.chain = chain;
     lp.first_tile = first_tile;
     lp.end_tile = end_tile;
     lp.partials = partials;
@@ -146,7 +147,10 @@ int plan_batch(const qmc_batch_item *in, int count, const qmc_batch_config *cfg,
         P.items[q].slot = q;
     }
     // the kernel is compiled per transform kind: a batch of one kind (the usual one) is one
-    // launch in input order, a mixed one a launch per kind
+    // launch in input order, a mixed one a launch per kind.  These overlap: alone, each of 24
+    // integrals' six launches (n = 1021, m = 32) leaves the chip half empty and takes its own
+    // latency, 286 us with the reduction, 134 overlapped (272 for one launch of all kinds compiled
+    // together).
     std::stable_sort(P.items.begin(), P.items.end(),
                      [](const Integral &a, const Integral &b) { return a.t.kind < b.t.kind; });
     uint64_t tiles = 0, poff = 0;
@@ -184,8 +188,9 @@ int launch_planned(const BatchPlan &P, int count, void *workspace, double *sums,
     double *d_part = (double *)(ws + P.off_partials);
     for (const auto &g : P.groups)
         if (launch_batch(P.family, g.kind, g.max_d, d_items + g.begin, d_tb + g.begin, g.end - g.begin,
-                         P.tile_begin[g.begin], P.tile_begin[g.end], P.m, P.spb, d_part, counters,
-                         s) != cudaSuccess)
+                         P.tile_begin[g.begin], P.tile_begin[g.end], P.m, P.spb,
+                         P.groups.size() == 1 ? kNoChain : g.begin == 0 ? kChainFirst : kChainLater, d_part,
+                         counters, s) != cudaSuccess)
             return QMC_ERR_CUDA;
     if (launch_batch_reduce(d_items, count, P.m, P.cplx, d_part, sums, s) != cudaSuccess) return QMC_ERR_CUDA;
     if (results) {

@@ -51,7 +51,7 @@ bool batch_family_supported(int fam);
 // One launch over items[0..count) of one transform kind, tiles [first_tile, end_tile).
 cudaError_t launch_batch(int family, int tkind, int max_d, const Integral *items,
                          const uint64_t *tile_begin, int count, uint64_t first_tile,
-                         uint64_t end_tile, int m, int spb, double *partials,
+                         uint64_t end_tile, int m, int spb, int chain, double *partials,
                          unsigned long long *counters, cudaStream_t s);
 cudaError_t launch_batch_reduce(const Integral *d_items, int count, int m, int cplx,
                                 const double *partials, double *sums, cudaStream_t s);

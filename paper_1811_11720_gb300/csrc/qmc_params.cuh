@@ -62,6 +62,10 @@ struct Integral {
     double pa, pb, lam;
 };
 
+// Launches of one batch, one after another in a stream, that share nothing but their inputs: each
+// later one may start when all blocks of the one before it have started, and ends after it.
+enum { kNoChain = 0, kChainFirst = 1, kChainLater = 2 };
+
 // A launch of the lattice-sum kernel: one integral (items null) or the integrals items[0..count)
 // whose tiles, laid end to end, are numbered by tile_begin[0..count]; all of one transform kind.
 struct LatticeLaunch {
@@ -70,6 +74,7 @@ struct LatticeLaunch {
     const uint64_t *tile_begin;
     int count;
     int m, spb;                       // shifts, streams per block (blockDim = spb * m)
+    int chain;                        // kNoChain, or its place among launches that may overlap
     uint64_t first_tile, end_tile;    // the tiles of this launch
     double *partials;                 // per integral: [tiles][m] (sum, comp) re, then im
     unsigned long long *counters;     // [2] per integral, or nullptr

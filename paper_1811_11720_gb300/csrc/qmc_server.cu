@@ -422,7 +422,7 @@ extern "C" int qmc_server_step(qmc_server *s, int *completed) {
         if (cudaMemcpyAsync(di, s->h_items + g0, sizeof(Integral) * cnt, cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
             cudaMemcpyAsync(s->d_tb, s->h_tb, sizeof(uint64_t) * (cnt + 1), cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
             return QMC_ERR_CUDA;
-        if (launch_batch(fam, kind, max_d, di, s->d_tb, cnt, 0, tiles, m, spb, (double *)s->pool,
+        if (launch_batch(fam, kind, max_d, di, s->d_tb, cnt, 0, tiles, m, spb, kNoChain, (double *)s->pool,
                          s->d_counters + 2 * g0, s->stream) != cudaSuccess ||
             launch_batch_reduce(di, cnt, m, cplx, (double *)s->pool, s->d_sums + g0 * 4 * m, s->stream) != cudaSuccess ||
             launch_batch_finalize(di, cnt, m, cplx, s->d_sums + g0 * 4 * m, s->d_results + 4 * g0, s->stream) != cudaSuccess)

@@ -498,6 +498,7 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
     const int tid = threadIdx.x;
     const int m = lp.m, spb = lp.spb;
     const WarpStreams ws = warp_streams(m);
+    if (lp.chain) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (uint64_t tile = lp.first_tile + blockIdx.x; tile < lp.end_tile; tile += gridDim.x) {
         __syncthreads();   // the previous tile's shared data is no longer read
         const Integral *src = &lp.one;
@@ -561,6 +562,8 @@ __global__ void __launch_bounds__(kSumsThreads, MINB)
             if (acc.signfail) atomicAdd(lp.counters + 2 * it.slot + 1, acc.signfail);
         }
     }
+    // ends after the launch before it, whose end then follows from this one's
+    if (lp.chain) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace qmc

@@ -22,6 +22,19 @@ static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s
                                                    (int)sizeof(uint64_t) * kMaxDim * kSumsThreads);
         if (e != cudaSuccess) return e;
     }
+    if (lp.chain == kChainLater) {
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(lp.spb * lp.m);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, lattice_kernel<FAM, TK, MINB>, lp);
+    }
     lattice_kernel<FAM, TK, MINB><<<(unsigned)grid, lp.spb * lp.m, smem, s>>>(lp);
     return cudaGetLastError();
 }
