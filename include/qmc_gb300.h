@@ -94,12 +94,25 @@ enum {
  *   Polynomial families: U = sum_m ucoef[m] prod_k x_k^uexp[m*dim+k] (nu terms), F likewise
  *   (nf terms), exponents 0..15; the value is U^pa F^-pb (principal branch) times, for
  *   QMC_FEYNMAN, det(dz/dx) at z_k = x_k - i lambda x_k (1 - x_k) dF/dx_k (real x).
- *   Arithmetic is FP64 except for two integer-pipe forms in 64-bit fixed point, chosen at
- *   staging: QMC_SECTOR's dense F when its coefficients are non-negative with a constant
- *   term c0 > 0 and the bound 4.5 N (sum of coefficients / c0) 2^-62 on its relative error
- *   (N products) is at most 2^-42; QMC_FEYNMAN's Hessian, dF and dU for dim 3..6 (deg U <= 2,
- *   deg F <= 3), each within 2^-49 of the sum of |coefficients|.  U(x), F(x) of QMC_FEYNMAN,
- *   and everything else, stay FP64. */
+ *   Arithmetic is FP64 except for forms in 64-bit fixed point on the integer pipe, chosen at
+ *   staging where their bounds hold, on FP64 otherwise:
+ *   - coordinates under no transform, baker and Korobov<r0,r1> with orders 1..6 and no fit: x to
+ *     a few units of 2^-57 or better (2^-54 at unequal orders 5 and 6), absolutely.  Unequal orders
+ *     keep FP64, relative near the ends, for corner peaks and C0 with sum c >= 32 and for polynomials
+ *     whose forms below do not hold;
+ *   - the Genz families with c >= 0 and 0 <= w <= 1 (Gaussian and product peak: max c < 32), their
+ *     exponentials, cosines, powers and reciprocals within 2^-55 of the value;
+ *   - QMC_SECTOR's dense F, coefficients non-negative, constant term c0 > 0 and the bound
+ *     4.5 N (sum of coefficients / c0) 2^-62 (N products) at most 2^-42: relative error 2^-42;
+ *     and its dense U with pa = 1, pb = n + 1/2 and non-negative coefficients, each value within
+ *     2^-42 of itself (smaller ones, where the absolute error would be more, in FP64);
+ *   - the fit map of the polynomial families with moderate parameters, to 7 units of 2^-58 (4 near
+ *     x = 0), where both polynomials are in fixed point with room for that error; points that it
+ *     sends outside [0, 1] are evaluated there in FP64;
+ *   - QMC_FEYNMAN's Hessian, dF and dU for dim 3..6 (deg U <= 2, deg F <= 3), each within 2^-49 of the
+ *     sum of |coefficients|; and U(z), F(z) to a few units of 2^-57 of their coefficients' sums (at
+ *     most 2^-40 of F's constant term), where that term is at least 1/16 of F's sum, U's too unless
+ *     pa > 0, and the deformation is moderate. */
 typedef struct {
     int family;
     int dim;
@@ -237,7 +250,7 @@ int qmc_evaluate(const qmc_integrand *f, uint64_t n, const uint64_t *z, int dim,
  * of the fit, Sec. 2.4): hist (device) [dim][bins] += |f(x_i)| at bin floor(x_ij * bins)
  * (clamped to bins-1); hist is zeroed first.  workspace (device) must hold
  * qmc_histogram_workspace_bytes(n, dim, bins) bytes (per-block partial histograms, summed
- * in block order: the result is deterministic).  dim * bins <= 20480. */
+ * in a fixed order: the result is deterministic).  dim * bins <= 20480. */
 size_t qmc_histogram_workspace_bytes(uint64_t n, int dim, int bins);
 int qmc_histogram(const qmc_integrand *f, uint64_t n, const uint64_t *z, int dim,
                   const uint64_t *shift, int bins, double *hist, void *workspace,
@@ -269,8 +282,9 @@ typedef struct {
 size_t qmc_batch_workspace_bytes(const qmc_batch_item *items, int count,
                                  const qmc_batch_config *cfg);
 
-/* Per-shift sums of every item in one kernel launch, then one reduction launch and
- * (results != NULL) one finalize launch (Eq. (lattice), Eq. (lattice-error)).
+/* Per-shift sums of every item in one kernel launch (one per transform kind, overlapping, when
+ * the items' transforms are of several), then one reduction launch and (results != NULL) one
+ * finalize launch (Eq. (lattice), Eq. (lattice-error)).
  *   items: host array of count items.  sums (device) [count][4m]: item q's double-double
  *   sums at q*4m in the qmc_sums layout.  results (device, may be NULL) [count][4]:
  *   Qbar_re, sigma_re, Qbar_im, sigma_im (needs m >= 2).  counters (device, may be NULL)
@@ -285,7 +299,7 @@ int qmc_batch_sums(const qmc_batch_item *items, int count, const qmc_batch_confi
  * qmc_batch_plan_create validates the items, uploads their descriptors into `workspace`
  * (stream-ordered, then synchronises `stream`) and returns a host handle; the items' device
  * arrays and the workspace must outlive the plan.  qmc_batch_plan_run enqueues only kernel
- * launches (batch kernel, reduction, optional finalize), so it can be captured.
+ * launches (batch kernels, reduction, optional finalize), so it can be captured.
  * qmc_batch_plan_destroy frees the handle (host memory). */
 typedef struct qmc_batch_plan qmc_batch_plan;
 int qmc_batch_plan_create(const qmc_batch_item *items, int count, const qmc_batch_config *cfg,
@@ -371,7 +385,7 @@ int qmc_server_completed(qmc_server *s, uint64_t *ids, int cap, int *count);
 /* ---- tile-aligned sharding --------------------------------------------------------- */
 
 /* qmc_sums cuts an i-range into tiles that depend only on the range's length and m (one
- * shift group, m <= 256) and folds the per-tile partial sums in tile order in double-double.
+ * shift group, m <= 256) and folds the per-tile partial sums in a fixed order in two words.
  * A range split at tile boundaries, its tiles' partials gathered in tile order and folded
  * by qmc_reduce_tiles gives the per-shift sums of qmc_sums bit for bit (Sec. 2.1: the
  * points of one rule are independent, so shards need no other exchange). */
