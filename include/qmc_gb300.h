@@ -107,8 +107,8 @@ enum {
  *     and its dense U with pa = 1, pb = n + 1/2 and non-negative coefficients, each value within
  *     2^-42 of itself (smaller ones, where the absolute error would be more, in FP64);
  *   - the fit map of the polynomial families with moderate parameters, to 7 units of 2^-58 (4 near
- *     x = 0), where both polynomials are in fixed point with room for that error; points that it
- *     sends outside [0, 1] are evaluated there in FP64;
+ *     x = 0), where F (QMC_FEYNMAN: F(z) and U(z)) is in fixed point with room for that error and
+ *     pa > 0; points that it sends outside [0, 1] are evaluated there in FP64;
  *   - QMC_FEYNMAN's Hessian, dF and dU for dim 3..6 (deg U <= 2, deg F <= 3), each within 2^-49 of the
  *     sum of |coefficients|; and U(z), F(z) to a few units of 2^-57 of their coefficients' sums (at
  *     most 2^-40 of F's constant term), where that term is at least 1/16 of F's sum, U's too unless

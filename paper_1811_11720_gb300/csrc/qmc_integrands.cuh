@@ -41,9 +41,10 @@ namespace qmc {
 //     had to be normalized first.
 // S is capped at 64 otherwise (small c keep 2^-64 absolute precision), so that the
 // exponential's argument scale, S or 2S - 64, lies in [2, 64] (exp_fixed).
-// Each term truncates by at most three units (2^-S, or 2^(64 - 2S) for squares); the forms
-// are therefore exact to ~2^-48 absolutely or better.  ok is false (double path) unless
-// every c_j >= 0 and 0 <= w_j <= 1.
+// Each term truncates by at most three units (2^-S, or 2^(64 - 2S) for squares): the forms are
+// exact to 2^-44 absolutely for sum c < 2^12 and d <= 16, and lose a bit for each doubling of it
+// (as c (x - w) itself does in FP64).  ok is false (double path) unless every c_j >= 0 and
+// 0 <= w_j <= 1; the asymmetric Korobov map asks for more (fixed_form_ok).
 //   oscillatory (1), integer finish: the phase in turns, (w_1 + sum_j c_j x_j / (2 pi)) mod 1
 //     as a 64-bit fraction: c_j / (2 pi) = tk_j + tg_j 2^-64 (integer and fraction parts,
 //     from a double-double product), so each term is tk_j X_j + floor(tg_j X_j 2^-64) mod

@@ -536,9 +536,9 @@ __device__ __forceinline__ void stage_poly(const P &p, PolyShared &ps, bool allo
             ps.fixed_u = ok_u;
             ps.sfix_u = ok_u ? 62 - ilogb(Bu) : 0;
             ps.err_u = (9 * (dense_size(V, use_u) + (use_u == 3 ? dense_size(V, 2) : 0) + V) + 1) / 2;
-            // the compensation, and the outermost product of each variable
-            ps.err_u0 = use_u ? (int)dense_truncation(d, use_u) + 4 * d + 1 : 0;
-            ps.room_x = ok ? (int)(fmin(ldexp(c0, ps.sfix - 42) - 4.5 * N, 0x1p30) / fmax(p.pb, 1.0)) : 0;
+            // at x = 0: up by the compensation, or down by the outermost product of each variable
+            ps.err_u0 = use_u ? max((int)dense_truncation(d, use_u), (7 * d + 1) / 2) + 2 : 0;
+            ps.room_x = ok ? (int)(fmin(ldexp(c0, ps.sfix - 42) - 4.5 * N, 0x1p30) / fmax(fmax(p.pa, p.pb), 1.0)) : 0;
         }
         __syncthreads();
         if (ps.fixed_f)
@@ -831,9 +831,9 @@ static __device__ __noinline__ double sector_value_fixed_f(const uint64_t *Xin, 
 // Whether sector_value_x serves this integrand (uniform over the block).  extra: what an absolute
 // error of the coordinates adds to a cubic, in units of 2^-62 of its bound (0: they are exact).
 // Where F^-b sits in a corner, at x ~ c0 / (b B), that error is U's relative one too, and b times
-// F's: room_x bounds both by 2^-42.  (Other powers of U are not bounded by it.)
+// F's: room_x bounds both, to their powers, by 2^-42.  (U in the denominator is not bounded by it.)
 __device__ __forceinline__ bool sector_fixed_ok(const PolyShared &ps, int d, int extra) {
-    return ps.fixed_f && ps.dense_u && d >= 3 && d <= 8 && (!extra || (ps.fixed_u && extra <= ps.room_x));
+    return ps.fixed_f && ps.dense_u && d >= 3 && d <= 8 && (!extra || (ps.pa > 0.0 && extra <= ps.room_x));
 }
 
 #define QMC_SECTOR_DIM(FN, ...)                                                                                      \

@@ -7,9 +7,9 @@
 // coefficients, and share the family and the transform kind (template parameters) and m (the
 // block shape).  Thread (s, k) evaluates shift k on the L consecutive points of stream s.
 // The transform and, where the integrand allows, the integrand's linear and quadratic forms
-// run in integer fixed point (qmc_fixed.cuh, qmc_integrands.cuh), and under the cheaper maps
-// so does its final function (qmc_exp.cuh, qmc_cos.cuh); FP64 is left to the final function
-// under the higher Korobov orders and to the sums.
+// run in integer fixed point (qmc_fixed.cuh, qmc_integrands.cuh), and so does its final function
+// (qmc_exp.cuh, qmc_cos.cuh); FP64 is left to the sums, the polynomial families' powers and what
+// has no fixed-point form.
 // Each thread accumulates its L samples in FP64; the tile's per-shift partial is
 // the Neumaier-compensated sum over its spb streams in fixed order, written to
 // partials[tile][k].  Tiles depend only on the i-range, so the result is bit-identical for
@@ -213,12 +213,12 @@ __device__ __forceinline__ void eval_point(const Integral &p, const FamilyShared
         // the polynomial families' fixed-point forms take the coordinates as x 2^64 from the
         // integer-pipe transform, through the integer fit map where there is one.  The asymmetric
         // map and the fit leave x absolute to a few units of 2^-kf and 2^-58, where in FP64 it is
-        // relative near 0 and may be raised to any power: they serve where both polynomials are in
-        // fixed point with room for it (extra: what the error, 4 units, adds to a cubic, in units of
-        // 2^-62 of its bound)
+        // relative near 0 and may be raised to any power: they serve where the polynomials are bounded
+        // away from zero, or only factors, with room for it (extra: what the error, 4 and on average
+        // 2 units, adds to a cubic, in units of 2^-62 of its bound)
         bool fixed = !use_fit || fit_fixed->ok;
         int extra = use_fit ? FitFixed::kErrorUnits : 0;
-        if constexpr (kGen) extra += (use_fit ? fit_fixed->slope : 1) * (3 * 4) << (63 - p.t.kf);
+        if constexpr (kGen) extra += (use_fit ? fit_fixed->slope : 1) * (3 * 2) << (63 - p.t.kf);
         if constexpr (FAM == QMC_SECTOR) fixed = fixed && sector_fixed_ok(fsh.poly, p.d, extra);
         else fixed = fixed && feyn_fixed_ok(fsh.poly, p.d) && (!extra || fsh.poly.feyn_full);
         if (fixed) {   // uniform over the block
