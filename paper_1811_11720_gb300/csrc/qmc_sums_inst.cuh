@@ -7,7 +7,7 @@
 
 namespace qmc {
 
-template <int FAM, int TK, int MINB>
+template <int FAM, int TK, int MINB, bool kOne = false>
 static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s) {
     const uint64_t tiles = lp.end_tile - lp.first_tile;
     const uint64_t grid = tiles < 0x7FFFFFFFull ? tiles : 0x7FFFFFFFull;
@@ -17,7 +17,7 @@ static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s
     // function that all threads share: always the largest table's size, so that no call lowers it
     // under another one's launch.
     if (smem > 2048) {
-        const cudaError_t e = cudaFuncSetAttribute(lattice_kernel<FAM, TK, MINB>,
+        const cudaError_t e = cudaFuncSetAttribute(lattice_kernel<FAM, TK, MINB, kOne>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)sizeof(uint64_t) * kMaxDim * kSumsThreads);
         if (e != cudaSuccess) return e;
@@ -33,9 +33,9 @@ static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s
         cfg.stream = s;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, lattice_kernel<FAM, TK, MINB>, lp);
+        return cudaLaunchKernelEx(&cfg, lattice_kernel<FAM, TK, MINB, kOne>, lp);
     }
-    lattice_kernel<FAM, TK, MINB><<<(unsigned)grid, lp.spb * lp.m, smem, s>>>(lp);
+    lattice_kernel<FAM, TK, MINB, kOne><<<(unsigned)grid, lp.spb * lp.m, smem, s>>>(lp);
     return cudaGetLastError();
 }
 
@@ -44,7 +44,9 @@ static cudaError_t launch_family(int tkind, const LatticeLaunch &lp, int max_d, 
     switch (tkind) {
     case QMC_T_NONE: return launch_one<FAM, QMC_T_NONE, MINB>(lp, max_d, s);
     case QMC_T_BAKER: return launch_one<FAM, QMC_T_BAKER, MINB>(lp, max_d, s);
-    case QMC_T_KOROBOV: return launch_one<FAM, QMC_T_KOROBOV, MINB>(lp, max_d, s);
+    case QMC_T_KOROBOV:
+        if (!lp.items) return launch_one<FAM, QMC_T_KOROBOV, MINB, true>(lp, max_d, s);
+        return launch_one<FAM, QMC_T_KOROBOV, MINB>(lp, max_d, s);
     case QMC_T_SIDI: return launch_one<FAM, QMC_T_SIDI, MINB>(lp, max_d, s);
     case kTKorobovInt: return launch_one<FAM, kTKorobovInt, MINB>(lp, max_d, s);
     case kTKorobovGen: return launch_one<FAM, kTKorobovGen, MINB>(lp, max_d, s);
