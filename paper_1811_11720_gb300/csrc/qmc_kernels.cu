@@ -155,7 +155,7 @@ __device__ __forceinline__ void eval_point(const FamilyShared<FAM> &fsh, const d
 }
 
 constexpr int kEvalThreads = 128;
-constexpr uint32_t kEvalChunk = 32;
+constexpr uint32_t kEvalChunk = 16;   // points a thread: latency-bound, and a start costs about three steps
 
 template <int FAM>
 __global__ void __launch_bounds__(kEvalThreads) evaluate_kernel(const Integral p, double *out) {
