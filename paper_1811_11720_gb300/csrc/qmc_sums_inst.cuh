@@ -39,13 +39,23 @@ static cudaError_t launch_one(const LatticeLaunch &lp, int max_d, cudaStream_t s
     return cudaGetLastError();
 }
 
+// Whether a launch under the FP64 Korobov map reads its integral in place (lattice_kernel's kOne):
+// single integrals of the separable families; of the polynomial ones, whose loops need the
+// registers that uniform operands take, those with an order 0 (sector d = 8, n = 108,863, m = 32: 643
+// us, 714 from shared memory) or of at most one wave of blocks (sparse sector d = 6, n = 1021, orders
+// 8: 150, 163; at n = 108,863 1647, 1443).
+template <int FAM, int MINB>
+static bool reads_in_place(const LatticeLaunch &lp) {
+    return !lp.items && (!kPolyFamily<FAM> || !lp.one.t.r0 || !lp.one.t.r1 || lp.end_tile - lp.first_tile <= 152 * MINB);
+}
+
 template <int FAM, int MINB = kSumsMinBlocks<FAM>>
 static cudaError_t launch_family(int tkind, const LatticeLaunch &lp, int max_d, cudaStream_t s) {
     switch (tkind) {
     case QMC_T_NONE: return launch_one<FAM, QMC_T_NONE, MINB>(lp, max_d, s);
     case QMC_T_BAKER: return launch_one<FAM, QMC_T_BAKER, MINB>(lp, max_d, s);
     case QMC_T_KOROBOV:
-        if (!lp.items) return launch_one<FAM, QMC_T_KOROBOV, MINB, true>(lp, max_d, s);
+        if (reads_in_place<FAM, MINB>(lp)) return launch_one<FAM, QMC_T_KOROBOV, MINB, true>(lp, max_d, s);
         return launch_one<FAM, QMC_T_KOROBOV, MINB>(lp, max_d, s);
     case QMC_T_SIDI: return launch_one<FAM, QMC_T_SIDI, MINB>(lp, max_d, s);
     case kTKorobovInt: return launch_one<FAM, kTKorobovInt, MINB>(lp, max_d, s);
