@@ -11,7 +11,7 @@
 // x near 1 to 2^-53 before a0 - x divides by it, but is relative near 0 (see eval_point).
 // ~230 integer instructions per dimension against 20 FP64 ones of 17 SM cycles a warp each,
 // which kept fitted sector integrands FP64-bound: a batch of 256 (half of them fitted) took 62 ms
-// and takes 52, the fitted d = 5 call with n = 108,863, m = 32 1090 us and takes 800.
+// and takes 50, the fitted d = 5 call with n = 108,863, m = 32 1090 us and takes 755.
 //
 // The form is taken when the coefficients are moderate (FitFixed::stage); a point that a map
 // which is not monotone sends outside [0, 1], or where p' is not positive, is left to the FP64

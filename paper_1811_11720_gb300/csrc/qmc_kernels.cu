@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kEvalThreads) evaluate_kernel(const Integral p
 // blocks (host: ~512 points each): one thread per dimension adding 128 points one after the
 // other, in blocks of 4096, took 519 us for the 1.1e5 evaluations of a d = 5 sector
 // integrand, of the 1764 us of the whole fitting call (the sums' fit map since changed too:
-// 761 us now).
+// 755 us now).
 constexpr int kHistThreads = 256;
 
 template <int FAM>

@@ -469,7 +469,7 @@ __device__ __forceinline__ void tile_partial(const StreamSum &acc, double *s_red
 
 // Blocks per SM the register allocation must allow: five for the separable families (48
 // registers; their throughput depends on hiding integer latency), three for the sector family
-// (85 registers; d = 8, n = 1,072,187, m = 32: 4.55 ms with two blocks, 4.43 with three, 9.0
+// (85 registers; d = 8, n = 1,072,187, m = 32: 4.55 ms with two blocks, 4.43 with three (4.53 since U's check), 9.0
 // with the one the compiler leaves room for by itself), two for the complex family with the
 // dimension compiled in (128 registers with a few spills; d = 5 at the same size: 23.3 ms with
 // one, 19.1 with two) and one without (d = 8 with two blocks was 15 % slower).
